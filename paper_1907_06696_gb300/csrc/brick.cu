@@ -87,49 +87,39 @@ __global__ void __launch_bounds__(BS, sizeof(T) == 4 ? 384 / BS : 1) k_cell_atom
 }
 
 // ---- component-split variant: three threads per cell, warp c of each group of three computes
-// output component c. A cell's output row c is
-//   w_c = 2 D_c^T W (d_c U_c) + sum_{d != c} D_d^T W (d_d U_c + d_c U_d),
-// so the thread of component c interpolates only its own component U_c, forms its three
-// derivatives d_e U_c, and takes the cross terms d_c U_d from the other two threads through
-// shared memory. The arithmetic per cell is that of the one-thread kernel (the same sweeps), the
-// serial work per thread a third of it: the small levels, where a level operator is one wave of
-// a few warps and its time is one thread's latency, get faster; the product is the same up to
-// the order of the sums.
+// output component c: it transforms only its own component to the modes, leaves them in shared
+// memory, and takes the 12 modes that it needs of each of the other two from there. The arithmetic
+// per cell is that of the one-thread kernel, the serial work per thread a third of it: the small
+// levels, where a level operator is one wave of a few warps and its time is one thread's latency,
+// get faster; the product is the same up to the order of the sums.
 constexpr int kSplitCells = 32;   // cells per block; block = 3 warps
+
+// The modes of row component C from those of the three components in shared memory (lane lc).
+template <int C>
+__device__ __forceinline__ void split_row(const float (&D)[3][27][kSplitCells], int lc, float (&u)[27]) {
+    float u1[27], u2[27], w[27];
+#pragma unroll
+    for (int m = 0; m < 27; ++m) {   // the modes that modes_A does not use are never loaded
+        u1[m] = D[(C + 1) % 3][m][lc];
+        u2[m] = D[(C + 2) % 3][m][lc];
+    }
+    q2::modes_A<C>(u, u1, u2, w);
+#pragma unroll
+    for (int m = 0; m < 27; ++m) u[m] = w[m];
+}
 
 // The cell product of the component-split kernels: u holds the nodal values of this thread's
 // component on entry and the cell's output row c (without mu h) on return; all threads of the
 // block take part (the exchange has a barrier).
-__device__ __forceinline__ void split_apply(float (&u)[27], float (&D)[3][3][27][kSplitCells], int c, int lc) {
-    q2::interp<0>(u);
-    q2::interp<1>(u);
-    q2::interp<2>(u);
-    float g[27];
-    q2::deriv<0, false>(u, g);
+__device__ __forceinline__ void split_apply(float (&u)[27], float (&D)[3][27][kSplitCells], int c, int lc) {
+    q2::to_modes3(u);
 #pragma unroll
-    for (int q = 0; q < 27; ++q) D[c][0][q][lc] = g[q];
-    q2::deriv<1, false>(u, g);
-#pragma unroll
-    for (int q = 0; q < 27; ++q) D[c][1][q][lc] = g[q];
-    q2::deriv<2, false>(u, g);
-#pragma unroll
-    for (int q = 0; q < 27; ++q) D[c][2][q][lc] = g[q];
+    for (int m = 0; m < 27; ++m) D[c][m][lc] = u[m];
     __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 27; ++q) u[q] = 0.0f;
-    // d = 0, 1, 2 at compile time; the diagonal term (d == c) carries the factor 2
-#pragma unroll
-    for (int q = 0; q < 27; ++q) g[q] = c == 0 ? D[0][0][q][lc] : D[c][0][q][lc] + D[0][c][q][lc];
-    if (c == 0) q2::derivT_w<0, 2>(g, u); else q2::derivT_w<0, 1>(g, u);
-#pragma unroll
-    for (int q = 0; q < 27; ++q) g[q] = c == 1 ? D[1][1][q][lc] : D[c][1][q][lc] + D[1][c][q][lc];
-    if (c == 1) q2::derivT_w<1, 2>(g, u); else q2::derivT_w<1, 1>(g, u);
-#pragma unroll
-    for (int q = 0; q < 27; ++q) g[q] = c == 2 ? D[2][2][q][lc] : D[c][2][q][lc] + D[2][c][q][lc];
-    if (c == 2) q2::derivT_w<2, 2>(g, u); else q2::derivT_w<2, 1>(g, u);
-    q2::interpT<0>(u);
-    q2::interpT<1>(u);
-    q2::interpT<2>(u);
+    if (c == 0) split_row<0>(D, lc, u);
+    else if (c == 1) split_row<1>(D, lc, u);
+    else split_row<2>(D, lc, u);
+    q2::from_modes3(u);
 }
 
 // Scatter of component c of a cell's output row (times sc) into acc at out = acc + c nodes +
@@ -162,7 +152,7 @@ __device__ __forceinline__ void split_scatter(float* out, int c, int M, int ci, 
 
 template <bool PAIRS>
 __global__ void __launch_bounds__(3 * kSplitCells) k_cell_split(BrickArgs<float> a, float* acc) {
-    __shared__ float D[3][3][27][kSplitCells];   // D[c][e][q][cell] = d_e U_c at Gauss point q
+    __shared__ float D[3][27][kSplitCells];   // D[c][m][cell]: mode m of component c
     const int c = threadIdx.x / kSplitCells;     // warp-uniform
     const int lc = threadIdx.x % kSplitCells;
     const size_t cells = size_t(a.n) * a.n * a.n;
@@ -272,7 +262,7 @@ __global__ void __launch_bounds__(3 * kSplitCells)
                       const float* __restrict__ dinv, const float* __restrict__ d_old, const float* __restrict__ x_old,
                       float* __restrict__ d_new, float* __restrict__ x_new, float* __restrict__ acc_zero, float c1,
                       float c2, float* __restrict__ acc) {
-    __shared__ float D[3][3][27][kSplitCells];
+    __shared__ float D[3][27][kSplitCells];
     const int c = threadIdx.x / kSplitCells;
     const int lc = threadIdx.x % kSplitCells;
     const size_t cells = size_t(a.n) * a.n * a.n;

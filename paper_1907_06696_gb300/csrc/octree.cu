@@ -252,45 +252,23 @@ __global__ void __launch_bounds__(128) k_oct_active(OctActiveDev a, const double
     const int32_t* rp = a.leaf_p + size_t(leaf) * 8;
     const double h = ldexp(1.0, -int(a.level[leaf]));
     const double s = -h * h;
-    double w[3][27];
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-        for (int m = 0; m < 27; ++m) w[c][m] = 0.0;
+    double u[3][27], w[3][27], p8[8], pb[8];
     if (DO_A || DO_B) {
-        double u[3][27];
 #pragma unroll
         for (int m = 0; m < 27; ++m) {
             const int32_t r = ru[m];
 #pragma unroll
             for (int c = 0; c < 3; ++c) u[c][m] = gather_u(a, src_u, c, r, size_t(leaf) * 27 + m);
         }
-        if (DO_B) {
-            double pb[8];
-#pragma unroll
-            for (int v = 0; v < 8; ++v) pb[v] = 0.0;
-            q2::b_component<0>(u[0], pb);
-            q2::b_component<1>(u[1], pb);
-            q2::b_component<2>(u[2], pb);
-#pragma unroll
-            for (int v = 0; v < 8; ++v) scatter_p(a, dst_p, rp[v], s * pb[v], size_t(leaf) * 8 + v);
-        }
-        if (DO_A) {
-            q2::cell_A(u, w);
-            const double sa = a.mu[leaf] * h;
-#pragma unroll
-            for (int c = 0; c < 3; ++c)
-#pragma unroll
-                for (int m = 0; m < 27; ++m) w[c][m] *= sa;
-        }
     }
     if (DO_BT) {
-        double p8[8];
 #pragma unroll
         for (int v = 0; v < 8; ++v) p8[v] = s * gather_p(a, src_p, rp[v], size_t(leaf) * 8 + v);
-        q2::bt_component<0>(p8, w[0]);
-        q2::bt_component<1>(p8, w[1]);
-        q2::bt_component<2>(p8, w[2]);
+    }
+    q2::cell_stokes<DO_A, DO_BT, DO_B>(u, p8, DO_A ? a.mu[leaf] * h : 0.0, w, pb);
+    if (DO_B) {
+#pragma unroll
+        for (int v = 0; v < 8; ++v) scatter_p(a, dst_p, rp[v], s * pb[v], size_t(leaf) * 8 + v);
     }
     if (DO_A || DO_BT) {
 #pragma unroll

@@ -141,53 +141,26 @@ __global__ void __launch_bounds__(kCellThreads) k_stokes_blocks(int n, double h,
     const int M = 2 * n + 1;
     const size_t nodes = size_t(M) * M * M;
     const int P = n + 1;
-    CT u[3][27], w[3][27];
+    CT u[3][27], w[3][27], p8[8], pb[8];
+    // B^T and B carry the factor -h^2: (B^T p)_(c,m) = -int d_c(phi_m) p_h, (B u)_v = -int div(u_h) psi_v
+    const double s = -h * h;
     if (DO_A || DO_B) gather_io<CT>(src_u, nodes, M, ci, cj, ck, u);
-    if (DO_B) {
-        // (B u)_v = -int div(u_h) psi_v = -h^2 sum_c (moments along each axis) . u_c
-        CT bp[8];
-#pragma unroll
-        for (int v = 0; v < 8; ++v) bp[v] = CT(0);
-        q2::b_component<0>(u[0], bp);
-        q2::b_component<1>(u[1], bp);
-        q2::b_component<2>(u[2], bp);
-        const double s = -h * h;
+    if (DO_BT) {
 #pragma unroll
         for (int v = 0; v < 8; ++v) {
             const size_t vert = size_t(ci + (v & 1)) + size_t(P) * (cj + ((v >> 1) & 1) + size_t(P) * (ck + (v >> 2)));
-            atomicAdd(dst_p + vert, s * to_io(bp[v]));
+            p8[v] = from_io<CT>(s * src_p[vert]);
         }
     }
-    if (DO_A || DO_BT) {
-        if (DO_A) {
-            q2::cell_A(u, w);
-            const CT sA = from_io<CT>(mu[cell] * h);
+    q2::cell_stokes<DO_A, DO_BT, DO_B>(u, p8, DO_A ? from_io<CT>(mu[cell] * h) : CT(0), w, pb);
+    if (DO_B) {
 #pragma unroll
-            for (int c = 0; c < 3; ++c)
-#pragma unroll
-                for (int a = 0; a < 27; ++a) w[c][a] *= sA;
-        } else {
-#pragma unroll
-            for (int c = 0; c < 3; ++c)
-#pragma unroll
-                for (int a = 0; a < 27; ++a) w[c][a] = CT(0);
+        for (int v = 0; v < 8; ++v) {
+            const size_t vert = size_t(ci + (v & 1)) + size_t(P) * (cj + ((v >> 1) & 1) + size_t(P) * (ck + (v >> 2)));
+            atomicAdd(dst_p + vert, s * to_io(pb[v]));
         }
-        if (DO_BT) {
-            // (B^T p)_(c,m) = -int d_c(phi_m) p_h = -h^2 sum_v (moments along each axis) p_v
-            CT p8[8];
-            const double s = -h * h;
-#pragma unroll
-            for (int v = 0; v < 8; ++v) {
-                const size_t vert =
-                    size_t(ci + (v & 1)) + size_t(P) * (cj + ((v >> 1) & 1) + size_t(P) * (ck + (v >> 2)));
-                p8[v] = from_io<CT>(s * src_p[vert]);
-            }
-            q2::bt_component<0>(p8, w[0]);
-            q2::bt_component<1>(p8, w[1]);
-            q2::bt_component<2>(p8, w[2]);
-        }
-        scatter_io<CT>(dst_u, nodes, M, ci, cj, ck, w);
     }
+    if (DO_A || DO_BT) scatter_io<CT>(dst_u, nodes, M, ci, cj, ck, w);
 }
 
 // ---------------------------------------------------------------- pressure mass

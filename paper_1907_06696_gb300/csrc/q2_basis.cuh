@@ -9,14 +9,12 @@
 // The velocity operator of one cube cell of side h with cell viscosity mu is
 //   (A u)_(a,c) = mu h sum_q w_q sum_d sigma_cd(q) d_d phi_a(q),
 //   sigma = grad_ref u + grad_ref u^T   (= 2 eps in reference coordinates),
-// evaluated by sum factorisation in the Gauss-point collocation basis:
-// U = (V x V x V) u interpolates the nodal values to the Gauss points, the
-// reference gradient along axis d is then the 1D collocation derivative DC
-// applied along d, and the transposed sweeps bring the quadrature sums back
-// to the nodes. All 1D tables are compile-time constants computed from the
-// closed-form Lagrange polynomials and Gauss points, and every loop is fully
-// unrolled, so each coefficient (including the quadrature weight of the
-// line) is an immediate operand of one FMA.
+// which on a cube is a fixed 81 x 81 matrix times mu h, a sum of tensor products
+// of 1D integrals. It is applied in the Legendre modes of each axis, where those
+// integrals are diagonal or have two entries (below): 1D transforms of the nodal
+// values to the modes, a diagonal and a few products, and the transposed
+// transforms. Every table is a compile-time constant and every loop fully
+// unrolled, so each coefficient is an immediate operand of one FMA.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -69,20 +67,6 @@ __host__ __device__ constexpr int lin(int a, int o1, int o2) {
 }
 
 // ---------------------------------------------------------------- 1D sweeps
-// x <- V x along AX, in place (nodes -> Gauss points).
-template <int AX, typename T>
-__host__ __device__ __forceinline__ void interp(T* x) {
-#pragma unroll
-    for (int o2 = 0; o2 < 3; ++o2)
-#pragma unroll
-        for (int o1 = 0; o1 < 3; ++o1) {
-            const T a0 = x[lin<AX>(0, o1, o2)], a1 = x[lin<AX>(1, o1, o2)], a2 = x[lin<AX>(2, o1, o2)];
-#pragma unroll
-            for (int q = 0; q < 3; ++q)
-                x[lin<AX>(q, o1, o2)] = T(Vq(q, 0)) * a0 + T(Vq(q, 1)) * a1 + T(Vq(q, 2)) * a2;
-        }
-}
-
 // x <- V^T x along AX, in place (Gauss-point sums -> nodes).
 template <int AX, typename T>
 __host__ __device__ __forceinline__ void interpT(T* x) {
@@ -94,47 +78,6 @@ __host__ __device__ __forceinline__ void interpT(T* x) {
 #pragma unroll
             for (int m = 0; m < 3; ++m)
                 x[lin<AX>(m, o1, o2)] = T(Vq(0, m)) * a0 + T(Vq(1, m)) * a1 + T(Vq(2, m)) * a2;
-        }
-}
-
-// The Gauss points are symmetric about 1/2, so DC(2-q, 2-m) = -DC(q, m): the middle row and
-// column of DC are DC(1,0) (1, 0, -1) and DC(0,1) (1, 0, -1) (DC(1,1) = 0), and gw(0) = gw(2).
-// The sweeps use that for the middle output (two operations instead of three multiply-adds).
-
-// g (+)= DC x along AX (collocation derivative at the Gauss points).
-template <int AX, bool ADD, typename T>
-__host__ __device__ __forceinline__ void deriv(const T* x, T* g) {
-#pragma unroll
-    for (int o2 = 0; o2 < 3; ++o2)
-#pragma unroll
-        for (int o1 = 0; o1 < 3; ++o1) {
-            const T a0 = x[lin<AX>(0, o1, o2)], a1 = x[lin<AX>(1, o1, o2)], a2 = x[lin<AX>(2, o1, o2)];
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                const T v = q == 1 ? T(DC(1, 0)) * (a0 - a2)
-                                   : T(DC(q, 0)) * a0 + T(DC(q, 1)) * a1 + T(DC(q, 2)) * a2;
-                if (ADD) g[lin<AX>(q, o1, o2)] += v; else g[lin<AX>(q, o1, o2)] = v;
-            }
-        }
-}
-
-// w += S * DC^T (W3 .* g) along AX, W3 the 3D quadrature weight of each Gauss point.
-template <int AX, int S, typename T>
-__host__ __device__ __forceinline__ void derivT_w(const T* g, T* w) {
-#pragma unroll
-    for (int o2 = 0; o2 < 3; ++o2)
-#pragma unroll
-        for (int o1 = 0; o1 < 3; ++o1) {
-            const T a0 = g[lin<AX>(0, o1, o2)], a1 = g[lin<AX>(1, o1, o2)], a2 = g[lin<AX>(2, o1, o2)];
-#pragma unroll
-            for (int m = 0; m < 3; ++m) {
-                const double wl = gw(o1) * gw(o2) * double(S);
-                if (m == 1)
-                    w[lin<AX>(1, o1, o2)] += T(DC(0, 1) * gw(0) * wl) * (a0 - a2);
-                else
-                    w[lin<AX>(m, o1, o2)] += T(DC(0, m) * gw(0) * wl) * a0 + T(DC(1, m) * gw(1) * wl) * a1 +
-                                             T(DC(2, m) * gw(2) * wl) * a2;
-            }
         }
 }
 
@@ -203,32 +146,214 @@ __host__ __device__ __forceinline__ void derivT_w(const df64* g, df64* w) {
         }
 }
 
+// ---------------------------------------------------------------- Legendre modes
+// A quadratic on [0,1] with nodal values a0, a1, a2 is w/6 P_0 + d/2 P_1 + e/3 P_2 in the Legendre
+// polynomials of [0,1], with w = a0 + 4 a1 + a2, d = a2 - a0, e = a0 - 2 a1 + a2: small integers only.
+// In these modes the 1D forms of the element integrals are diagonal or have two entries,
+//   int u v   = w w'/36 + d d'/12 + e e'/45,   int u' v' = d d' + 4/3 e e',
+//   int u v'  = w d'/6 + d e'/3,
+// so the element operator is a diagonal plus 12 products per pair of components, and its cost is
+// that of the transforms (4 and 5 operations a line): about 960 operations per cell against 2,633
+// for sweeps through the Gauss points, with half their rounding error (the first and second
+// differences of the nodal values are formed directly). The FP32 product at 128^3 takes 229 us, at
+// 64^3 37 us (320 and 50 us through the Gauss points: gather and atomic adds bound it now), the FP64
+// one at 40^3 166 us (428 us: its FP64 instructions).
+enum Mode { MODE_W = 0, MODE_D = 1, MODE_E = 2 };
+__host__ __device__ constexpr double mode_mass(int a) { return a == 0 ? 1.0 / 36.0 : (a == 1 ? 1.0 / 12.0 : 1.0 / 45.0); }
+__host__ __device__ constexpr double mode_stiff(int a) { return a == 0 ? 0.0 : (a == 1 ? 1.0 : 4.0 / 3.0); }
+// int u v' couples mode a of u with mode a + 1 of v (a = 0, 1).
+__host__ __device__ constexpr double mode_grad(int a) { return a == 0 ? 1.0 / 6.0 : 1.0 / 3.0; }
+// Diagonal of row component c: 2 int d_c u d_c v + sum over the other axes of int d_d u d_d v.
+__host__ __device__ constexpr double mode_diag(int c, int i, int j, int k) {
+    return (c == 0 ? 2.0 : 1.0) * mode_stiff(i) * mode_mass(j) * mode_mass(k) +
+           (c == 1 ? 2.0 : 1.0) * mode_mass(i) * mode_stiff(j) * mode_mass(k) +
+           (c == 2 ? 2.0 : 1.0) * mode_mass(i) * mode_mass(j) * mode_stiff(k);
+}
+
+// Nodal values <-> modes along AX, in place: to_modes x <- (w, d, e), from_modes its transpose.
+template <int AX, typename T>
+__host__ __device__ __forceinline__ void to_modes(T* x) {
+#pragma unroll
+    for (int o2 = 0; o2 < 3; ++o2)
+#pragma unroll
+        for (int o1 = 0; o1 < 3; ++o1) {
+            const T a0 = x[lin<AX>(0, o1, o2)], a1 = x[lin<AX>(1, o1, o2)], a2 = x[lin<AX>(2, o1, o2)];
+            const T s = a0 + a2;
+            x[lin<AX>(MODE_W, o1, o2)] = s + T(4) * a1;
+            x[lin<AX>(MODE_D, o1, o2)] = a2 - a0;
+            x[lin<AX>(MODE_E, o1, o2)] = s - T(2) * a1;
+        }
+}
+template <int AX, typename T>
+__host__ __device__ __forceinline__ void from_modes(T* x) {
+#pragma unroll
+    for (int o2 = 0; o2 < 3; ++o2)
+#pragma unroll
+        for (int o1 = 0; o1 < 3; ++o1) {
+            const T w = x[lin<AX>(MODE_W, o1, o2)], d = x[lin<AX>(MODE_D, o1, o2)], e = x[lin<AX>(MODE_E, o1, o2)];
+            const T t = w + e;
+            x[lin<AX>(0, o1, o2)] = t - d;
+            x[lin<AX>(1, o1, o2)] = T(4) * w - T(2) * e;
+            x[lin<AX>(2, o1, o2)] = t + d;
+        }
+}
+template <typename T>
+__host__ __device__ __forceinline__ void to_modes3(T* x) { to_modes<0>(x); to_modes<1>(x); to_modes<2>(x); }
+template <typename T>
+__host__ __device__ __forceinline__ void from_modes3(T* x) { from_modes<2>(x); from_modes<1>(x); from_modes<0>(x); }
+
+// Contribution of column component D to mode (i,j,k) of row component C (C != D):
+// int d_C u_D d_D v_C couples v's mode a along C with u's a + 1, and v's b along D with u's b - 1.
+template <int C, int D>
+__host__ __device__ constexpr int mode_partner(int i, int j, int k) {
+    const int m[3] = {i, j, k};
+    if (m[C] > 1 || m[D] < 1) return -1;
+    const int b0 = i + (C == 0) - (D == 0), b1 = j + (C == 1) - (D == 1), b2 = k + (C == 2) - (D == 2);
+    return b0 + 3 * b1 + 9 * b2;
+}
+template <int C, int D>
+__host__ __device__ constexpr double mode_cross(int i, int j, int k) {
+    const int m[3] = {i, j, k};
+    return mode_grad(m[C]) * mode_grad(m[D] - 1) * mode_mass(m[3 - C - D]);
+}
+
+// Modes of row component C of the velocity operator: w = (A U)_C without the factor mu h, U1 and U2
+// the modes of components (C + 1) % 3 and (C + 2) % 3.
+template <int C, typename T>
+__host__ __device__ __forceinline__ void modes_A(const T* U, const T* U1, const T* U2, T* w) {
+    constexpr int D1 = (C + 1) % 3, D2 = (C + 2) % 3;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const int m = i + 3 * j + 9 * k;
+                T v = T(0);
+                if (m != 0) v = T(mode_diag(C, i, j, k)) * U[m];
+                const int p1 = mode_partner<C, D1>(i, j, k), p2 = mode_partner<C, D2>(i, j, k);
+                if (p1 >= 0) v += T(mode_cross<C, D1>(i, j, k)) * U1[p1 < 0 ? 0 : p1];
+                if (p2 >= 0) v += T(mode_cross<C, D2>(i, j, k)) * U2[p2 < 0 ? 0 : p2];
+                w[m] = v;
+            }
+}
+
 // ---------------------------------------------------------------- cell kernels
 // Velocity operator of one reference cell, without the factor mu h:
-// in: u[c][a] nodal values (overwritten by their Gauss-point values);
-// out: w[c][a] = sum_q w_q sum_d sigma_cd d_d phi_a.
+// in: u[c][a] nodal values (overwritten by their modes);
+// out: w[c][a] = int sum_d sigma_cd d_d phi_a, sigma = grad u + grad u^T.
 template <typename T>
 __host__ __device__ __forceinline__ void cell_A(T (&u)[3][27], T (&w)[3][27]) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        interp<0>(u[c]); interp<1>(u[c]); interp<2>(u[c]);
+    for (int c = 0; c < 3; ++c) to_modes3(u[c]);
+    modes_A<0>(u[0], u[1], u[2], w[0]);
+    modes_A<1>(u[1], u[2], u[0], w[1]);
+    modes_A<2>(u[2], u[0], u[1], w[2]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) from_modes3(w[c]);
+}
+
+// ---- B and B^T in the modes: a Q1 pressure with vertex values p0, p1 along an axis has the modes
+// P = p0 + p1, D = p1 - p0 (p = P/2 + D/2 P_1), and int v p = (w P + d D)/12, int v' p = d P/2 + e D/3.
+// So mode (i,j,k) of component C meets the pressure mode with index i - 1 along C and i elsewhere.
+template <int C>
+__host__ __device__ constexpr int mode_pressure(int i, int j, int k) {
+    const int b0 = i - (C == 0), b1 = j - (C == 1), b2 = k - (C == 2);
+    return (b0 < 0 || b0 > 1 || b1 < 0 || b1 > 1 || b2 < 0 || b2 > 1) ? -1 : b0 + 2 * b1 + 4 * b2;
+}
+template <int C>
+__host__ __device__ constexpr double mode_moment(int i, int j, int k) {
+    const int m[3] = {i, j, k};
+    return (m[C] == 1 ? 1.0 / 2.0 : 1.0 / 3.0) / 144.0;
+}
+// Vertex values -> pressure modes (in place), and the transpose.
+template <typename T>
+__host__ __device__ __forceinline__ void to_pressure_modes(T (&p)[8]) {
+#pragma unroll
+    for (int s = 1; s < 8; s *= 2)
+#pragma unroll
+        for (int v = 0; v < 8; ++v)
+            if (!(v & s)) {
+                const T a = p[v], b = p[v + s];
+                p[v] = a + b;
+                p[v + s] = b - a;
+            }
+}
+template <typename T>
+__host__ __device__ __forceinline__ void from_pressure_modes(T (&p)[8]) {
+#pragma unroll
+    for (int s = 1; s < 8; s *= 2)
+#pragma unroll
+        for (int v = 0; v < 8; ++v)
+            if (!(v & s)) {
+                const T a = p[v], b = p[v + s];
+                p[v] = a - b;
+                p[v + s] = a + b;
+            }
+}
+// w += modes of int d_C(phi) p (B^T without -h^2); P += pressure modes of int d_C(u_C) psi (B without -h^2).
+template <int C, typename T>
+__host__ __device__ __forceinline__ void modes_BT(const T (&P)[8], T* w) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const int q = mode_pressure<C>(i, j, k);
+                if (q >= 0) w[i + 3 * j + 9 * k] += T(mode_moment<C>(i, j, k)) * P[q < 0 ? 0 : q];
+            }
+}
+template <int C, typename T>
+__host__ __device__ __forceinline__ void modes_B(const T* U, T (&P)[8]) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const int q = mode_pressure<C>(i, j, k);
+                if (q >= 0) P[q < 0 ? 0 : q] += T(mode_moment<C>(i, j, k)) * U[i + 3 * j + 9 * k];
+            }
+}
+
+// The blocks [A, B^T; B, 0] of one cell: in: u[c] nodal values (DO_A or DO_B; overwritten by their
+// modes), p vertex values times -h^2 (DO_BT; overwritten), sA = mu h; out: w = sA A u + B^T p
+// (DO_A or DO_BT), pb = B u without -h^2 (DO_B).
+template <bool DO_A, bool DO_BT, bool DO_B, typename T>
+__host__ __device__ __forceinline__ void cell_stokes(T (&u)[3][27], T (&p)[8], T sA, T (&w)[3][27], T (&pb)[8]) {
+    if (DO_A || DO_B) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) to_modes3(u[c]);
     }
+    if (DO_B) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
+        for (int v = 0; v < 8; ++v) pb[v] = T(0);
+        modes_B<0>(u[0], pb);
+        modes_B<1>(u[1], pb);
+        modes_B<2>(u[2], pb);
+        from_pressure_modes(pb);
+    }
+    if (DO_A) {
+        modes_A<0>(u[0], u[1], u[2], w[0]);
+        modes_A<1>(u[1], u[2], u[0], w[1]);
+        modes_A<2>(u[2], u[0], u[1], w[2]);
+    }
+    if (DO_A || DO_BT) {
 #pragma unroll
-        for (int a = 0; a < 27; ++a) w[c][a] = T(0);
-    T g[27];
-    // sigma_cc = 2 d_c U_c
-    deriv<0, false>(u[0], g); derivT_w<0, 2>(g, w[0]);
-    deriv<1, false>(u[1], g); derivT_w<1, 2>(g, w[1]);
-    deriv<2, false>(u[2], g); derivT_w<2, 2>(g, w[2]);
-    // sigma_cd = d_d U_c + d_c U_d, c < d, added to rows (c, d) and (d, c)
-    deriv<1, false>(u[0], g); deriv<0, true>(u[1], g); derivT_w<1, 1>(g, w[0]); derivT_w<0, 1>(g, w[1]);
-    deriv<2, false>(u[0], g); deriv<0, true>(u[2], g); derivT_w<2, 1>(g, w[0]); derivT_w<0, 1>(g, w[2]);
-    deriv<2, false>(u[1], g); deriv<1, true>(u[2], g); derivT_w<2, 1>(g, w[1]); derivT_w<1, 1>(g, w[2]);
+        for (int c = 0; c < 3; ++c)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        interpT<0>(w[c]); interpT<1>(w[c]); interpT<2>(w[c]);
+            for (int m = 0; m < 27; ++m) w[c][m] = DO_A ? w[c][m] * sA : T(0);
+    }
+    if (DO_BT) {
+        to_pressure_modes(p);
+        modes_BT<0>(p, w[0]);
+        modes_BT<1>(p, w[1]);
+        modes_BT<2>(p, w[2]);
+    }
+    if (DO_A || DO_BT) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) from_modes3(w[c]);
     }
 }
 
