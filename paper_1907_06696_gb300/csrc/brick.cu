@@ -481,7 +481,10 @@ cudaError_t accumulate(const BrickArgs<T>& a, T* acc, int bs, const TcArgs* tc, 
             return cudaGetLastError();
         }
     }
-    return launch_cell<T>(a, acc, bs == kSplitKernel ? 128 : bs, s);
+    if constexpr (sizeof(T) == 8)   // FP64 to its accuracy on the integer pipes (outer.cuh)
+        return launch_outer_fix(make_geom(a.n), a.mu, a.src, nullptr, acc, nullptr, true, false, false, s);
+    else
+        return launch_cell<T>(a, acc, bs == kSplitKernel ? 128 : bs, s);
 }
 
 template <typename T>

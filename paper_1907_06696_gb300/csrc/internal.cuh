@@ -35,13 +35,14 @@ inline LevelGeom make_geom(int n) {
 // Finest-level FP64 blocks. Flags select the parts of [[A, B^T], [B, 0]]:
 // the u-part of dst gets A u (DO_A) + B^T p (DO_BT), the p-part gets B u (DO_B).
 // src_u / src_p may be null when unused; dst parts are overwritten.
-// df64 selects double-float arithmetic on the FP32 pipes (q2::df64) instead of native FP64.
+// bt_df64: B^T alone may be formed in double-float (launch_bt_gather); every other block is to FP64 accuracy.
 cudaError_t launch_stokes_blocks(const LevelGeom& g, const double* mu, const double* src_u, const double* src_p,
-                                 double* dst_u, double* dst_p, bool do_a, bool do_bt, bool do_b, bool df64,
+                                 double* dst_u, double* dst_p, bool do_a, bool do_bt, bool do_b, bool bt_df64,
                                  cudaStream_t s);
-// The same blocks in double-float arithmetic, one velocity component per thread (outer.cu).
-cudaError_t launch_outer_df64(const LevelGeom& g, const double* mu, const double* src_u, const double* src_p,
-                              double* dst_u, double* dst_p, bool do_a, bool do_bt, bool do_b, cudaStream_t s);
+// The same blocks added to dst in fixed point, one velocity component per thread (outer.cu); boundary
+// rows get nothing.
+cudaError_t launch_outer_fix(const LevelGeom& g, const double* mu, const double* src_u, const double* src_p,
+                             double* dst_u, double* dst_p, bool do_a, bool do_bt, bool do_b, cudaStream_t s);
 // The whole outer operator [A B^T; B 0] to FP64 accuracy on the tensor cores, by exact integer
 // products with fixed-point digit slices (outer_tc.cu; the caller clears dst_u and dst_p and copies
 // the constrained rows afterwards). outer_tc_setup builds the f16 table (outer_tc_table_bytes()

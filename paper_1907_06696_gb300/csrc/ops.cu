@@ -1,10 +1,7 @@
 // ops.cu -- matrix-free Q2-Q1 operators and the set-up kernels.
 //
-// The FP64 outer operator [A, B^T; B, 0] (Section 2.1): one thread per cube
-//   cell, sum-factorised A (q2::cell_A) and the 1D-moment tensor products of
-//   B and B^T; contributions are accumulated into the zeroed outputs with
-//   atomic adds and constrained (boundary-node) rows then get src. (The level
-//   operators of the V-cycle use the brick-tiled kernel of brick.cuh.)
+// The FP64 outer operator [A, B^T; B, 0] (Section 2.1): the fixed-point kernel of outer.cuh adds the
+//   cells' contributions into the zeroed outputs; constrained (boundary-node) rows then get src.
 // M_p (Section 2.2.2): Q1 mass matrix weighted by 1/mu per cell.
 // Set-up: viscosity at the Gauss points and its harmonic cell average
 //   (Section 2.3), Q0 restriction (parent = mean of children, Section 2.3),
@@ -27,86 +24,7 @@ namespace stk {
 
 namespace {
 
-constexpr int kCellThreads = 128;
-
 __device__ __forceinline__ bool on_bnd(int gi, int M) { return gi == 0 || gi == M - 1; }
-
-template <typename T>
-__device__ __forceinline__ void gather_u(const T* __restrict__ src, size_t nodes, int M, int ci, int cj, int ck,
-                                         T (&u)[3][27]) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                const int gi = 2 * ci + i, gj = 2 * cj + j, gk = 2 * ck + k;
-                const bool b = on_bnd(gi, M) || on_bnd(gj, M) || on_bnd(gk, M);
-                const size_t node = size_t(gi) + size_t(M) * (gj + size_t(M) * gk);
-#pragma unroll
-                for (int c = 0; c < 3; ++c) u[c][i + 3 * j + 9 * k] = b ? T(0) : src[c * nodes + node];
-            }
-}
-
-__device__ __forceinline__ double to_io(double v) { return v; }
-__device__ __forceinline__ double to_io(const q2::df64& v) { return double(v.hi) + double(v.lo); }
-template <typename CT> __device__ __forceinline__ CT from_io(double v);
-template <> __device__ __forceinline__ double from_io<double>(double v) { return v; }
-template <> __device__ __forceinline__ q2::df64 from_io<q2::df64>(double v) { return q2::from_double(v); }
-
-// dst += w (converted to FP64) on the free nodes of one cell.
-template <typename CT>
-__device__ __forceinline__ void scatter_io(double* __restrict__ dst, size_t nodes, int M, int ci, int cj, int ck,
-                                           const CT (&w)[3][27]) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                const int gi = 2 * ci + i, gj = 2 * cj + j, gk = 2 * ck + k;
-                if (on_bnd(gi, M) || on_bnd(gj, M) || on_bnd(gk, M)) continue;
-                const size_t node = size_t(gi) + size_t(M) * (gj + size_t(M) * gk);
-#pragma unroll
-                for (int c = 0; c < 3; ++c) atomicAdd(dst + c * nodes + node, to_io(w[c][i + 3 * j + 9 * k]));
-            }
-}
-
-// u = src on the free nodes of one cell, 0 on constrained ones, converted to the compute type.
-template <typename CT>
-__device__ __forceinline__ void gather_io(const double* __restrict__ src, size_t nodes, int M, int ci, int cj, int ck,
-                                          CT (&u)[3][27]) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                const int gi = 2 * ci + i, gj = 2 * cj + j, gk = 2 * ck + k;
-                const bool b = on_bnd(gi, M) || on_bnd(gj, M) || on_bnd(gk, M);
-                const size_t node = size_t(gi) + size_t(M) * (gj + size_t(M) * gk);
-#pragma unroll
-                for (int c = 0; c < 3; ++c) u[c][i + 3 * j + 9 * k] = b ? CT(0) : from_io<CT>(src[c * nodes + node]);
-            }
-}
-
-template <typename T>
-__device__ __forceinline__ void scatter_u(T* __restrict__ dst, size_t nodes, int M, int ci, int cj, int ck,
-                                          const T (&w)[3][27], T scale) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                const int gi = 2 * ci + i, gj = 2 * cj + j, gk = 2 * ck + k;
-                const bool b = on_bnd(gi, M) || on_bnd(gj, M) || on_bnd(gk, M);
-                if (b) continue;
-                const size_t node = size_t(gi) + size_t(M) * (gj + size_t(M) * gk);
-#pragma unroll
-                for (int c = 0; c < 3; ++c) atomicAdd(dst + c * nodes + node, scale * w[c][i + 3 * j + 9 * k]);
-            }
-}
 
 // Boundary nodes of an M^3 lattice: 6 faces of M*M nodes (edges repeated; writes are identical).
 template <typename T>
@@ -123,44 +41,6 @@ __global__ void k_copy_boundary(int M, const T* __restrict__ in, T* __restrict__
     const size_t node = size_t(i) + size_t(M) * (j + size_t(M) * k);
 #pragma unroll
     for (int c = 0; c < 3; ++c) out[c * nodes + node] = in ? in[c * nodes + node] : T(0);
-}
-
-// ---------------------------------------------------------------- Stokes blocks (FP64 in/out)
-// Native FP64, one thread per cell (CT = double). The double-float variant is the
-// component-split kernel of outer.cuh.
-template <typename CT, bool DO_A, bool DO_BT, bool DO_B>
-__global__ void __launch_bounds__(kCellThreads) k_stokes_blocks(int n, double h, const double* __restrict__ mu,
-                                                                const double* __restrict__ src_u,
-                                                                const double* __restrict__ src_p,
-                                                                double* __restrict__ dst_u,
-                                                                double* __restrict__ dst_p) {
-    const size_t cell = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    const size_t cells = size_t(n) * n * n;
-    if (cell >= cells) return;
-    const int ci = int(cell % n), cj = int((cell / n) % n), ck = int(cell / (size_t(n) * n));
-    const int M = 2 * n + 1;
-    const size_t nodes = size_t(M) * M * M;
-    const int P = n + 1;
-    CT u[3][27], w[3][27], p8[8], pb[8];
-    // B^T and B carry the factor -h^2: (B^T p)_(c,m) = -int d_c(phi_m) p_h, (B u)_v = -int div(u_h) psi_v
-    const double s = -h * h;
-    if (DO_A || DO_B) gather_io<CT>(src_u, nodes, M, ci, cj, ck, u);
-    if (DO_BT) {
-#pragma unroll
-        for (int v = 0; v < 8; ++v) {
-            const size_t vert = size_t(ci + (v & 1)) + size_t(P) * (cj + ((v >> 1) & 1) + size_t(P) * (ck + (v >> 2)));
-            p8[v] = from_io<CT>(s * src_p[vert]);
-        }
-    }
-    q2::cell_stokes<DO_A, DO_BT, DO_B>(u, p8, DO_A ? from_io<CT>(mu[cell] * h) : CT(0), w, pb);
-    if (DO_B) {
-#pragma unroll
-        for (int v = 0; v < 8; ++v) {
-            const size_t vert = size_t(ci + (v & 1)) + size_t(P) * (cj + ((v >> 1) & 1) + size_t(P) * (ck + (v >> 2)));
-            atomicAdd(dst_p + vert, s * to_io(pb[v]));
-        }
-    }
-    if (DO_A || DO_BT) scatter_io<CT>(dst_u, nodes, M, ci, cj, ck, w);
 }
 
 // ---------------------------------------------------------------- pressure mass
@@ -418,31 +298,13 @@ cudaError_t launch_zero_boundary(const LevelGeom& g, T* x, cudaStream_t s) {
 template cudaError_t launch_zero_boundary<float>(const LevelGeom&, float*, cudaStream_t);
 template cudaError_t launch_zero_boundary<double>(const LevelGeom&, double*, cudaStream_t);
 
-template <typename CT>
-cudaError_t stokes_blocks_ct(const LevelGeom& g, const double* mu, const double* src_u, const double* src_p,
-                             double* dst_u, double* dst_p, bool do_a, bool do_bt, bool do_b, cudaStream_t s) {
-    const unsigned nb = blocks_for(g.cells, kCellThreads);
-    const double h = g.h;
-    if (do_a && do_bt && do_b)
-        LAUNCH(PROF_STOKES_F64, s, (k_stokes_blocks<CT, true, true, true><<<nb, kCellThreads, 0, s>>>(g.n, h, mu, src_u, src_p, dst_u, dst_p)));
-    else if (do_a && !do_bt && !do_b)
-        LAUNCH(PROF_STOKES_F64, s, (k_stokes_blocks<CT, true, false, false><<<nb, kCellThreads, 0, s>>>(g.n, h, mu, src_u, src_p, dst_u, dst_p)));
-    else if (!do_a && do_bt && !do_b)
-        LAUNCH(PROF_BT_F64, s, (k_stokes_blocks<CT, false, true, false><<<nb, kCellThreads, 0, s>>>(g.n, h, mu, src_u, src_p, dst_u, dst_p)));
-    else if (!do_a && !do_bt && do_b)
-        LAUNCH(PROF_STOKES_F64, s, (k_stokes_blocks<CT, false, false, true><<<nb, kCellThreads, 0, s>>>(g.n, h, mu, src_u, src_p, dst_u, dst_p)));
-    else
-        return cudaErrorInvalidValue;
-    return cudaGetLastError();
-}
-
 cudaError_t launch_stokes_blocks(const LevelGeom& g, const double* mu, const double* src_u, const double* src_p,
-                                 double* dst_u, double* dst_p, bool do_a, bool do_bt, bool do_b, bool df64,
+                                 double* dst_u, double* dst_p, bool do_a, bool do_bt, bool do_b, bool bt_df64,
                                  cudaStream_t s) {
     cudaError_t e;
-    // B^T alone (the preconditioner's): the gather writes every velocity entry, no clear needed;
-    // its blocks hold one thread per vertex of a line (n + 1 <= 1024)
-    if (df64 && !do_a && do_bt && !do_b && g.n + 1 <= 1024) return launch_bt_gather(g, src_p, dst_u, s);
+    // B^T alone (the preconditioner's) in double-float: the gather writes every velocity entry, no
+    // clear needed; its blocks hold one thread per vertex of a line (n + 1 <= 1024)
+    if (bt_df64 && !do_a && do_bt && !do_b && g.n + 1 <= 1024) return launch_bt_gather(g, src_p, dst_u, s);
     if (do_a || do_bt) {
         e = cudaMemsetAsync(dst_u, 0, g.n_u * sizeof(double), s);
         if (e != cudaSuccess) return e;
@@ -451,10 +313,7 @@ cudaError_t launch_stokes_blocks(const LevelGeom& g, const double* mu, const dou
         e = cudaMemsetAsync(dst_p, 0, g.n_p * sizeof(double), s);
         if (e != cudaSuccess) return e;
     }
-    // double-float on the FP32 pipes for every block (GB300's FP64 pipe retires 1/72 of the FP32
-    // rate): B^T alone, the preconditioner's, takes 148 us at 64^3 against 221 us in native FP64
-    e = df64 ? launch_outer_df64(g, mu, src_u, src_p, dst_u, dst_p, do_a, do_bt, do_b, s)
-                       : stokes_blocks_ct<double>(g, mu, src_u, src_p, dst_u, dst_p, do_a, do_bt, do_b, s);
+    e = launch_outer_fix(g, mu, src_u, src_p, dst_u, dst_p, do_a, do_bt, do_b, s);
     if (e != cudaSuccess) return e;
     if (do_a) {
         const size_t nbd = 6 * size_t(g.M) * g.M;

@@ -1,22 +1,31 @@
 // outer.cuh -- the FP64-interface outer Stokes blocks [A, B^T; B, 0]
-// (Section 2.1, eq. stokes_linear_system) in double-float arithmetic with one
-// velocity component per thread.
+// (Section 2.1, eq. stokes_linear_system) in fixed point, in the Legendre modes of
+// q2_basis.cuh, with one velocity component per thread.
+//
+// GB300 issues one FP64 instruction per ~38 integer ones, and the transforms between nodal values
+// and modes multiply by 1, 2 and 4 only. So each cell's values are written once as 64-bit integers
+// against the cell's largest magnitude and everything up to the last scaling is integer arithmetic,
+// exact but for the bits it drops:
+//   u = X 2^(Eu - 54), |X| <= 2^54 (rounding 2^-55 of the cell's largest |u|), modes
+//       U = (T x T x T) X, |U| <= 2^(54 + 7.76);
+//   97200 A is an integer matrix in the modes (stiffness (0,3,4)/3, mass (5,15,4)/180, derivative
+//       couplings (1,2)/6): Y = 97200 A U, |Y| <= 2^(54 + 15.99), formed in 96 bits and kept without
+//       its lowest 12;
+//   B^T p is added as (3|2) p' with p' = 112.5 h/mu p in the same units;
+//   the transposed transform gives |result| < 2^(42 + 20.43) (sums that leave 64 bits on the way
+//       return: two's complement), rounded to 53 bits and multiplied by mu h 2^E / 97200.
+// B u is (3|2) U / 864, |result| <= 2^(54 + 10.1) / 2.
+// The error is that of FP64 arithmetic (measured against exact sums on 12^3 cells, velocity rows: 1.2e-16
+// relative on random and 2.7e-16 on smooth fields; sum factorisation in FP64 4.8e-16 and 2.3e-15,
+// in double-float pairs 6.4e-15 and 3.6e-14).
 //
 // A CTA holds 32 cells and 96 threads; warp c owns velocity component c of
-// the 32 cells (lane g = cell g). Per thread, with U_c the Gauss-point values
-// of component c and DC_d the collocation derivative along axis d:
-//   W_c  = 2 DC_c^T (w .* DC_c U_c)                          (diagonal term)
-//        + sum_{d != c} DC_d^T (w .* (DC_d U_c + DC_c U_d))   (symmetric pairs)
-// The products DC_d U_c (d != c) and DC_c U_c are exchanged through shared
-// memory so that each thread only keeps its own component: the symmetric pair of
-// components c and c+1 (mod 3) has one slot, which warp c writes and warp c+1 adds to
-// after a barrier (three pair slots instead of six ordered ones: 41.5 KB of shared memory
-// per CTA, four CTAs per SM). Then
-// out_c = mu h V^T W_c - h^2 (moments of B^T) p, and B's moments of u_c are
-// added into the pressure output per component.
+// the 32 cells (lane g = cell g) and the three exchange their modes through shared memory (20.7 KB).
 // The phases are plain functions of the thread index so that a host program
 // can run them and compare with the FP64 kernel.
 #pragma once
+
+#include <cstring>
 
 #include "df64.cuh"
 #include "q2_basis.cuh"
@@ -37,16 +46,17 @@ struct OuterArgs {
     double* dst_p;
 };
 
-// Shared exchange buffer: X[c][q][g] = DC_{c+1} U_c + DC_c U_{c+1} (indices mod 3), the
-// symmetric pair of components c and c+1, and the diagonal term Dg[c][q][g] = DC_c U_c.
+// Exchange buffers: U[c][m][g] = mode m of component c in warp c's own frame, P[v][g] = pressure at
+// vertex v (the FP64 bits, after phase 1b the fixed-point value), biased exponents of the largest
+// |u| and |p| that each warp saw.
 struct OuterShared {
-    q2::df64 X[3][27][kOuterCells];
-    q2::df64 Dg[3][27][kOuterCells];
+    long long U[3][27][kOuterCells];
+    long long P[8][kOuterCells];
+    int eu[3][kOuterCells], ep[3][kOuterCells];
 };
 
 __host__ __device__ __forceinline__ bool outer_bnd(int g, int M) { return g == 0 || g == M - 1; }
 
-template <int C>
 __host__ __device__ __forceinline__ void outer_atomic_add(double* p, double v) {
 #ifdef __CUDA_ARCH__
     atomicAdd(p, v);
@@ -55,17 +65,123 @@ __host__ __device__ __forceinline__ void outer_atomic_add(double* p, double v) {
 #endif
 }
 
+// ---- fixed point
+constexpr int kFixBits = 54;      // |X| <= 2^54
+constexpr int kFixMid = 12;       // bits dropped after the element matrix
+constexpr int kFixMinExp = 64;    // cells whose largest value is below 2^-958 read as 0
+
+__host__ __device__ __forceinline__ double bits_to_dbl(long long b) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double(b);
+#else
+    double d;
+    __builtin_memcpy(&d, &b, sizeof d);
+    return d;
+#endif
+}
+__host__ __device__ __forceinline__ long long mul_hi(long long a, long long b) {
+#ifdef __CUDA_ARCH__
+    return __mul64hi(a, b);
+#else
+    return (long long)(((__int128)a * b) >> 64);
+#endif
+}
+__host__ __device__ __forceinline__ int clz_u64(unsigned long long x) {   // x > 0
+#ifdef __CUDA_ARCH__
+    return __clzll((long long)x);
+#else
+    return __builtin_clzll(x);
+#endif
+}
+__host__ __device__ __forceinline__ int exp_of(long long bits) { return int(bits >> 52) & 0x7FF; }
+
+// X = round(v 2^(54 - E)) for the FP64 bits of v, |v| < 2^E with E = emax - 1022 (emax >= kFixMinExp,
+// the largest biased exponent of the cell). Zero, and what is below 2^-60 of the largest, gives 0.
+__host__ __device__ __forceinline__ long long fix_round(long long bits, int emax) {
+    const unsigned long long m = (unsigned long long)(bits & 0xFFFFFFFFFFFFFLL) << 2 | (1ull << 54);
+    const int r = emax - exp_of(bits);
+    const long long X = (long long)(((m >> (r < 60 ? r : 60)) + 1) >> 1);
+    const long long s = bits >> 63;
+    return (X ^ s) - s;
+}
+
+// x scale with x rounded to 53 bits (half up), |x| < 2^63: the significand is placed by integer
+// instructions, one FP64 multiplication.
+__host__ __device__ __forceinline__ double fix_out(long long x, double scale) {
+    const long long sign = x >> 63;
+    const unsigned long long a = (unsigned long long)((x ^ sign) - sign);
+    const int lz = a ? clz_u64(a) : 0;
+    const unsigned long long v = a << lz;
+    const long long m = (long long)((v >> 11) + ((v >> 10) & 1));
+    const long long b = a ? m + ((long long)(1085 - lz) << 52) : 0;   // m in [2^52, 2^53]: |x| = m 2^(11 - lz)
+    return bits_to_dbl(b | (sign & (long long)(1ull << 63))) * scale;
+}
+// s 2^e; NaN where the cell holds one (or an infinity).
+__host__ __device__ __forceinline__ double fix_scale(double s, int e, bool zero, bool bad) {
+    if (bad) return bits_to_dbl(0x7FF8000000000000LL);
+    if (zero) return 0.0;
+    const int k = e < -1022 ? -1022 : (e > 1023 ? 1023 : e);
+    return s * bits_to_dbl((long long)(k + 1023) << 52);
+}
+// A 96-bit sum of products of modes with non-negative table entries below 2^12: high and low words apart.
+struct FixSum {
+    long long hi = 0;
+    unsigned long long lo = 0;
+    __host__ __device__ __forceinline__ void add(int c, long long u) {
+        hi += (long long)c * int(u >> 32);
+        lo += (unsigned long long)unsigned(c) * unsigned(u);
+    }
+    __host__ __device__ __forceinline__ long long shifted() const {
+        return (hi << (32 - kFixMid)) + (long long)(lo >> kFixMid);
+    }
+};
+
+// 97200 A in the modes, own component along local axis 0 (mode_diag and mode_cross as integers).
+__host__ __device__ constexpr int fix_stiff(int a) { return a == 0 ? 0 : (a == 1 ? 3 : 4); }
+__host__ __device__ constexpr int fix_mass(int a) { return a == 0 ? 5 : (a == 1 ? 15 : 4); }
+__host__ __device__ constexpr int fix_diag(int i, int j, int k) {
+    return 2 * fix_stiff(i) * fix_mass(j) * fix_mass(k) + fix_mass(i) * fix_stiff(j) * fix_mass(k) +
+           fix_mass(i) * fix_mass(j) * fix_stiff(k);
+}
+__host__ __device__ constexpr int fix_cross(int a, int b, int o) { return 15 * (a + 1) * b * fix_mass(o); }
+
+template <int AX>
+__host__ __device__ __forceinline__ void fix_to_modes(long long* x) {
+#pragma unroll
+    for (int o2 = 0; o2 < 3; ++o2)
+#pragma unroll
+        for (int o1 = 0; o1 < 3; ++o1) {
+            long long &a0 = x[q2::lin<AX>(0, o1, o2)], &a1 = x[q2::lin<AX>(1, o1, o2)], &a2 = x[q2::lin<AX>(2, o1, o2)];
+            const long long s = a0 + a2, d = a2 - a0, m = a1;
+            a0 = s + 4 * m;
+            a1 = d;
+            a2 = s - 2 * m;
+        }
+}
+template <int AX>
+__host__ __device__ __forceinline__ void fix_from_modes(long long* x) {
+#pragma unroll
+    for (int o2 = 0; o2 < 3; ++o2)
+#pragma unroll
+        for (int o1 = 0; o1 < 3; ++o1) {
+            long long &w = x[q2::lin<AX>(0, o1, o2)], &d = x[q2::lin<AX>(1, o1, o2)], &e = x[q2::lin<AX>(2, o1, o2)];
+            const long long t = w + e, a1 = 2 * (2 * w - e), dd = d;
+            w = t - dd;
+            d = a1;
+            e = t + dd;
+        }
+}
+
 // Every thread runs the same code: in its local frame the axes are rotated cyclically so that
 // its own velocity component C lies along local axis 0 (local axes = global axes C, C+1, C+2
 // mod 3). The operator is invariant under this relabelling (same 1D matrices and weights on every
-// axis), so only the addressing differs between the three warps: gathers, scatters and the
-// shared-memory exchange map local indices to global ones at run time. This keeps one copy of
-// the unrolled double-float code (three copies overflow the instruction cache).
+// axis), so only the addressing differs between the three warps: gathers and scatters map local
+// indices to global ones at run time, and warp C finds mode (i, j, k) of component C + 1 in that
+// warp's frame at (j, k, i), of component C + 2 at (k, i, j). This keeps one copy of
+// the unrolled code in the instruction cache.
 struct OuterFrame {
     int C;            // velocity component of this thread
-    int D1, D2;       // global axes of local axes 1 and 2
     size_t sn[3];     // global node strides of local axes 0, 1, 2
-    int sq[3];        // global Gauss-point strides (1, 3, 9 rotated)
     int sv[3];        // global Q1-vertex bits (1, 2, 4 rotated)
     int cl[3];        // cell coordinates along the local axes
     int ci, cj, ck;   // global cell coordinates
@@ -74,152 +190,177 @@ struct OuterFrame {
 __host__ __device__ __forceinline__ OuterFrame outer_frame(const OuterArgs& a, int C, size_t cell) {
     OuterFrame f;
     f.C = C;
-    f.D1 = (C + 1) % 3;
-    f.D2 = (C + 2) % 3;
     f.ci = int(cell % a.n);
     f.cj = int((cell / a.n) % a.n);
     f.ck = int(cell / (size_t(a.n) * a.n));
-    const size_t ns[3] = {1, size_t(a.M), size_t(a.M) * a.M};
-    const int qs[3] = {1, 3, 9}, vs[3] = {1, 2, 4};
-    const int cc[3] = {f.ci, f.cj, f.ck};
-    const int ax[3] = {C, f.D1, f.D2};
-    for (int d = 0; d < 3; ++d) {
-        f.sn[d] = ns[ax[d]];
-        f.sq[d] = qs[ax[d]];
-        f.sv[d] = vs[ax[d]];
-        f.cl[d] = cc[ax[d]];
+    const size_t M = size_t(a.M);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {   // selects, not indexed arrays: those would live in local memory
+        const int ax = (C + d) % 3;
+        f.sn[d] = ax == 0 ? 1 : (ax == 1 ? M : M * M);
+        f.sv[d] = 1 << ax;
+        f.cl[d] = ax == 0 ? f.ci : (ax == 1 ? f.cj : f.ck);
     }
     return f;
 }
 
-// Global Gauss-point index of local index q (= qa + 3 qb + 9 qc).
-__host__ __device__ __forceinline__ int outer_gq(const OuterFrame& f, int q) {
-    return (q % 3) * f.sq[0] + ((q / 3) % 3) * f.sq[1] + (q / 9) * f.sq[2];
+__host__ __device__ __forceinline__ size_t outer_vertex(const OuterArgs& a, const OuterFrame& f, int gv) {
+    const int P = a.n + 1;
+    return size_t(f.ci + (gv & 1)) + size_t(P) * (f.cj + ((gv >> 1) & 1) + size_t(P) * (f.ck + (gv >> 2)));
 }
 
-// Phase 1: gather own component, B moments, interpolation, and the diagonal derivative
-// DC_0 U and the cross product DC_1 U (local axes) into shared memory; the other cross product
-// DC_2 U is left in T2 for phase 1b.
-template <bool DO_A, bool DO_B>
+// Phase 1: gather the own component (raw FP64 bits, kept in T for phase 1b) and every third
+// pressure vertex, and the largest exponents. V is any 8-byte type; U is the caller's scratch and not used.
+template <bool DO_A, bool DO_B, bool DO_BT = true, typename V>
 __host__ __device__ __forceinline__ void outer_phase1(const OuterArgs& a, int C, int blk, int g, OuterShared& sh,
-                                                      q2::df64 (&U)[27], q2::df64 (&T2)[27]) {
-    using q2::df64;
+                                                      V (&U)[27], V (&T)[27]) {
+    static_assert(sizeof(V) == 8, "an 8-byte slot per value");
+    (void)U;
     const size_t cells = size_t(a.n) * a.n * a.n;
     const size_t cell = size_t(blk) * kOuterCells + g;
     const bool valid = cell < cells;
-#pragma unroll
-    for (int m = 0; m < 27; ++m) U[m] = df64(0);
-    if (!(DO_A || DO_B)) return;
-    if (valid) {
-        const OuterFrame f = outer_frame(a, C, cell);
+    const OuterFrame f = outer_frame(a, C, valid ? cell : 0);
+    if (DO_A || DO_B) {
         const double* src = a.src_u + size_t(C) * a.nodes +
                             (size_t(2 * f.ci) + size_t(a.M) * (size_t(2 * f.cj) + size_t(a.M) * size_t(2 * f.ck)));
+        int e = 0;
 #pragma unroll
         for (int c = 0; c < 3; ++c)
 #pragma unroll
             for (int b = 0; b < 3; ++b)
 #pragma unroll
                 for (int aa = 0; aa < 3; ++aa) {
-                    const int g0 = 2 * f.cl[0] + aa, g1 = 2 * f.cl[1] + b, g2 = 2 * f.cl[2] + c;
-                    if (!(outer_bnd(g0, a.M) || outer_bnd(g1, a.M) || outer_bnd(g2, a.M)))
-                        U[aa + 3 * b + 9 * c] = q2::split_double(src[aa * f.sn[0] + b * f.sn[1] + c * f.sn[2]]);
+                    const bool bnd = !valid || outer_bnd(2 * f.cl[0] + aa, a.M) || outer_bnd(2 * f.cl[1] + b, a.M) ||
+                                     outer_bnd(2 * f.cl[2] + c, a.M);
+                    const double v = bnd ? 0.0 : src[aa * f.sn[0] + b * f.sn[1] + c * f.sn[2]];
+                    const int ev = exp_of((long long)q2::dbl_bits(v));
+                    e = ev > e ? ev : e;
+                    memcpy(&T[aa + 3 * b + 9 * c], &v, 8);
                 }
-        if (DO_B) {
-            df64 bp[8];
-#pragma unroll
-            for (int v = 0; v < 8; ++v) bp[v] = df64(0);
-            q2::b_component<0>(U, bp);
-            const int P = a.n + 1;
-            const double s = -a.h * a.h;
-#pragma unroll
-            for (int v = 0; v < 8; ++v) {
-                const int gv = (v & 1) * f.sv[0] + ((v >> 1) & 1) * f.sv[1] + (v >> 2) * f.sv[2];
-                const size_t vert = size_t(f.ci + (gv & 1)) +
-                                    size_t(P) * (f.cj + ((gv >> 1) & 1) + size_t(P) * (f.ck + (gv >> 2)));
-                outer_atomic_add<0>(a.dst_p + vert, s * bp[v].to_double());
-            }
-        }
-    }
-    if (!DO_A) return;
-    const int D1 = (C + 1) % 3, D2 = (C + 2) % 3;
-    const OuterFrame f = outer_frame(a, C, valid ? cell : 0);
-    q2::interp<0>(U);
-    q2::interp<1>(U);
-    q2::interp<2>(U);
-    df64 T[27];
-    q2::deriv<0, false>(U, T);
-#pragma unroll
-    for (int q = 0; q < 27; ++q) sh.Dg[C][outer_gq(f, q)][g] = T[q];
-    q2::deriv<1, false>(U, T);
-#pragma unroll
-    for (int q = 0; q < 27; ++q) sh.X[C][outer_gq(f, q)][g] = T[q];     // pair (C, D1): writer
-    q2::deriv<2, false>(U, T2);
-    (void)D1;
-    (void)D2;
-}
-
-// Phase 1b (after a barrier): add this thread's DC_2 U (local axis 2 = global axis D2), i.e.
-// DC_{D2} U_C, into the slot of the pair (D2, C), which warp D2 wrote with DC_C U_{D2}.
-template <bool DO_A>
-__host__ __device__ __forceinline__ void outer_phase1b(const OuterArgs& a, int C, int blk, int g, OuterShared& sh,
-                                                       const q2::df64 (&T2)[27]) {
-    if (!DO_A) return;
-    const size_t cells = size_t(a.n) * a.n * a.n;
-    const size_t cell = size_t(blk) * kOuterCells + g;
-    const OuterFrame f = outer_frame(a, C, cell < cells ? cell : 0);
-    const int D2 = f.D2;
-#pragma unroll
-    for (int q = 0; q < 27; ++q) {
-        q2::df64& x = sh.X[D2][outer_gq(f, q)][g];
-        x = x + T2[q];
-    }
-}
-
-// Phase 2 (after a barrier): diagonal and symmetric pairs, transposed interpolation,
-// B^T moments, scatter into the velocity output.
-template <bool DO_A, bool DO_BT>
-__host__ __device__ __forceinline__ void outer_phase2(const OuterArgs& a, int C, int blk, int g, const OuterShared& sh,
-                                                      q2::df64 (&W)[27]) {
-    using q2::df64;
-    const size_t cells = size_t(a.n) * a.n * a.n;
-    const size_t cell = size_t(blk) * kOuterCells + g;
-    if (cell >= cells || !(DO_A || DO_BT)) return;
-    const OuterFrame f = outer_frame(a, C, cell);
-#pragma unroll
-    for (int m = 0; m < 27; ++m) W[m] = df64(0);
-    if (DO_A) {
-        const int D1 = f.D1, D2 = f.D2;
-        df64 T[27];
-#pragma unroll
-        for (int q = 0; q < 27; ++q) T[q] = sh.Dg[C][outer_gq(f, q)][g];
-        q2::derivT_w<0, 2>(T, W);
-#pragma unroll
-        for (int q = 0; q < 27; ++q) T[q] = sh.X[C][outer_gq(f, q)][g];    // pair (C, D1)
-        q2::derivT_w<1, 1>(T, W);
-#pragma unroll
-        for (int q = 0; q < 27; ++q) T[q] = sh.X[D2][outer_gq(f, q)][g];   // pair (D2, C)
-        q2::derivT_w<2, 1>(T, W);
-        (void)D1;
-        q2::interpT<0>(W);
-        q2::interpT<1>(W);
-        q2::interpT<2>(W);
-        const df64 sA = q2::from_double(a.mu[cell] * a.h);
-#pragma unroll
-        for (int m = 0; m < 27; ++m) W[m] *= sA;
+        sh.eu[C][g] = e;
     }
     if (DO_BT) {
-        const int P = a.n + 1;
-        const double s = -a.h * a.h;
-        df64 p8[8];
+        int e = 0;
+        for (int v = C; v < 8; v += 3) {
+            const double p = valid ? a.src_p[outer_vertex(a, f, v)] : 0.0;
+            const long long b = (long long)q2::dbl_bits(p);
+            e = exp_of(b) > e ? exp_of(b) : e;
+            sh.P[v][g] = b;
+        }
+        sh.ep[C][g] = e;
+    }
+}
+
+__host__ __device__ __forceinline__ int max3(const int (&e)[3][kOuterCells], int g) {
+    const int m = e[0][g] > e[1][g] ? e[0][g] : e[1][g];
+    return m > e[2][g] ? m : e[2][g];
+}
+
+// Phase 1b (after a barrier): fixed point against the cell's largest magnitude, and the modes.
+template <bool DO_A, bool DO_B = true, bool DO_BT = true, typename V>
+__host__ __device__ __forceinline__ void outer_phase1b(const OuterArgs&, int C, int, int g, OuterShared& sh,
+                                                       const V (&T)[27]) {
+    if (DO_A || DO_B) {
+        const int e = max3(sh.eu, g);
+        long long X[27];
+#pragma unroll
+        for (int m = 0; m < 27; ++m) {
+            long long b;
+            memcpy(&b, &T[m], 8);
+            X[m] = fix_round(b, e);
+        }
+        fix_to_modes<0>(X);
+        fix_to_modes<1>(X);
+        fix_to_modes<2>(X);
+#pragma unroll
+        for (int m = 0; m < 27; ++m) sh.U[C][m][g] = X[m];
+    }
+    if (DO_BT) {
+        const int e = max3(sh.ep, g);
+        for (int v = C; v < 8; v += 3) sh.P[v][g] = fix_round(sh.P[v][g], e);
+    }
+}
+
+// Phase 2 (after a barrier): the element matrix in the modes, the transposed transform and the
+// scatter into the velocity output; B u at this warp's vertices.
+template <bool DO_A, bool DO_BT, bool DO_B = true, typename V>
+__host__ __device__ __forceinline__ void outer_phase2(const OuterArgs& a, int C, int blk, int g, const OuterShared& sh,
+                                                      V (&W)[27]) {
+    (void)W;
+    const size_t cells = size_t(a.n) * a.n * a.n;
+    const size_t cell = size_t(blk) * kOuterCells + g;
+    if (cell >= cells) return;
+    const OuterFrame f = outer_frame(a, C, cell);
+    const int D1 = (C + 1) % 3, D2 = (C + 2) % 3;
+    const int eu = DO_A || DO_B ? max3(sh.eu, g) : 0;
+    if (DO_B) {
+        long long b[8];
 #pragma unroll
         for (int v = 0; v < 8; ++v) {
-            const int gv = (v & 1) * f.sv[0] + ((v >> 1) & 1) * f.sv[1] + (v >> 2) * f.sv[2];
-            const size_t vert = size_t(f.ci + (gv & 1)) +
-                                size_t(P) * (f.cj + ((gv >> 1) & 1) + size_t(P) * (f.ck + (gv >> 2)));
-            p8[v] = q2::split_double(s * a.src_p[vert]);
+            const int i = v & 1, j = (v >> 1) & 1, k = v >> 2;
+            b[v] = ((3 - i) * sh.U[C][(i + 1) + 3 * j + 9 * k][g] >> 2) + ((3 - j) * sh.U[D1][(j + 1) + 3 * k + 9 * i][g] >> 2) +
+                   ((3 - k) * sh.U[D2][(k + 1) + 3 * i + 9 * j][g] >> 2);
         }
-        q2::bt_component<0>(p8, W);
+        q2::from_pressure_modes(b);
+        const double s = fix_scale(-a.h * a.h / 864.0, eu - 1022 - kFixBits + 2, eu < kFixMinExp, eu == 0x7FF);
+        // the vertex one step along the own axis and its opposite; the two that no rotation moves
+        // go to warps 0 and 1
+        outer_atomic_add(a.dst_p + outer_vertex(a, f, f.sv[0]), fix_out(b[1], s));
+        outer_atomic_add(a.dst_p + outer_vertex(a, f, 7 - f.sv[0]), fix_out(b[6], s));
+        if (C < 2) outer_atomic_add(a.dst_p + outer_vertex(a, f, C == 0 ? 0 : 7), fix_out(C == 0 ? b[0] : b[7], s));
     }
+    if (!(DO_A || DO_BT)) return;
+    const double mu = a.mu[cell];
+    long long Y[27];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const int m = i + 3 * j + 9 * k;
+                FixSum y;
+                if (DO_A) {
+                    if (m != 0) y.add(fix_diag(i, j, k), sh.U[C][m][g]);
+                    if (i < 2 && j > 0) y.add(fix_cross(i, j, k), sh.U[D1][(j - 1) + 3 * k + 9 * (i + 1)][g]);
+                    if (i < 2 && k > 0) y.add(fix_cross(i, k, j), sh.U[D2][(k - 1) + 3 * (i + 1) + 9 * j][g]);
+                }
+                Y[m] = y.shifted();
+            }
+    int E = DO_A && eu >= kFixMinExp ? eu : 0;
+    bool bad = DO_A && eu == 0x7FF;
+    if (DO_BT) {
+        // p' = 112.5 h/mu p: the vertex modes times the factor's significand, |R| <= 2^61; |p'| < 2^(epk - 1022)
+        // may exceed |u| by 2^10 before its share of the result is the larger one
+        const int ep = max3(sh.ep, g);
+        if (ep >= kFixMinExp) {
+            const long long kb = (long long)q2::dbl_bits(112.5 * a.h / mu);
+            const long long km = ((kb & 0xFFFFFFFFFFFFFLL) | (1LL << 52)) << 10;
+            const int epk = ep + exp_of(kb) - 1022;
+            E = E > epk - 10 ? E : epk - 10;
+            long long P[8];
+#pragma unroll
+            for (int v = 0; v < 8; ++v)
+                P[v] = sh.P[(v & 1) * f.sv[0] + ((v >> 1) & 1) * f.sv[1] + (v >> 2) * f.sv[2]][g];
+            q2::to_pressure_modes(P);
+            const int sp = E - epk + 16 < 63 ? E - epk + 16 : 63;
+            const int sa = DO_A ? (E - eu < 63 ? E - eu : 63) : 0;
+            if (sa > 0) {
+#pragma unroll
+                for (int m = 0; m < 27; ++m) Y[m] >>= sa;
+            }
+#pragma unroll
+            for (int v = 0; v < 8; ++v) {
+                const int i = v & 1, j = (v >> 1) & 1, k = v >> 2;
+                Y[(i + 1) + 3 * j + 9 * k] -= (3 - i) * (mul_hi(P[v] * 32, km) >> sp);
+            }
+            bad = bad || ep == 0x7FF;
+        }
+    }
+    fix_from_modes<2>(Y);
+    fix_from_modes<1>(Y);
+    fix_from_modes<0>(Y);
+    const double s = fix_scale(mu * a.h * (1.0 / 97200.0), E - 1022 - kFixBits + kFixMid, E == 0, bad);
     double* dst = a.dst_u + size_t(C) * a.nodes +
                   (size_t(2 * f.ci) + size_t(a.M) * (size_t(2 * f.cj) + size_t(a.M) * size_t(2 * f.ck)));
 #pragma unroll
@@ -230,7 +371,7 @@ __host__ __device__ __forceinline__ void outer_phase2(const OuterArgs& a, int C,
             for (int aa = 0; aa < 3; ++aa) {
                 const int g0 = 2 * f.cl[0] + aa, g1 = 2 * f.cl[1] + b, g2 = 2 * f.cl[2] + c;
                 if (outer_bnd(g0, a.M) || outer_bnd(g1, a.M) || outer_bnd(g2, a.M)) continue;
-                outer_atomic_add<0>(dst + aa * f.sn[0] + b * f.sn[1] + c * f.sn[2], W[aa + 3 * b + 9 * c].to_double());
+                outer_atomic_add(dst + aa * f.sn[0] + b * f.sn[1] + c * f.sn[2], fix_out(Y[aa + 3 * b + 9 * c], s));
             }
 }
 

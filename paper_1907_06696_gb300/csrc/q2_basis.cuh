@@ -43,16 +43,6 @@ __host__ __device__ constexpr double dlag(int m, double x) {
 }
 // V[q][m] = l_m(g_q): nodal values -> Gauss-point values.
 __host__ __device__ constexpr double Vq(int q, int m) { return lag(m, gp(q)); }
-// Derivative of the Lagrange polynomials through the Gauss points, at the Gauss points.
-__host__ __device__ constexpr double DC(int q, int m) {
-    // L_m(x) = prod_{k != m} (x - g_k) / (g_m - g_k)
-    return q == m
-        ? (m == 0 ? 1.0 / (gp(0) - gp(1)) + 1.0 / (gp(0) - gp(2))
-                  : (m == 1 ? 1.0 / (gp(1) - gp(0)) + 1.0 / (gp(1) - gp(2))
-                            : 1.0 / (gp(2) - gp(0)) + 1.0 / (gp(2) - gp(1))))
-        : ((gp(q) - gp(3 - q - m)) /
-           ((gp(m) - gp(q)) * (gp(m) - gp(3 - q - m))));
-}
 // Q1 basis on [0,1] at Gauss point q.
 __host__ __device__ constexpr double Pq(int q, int v) { return v == 0 ? 1.0 - gp(q) : gp(q); }
 // 1D Q1 mass matrix on [0,1] by the same quadrature.
@@ -78,71 +68,6 @@ __host__ __device__ __forceinline__ void interpT(T* x) {
 #pragma unroll
             for (int m = 0; m < 3; ++m)
                 x[lin<AX>(m, o1, o2)] = T(Vq(0, m)) * a0 + T(Vq(1, m)) * a1 + T(Vq(2, m)) * a2;
-        }
-}
-
-// ---------------------------------------------------------------- double-float sweeps
-// The same four sweeps for double-float values, each output formed by dot3 / dot3_acc
-// (one renormalisation per output instead of one per operation).
-template <int AX>
-__host__ __device__ __forceinline__ void interp(df64* x) {
-#pragma unroll
-    for (int o2 = 0; o2 < 3; ++o2)
-#pragma unroll
-        for (int o1 = 0; o1 < 3; ++o1) {
-            const df64 a0 = x[lin<AX>(0, o1, o2)], a1 = x[lin<AX>(1, o1, o2)], a2 = x[lin<AX>(2, o1, o2)];
-#pragma unroll
-            for (int q = 0; q < 3; ++q)
-                x[lin<AX>(q, o1, o2)] = dot3(df64(Vq(q, 0)), a0, df64(Vq(q, 1)), a1, df64(Vq(q, 2)), a2);
-        }
-}
-template <int AX>
-__host__ __device__ __forceinline__ void interpT(df64* x) {
-#pragma unroll
-    for (int o2 = 0; o2 < 3; ++o2)
-#pragma unroll
-        for (int o1 = 0; o1 < 3; ++o1) {
-            const df64 a0 = x[lin<AX>(0, o1, o2)], a1 = x[lin<AX>(1, o1, o2)], a2 = x[lin<AX>(2, o1, o2)];
-#pragma unroll
-            for (int m = 0; m < 3; ++m)
-                x[lin<AX>(m, o1, o2)] = dot3(df64(Vq(0, m)), a0, df64(Vq(1, m)), a1, df64(Vq(2, m)), a2);
-        }
-}
-template <int AX, bool ADD>
-__host__ __device__ __forceinline__ void deriv(const df64* x, df64* g) {
-#pragma unroll
-    for (int o2 = 0; o2 < 3; ++o2)
-#pragma unroll
-        for (int o1 = 0; o1 < 3; ++o1) {
-            const df64 a0 = x[lin<AX>(0, o1, o2)], a1 = x[lin<AX>(1, o1, o2)], a2 = x[lin<AX>(2, o1, o2)];
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                df64& out = g[lin<AX>(q, o1, o2)];
-                if (q == 1)
-                    out = ADD ? out + df64(DC(1, 0)) * (a0 - a2) : df64(DC(1, 0)) * (a0 - a2);
-                else
-                    out = ADD ? dot3_acc(out, df64(DC(q, 0)), a0, df64(DC(q, 1)), a1, df64(DC(q, 2)), a2)
-                              : dot3(df64(DC(q, 0)), a0, df64(DC(q, 1)), a1, df64(DC(q, 2)), a2);
-            }
-        }
-}
-template <int AX, int S>
-__host__ __device__ __forceinline__ void derivT_w(const df64* g, df64* w) {
-#pragma unroll
-    for (int o2 = 0; o2 < 3; ++o2)
-#pragma unroll
-        for (int o1 = 0; o1 < 3; ++o1) {
-            const df64 a0 = g[lin<AX>(0, o1, o2)], a1 = g[lin<AX>(1, o1, o2)], a2 = g[lin<AX>(2, o1, o2)];
-#pragma unroll
-            for (int m = 0; m < 3; ++m) {
-                const double wl = gw(o1) * gw(o2) * double(S);
-                df64& out = w[lin<AX>(m, o1, o2)];
-                if (m == 1)
-                    out = out + df64(DC(0, 1) * gw(0) * wl) * (a0 - a2);
-                else
-                    out = dot3_acc(out, df64(DC(0, m) * gw(0) * wl), a0, df64(DC(1, m) * gw(1) * wl), a1,
-                                   df64(DC(2, m) * gw(2) * wl), a2);
-            }
         }
 }
 
