@@ -125,8 +125,8 @@ struct LevelVecs {
     T* mu = nullptr;  // cell viscosity
     T* dinv = nullptr;
     T* acc = nullptr; // operator accumulator of the cell-parallel kernel (kept at zero between uses)
-    // the fused smoother's second (d, x) pair and its two further accumulators (zero between uses)
-    T* x2 = nullptr;
+    T* x2 = nullptr;  // second iterate of the smoothers that write x out of place
+    // the fused smoother's second direction and its two further accumulators (zero between uses)
     T* d2 = nullptr;
     T* acc2 = nullptr;
     T* acc3 = nullptr;
@@ -298,20 +298,38 @@ double tridiag_max_eig(const std::vector<double>& a, const std::vector<double>& 
 // FP32 levels of at most kSplitMaxN^3 cells take the component-split kernel: there a level
 // operator is one short wave and its time one thread's serial work, which the split divides by 3.
 constexpr int kSplitMaxN = 16;
+// From this size up the FP32 level operator marches over layers with the epilogue in the same launch:
+// a degree-4 smoothing takes 197 / 528 / 1,196 us at 64^3 / 96^3 / 128^3 (cell kernel and vector
+// passes 208 / 702 / 1,624 us); below, its layers are too few to hide one layer's latency (48^3: 90 and
+// 92 us, 32^3: equal, and slower inside the captured V-cycle).
+constexpr int kMarchMinN = 64;
 
 template <typename T>
 int level_kernel(const stokes_ctx* c, int l) {
     const int k = c->opt.vmult_kernel;
     if (k == 1 || k == 2 || k == 3) return k;
     if (sizeof(T) == 4 && c->lev[l].g.n <= kSplitMaxN) return 3;
+    if (sizeof(T) == 4 && c->opt.fused_smoother == 0 && c->lev[l].g.n >= kMarchMinN) return kMarchKernel;
     return c->cell_block;
+}
+
+// The marching operator copies 16-byte units: 16-byte aligned vectors (the level's own are; a caller's
+// view may not be, and takes the cell kernel).
+template <typename... P>
+bool aligned16(const P*... p) { return ((reinterpret_cast<uintptr_t>(p) | ...) & 15u) == 0; }
+
+template <typename T>
+bool marches(const stokes_ctx* c, int l, const T* a, const T* b) {
+    return level_kernel<T>(c, l) == kMarchKernel && aligned16(a, b);
 }
 
 template <typename T>
 stokes_status vmult_level(stokes_ctx* c, int l, const T* src, T* dst, cudaStream_t s) {
     Level& L = c->lev[l];
-    CK(launch_level_op<T>(level_kernel<T>(c, l), L.g, L.planes, EPI_PLAIN, vecs<T>(L).mu, src, dst, nullptr, nullptr,
-                          nullptr, 0.0, 0.0, slots<T>(L), vecs<T>(L).acc, s, &c->tc));
+    int k = level_kernel<T>(c, l);
+    if (k == kMarchKernel && !marches<T>(c, l, src, dst)) k = c->cell_block;
+    CK(launch_level_op<T>(k, L.g, L.planes, EPI_PLAIN, vecs<T>(L).mu, src, dst, nullptr, nullptr, nullptr, 0.0, 0.0,
+                          slots<T>(L), vecs<T>(L).acc, s, &c->tc));
     return STOKES_OK;
 }
 
@@ -320,8 +338,9 @@ template <typename T>
 stokes_status cheb_step(stokes_ctx* c, int l, const T* b, T* x, double c1, double c2, cudaStream_t s) {
     Level& L = c->lev[l];
     LevelVecs<T>& v = vecs<T>(L);
-    CK(launch_level_op<T>(level_kernel<T>(c, l), L.g, L.planes, EPI_CHEB, v.mu, x, nullptr, b, v.dinv, v.d, c1, c2,
-                          slots<T>(L), v.acc, s, &c->tc));
+    const int k = level_kernel<T>(c, l);
+    CK(launch_level_op<T>(k == kMarchKernel ? c->cell_block : k, L.g, L.planes, EPI_CHEB, v.mu, x, nullptr, b, v.dinv, v.d,
+                          c1, c2, slots<T>(L), v.acc, s, &c->tc));
     return STOKES_OK;
 }
 
@@ -334,14 +353,27 @@ stokes_status smooth(stokes_ctx* c, int l, const T* b, T* x, bool zero_guess, cu
     const double sigma = theta / delta;
     double rho = 1.0 / sigma;
     const size_t n = L.g.n_u;
+    // the marching operator writes the new iterate beside the old one (its neighbours read that): the
+    // iterates alternate between x and the level's x2, starting where the last step ends in x
+    const bool march = marches<T>(c, l, b, x);
+    T* X[2] = {x, v.x2};
+    int cur = march ? (c->opt.cheb_degree - (zero_guess ? 1 : 0)) & 1 : 0;
+    auto step = [&](double c1, double c2) -> stokes_status {
+        if (!march) return cheb_step<T>(c, l, b, x, c1, c2, s);
+        if constexpr (sizeof(T) == 4)
+            CK(launch_march(EPI_CHEB, L.g, v.mu, X[cur], X[cur ^ 1], b, v.dinv, v.d, c1, c2, s));
+        cur ^= 1;
+        return STOKES_OK;
+    };
     if (zero_guess) {
-        CK(launch_cheb_update<T>(n, b, nullptr, v.dinv, v.d, x, 0.0, 1.0 / theta, false, s));
+        CK(launch_cheb_update<T>(n, b, nullptr, v.dinv, v.d, X[cur], 0.0, 1.0 / theta, false, s));
     } else {
-        CKS(cheb_step<T>(c, l, b, x, 0.0, 1.0 / theta, s));
+        if (cur == 1) CK(cudaMemcpyAsync(v.x2, x, n * sizeof(T), cudaMemcpyDeviceToDevice, s));
+        CKS(step(0.0, 1.0 / theta));
     }
     for (int it = 1; it < c->opt.cheb_degree; ++it) {
         const double rho_new = 1.0 / (2.0 * sigma - rho);
-        CKS(cheb_step<T>(c, l, b, x, rho_new * rho, 2.0 * rho_new / delta, s));
+        CKS(step(rho_new * rho, 2.0 * rho_new / delta));
         rho = rho_new;
     }
     return STOKES_OK;
@@ -1725,6 +1757,7 @@ stokes_status setup_impl(const stokes_mesh* mesh, const stokes_mu* mu, const sto
     const stokes_options& o = c->opt;
     CKS(validate_options(o));
     CK(brick_configure());
+    CK(march_configure());
     CK(gs_configure());
     c->n = mesh->n;
     c->L = mesh->n_levels;
@@ -1743,6 +1776,10 @@ stokes_status setup_impl(const stokes_mesh* mesh, const stokes_mu* mu, const sto
             CKS(dalloc(c, p, nu));
         CK(cudaMemsetAsync(Lv.v64.acc, 0, nu * sizeof(double), s));
         CK(cudaMemsetAsync(Lv.v32.acc, 0, nu * sizeof(float), s));
+        if (level_kernel<float>(c, l) == kMarchKernel) {   // it leaves the boundary entries as they are: zero
+            CKS(dalloc(c, &Lv.v32.x2, nu));
+            for (float* p : {Lv.v32.x, Lv.v32.r, Lv.v32.x2}) CK(cudaMemsetAsync(p, 0, nu * sizeof(float), s));
+        }
         if (o.fused_smoother == 1 && l > 0) {
             for (auto* p : {&Lv.v64.x2, &Lv.v64.d2, &Lv.v64.acc2, &Lv.v64.acc3}) {
                 CKS(dalloc(c, p, nu));
@@ -2568,7 +2605,8 @@ stokes_status stokes_autotune(stokes_ctx* c, int what, void* stream, int* block_
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     stokes_status st = STOKES_OK;
-    if ((what & 1) && c->opt.vmult_kernel == 0) {   // only the cell kernel has a block size
+    // only the cell kernel has a block size
+    if ((what & 1) && c->opt.vmult_kernel == 0 && level_kernel<float>(c, c->L - 1) == c->cell_block) {
         // threads per block of the cell kernel: the fastest FP32 level operator on the finest level
         float best = 1e30f;
         int best_bs = c->cell_block;
@@ -2816,6 +2854,7 @@ stokes_status stokes_smooth(stokes_ctx* c, int level, int prec, const void* b, v
     if (prec == STOKES_FP32) {
         const float* bf = static_cast<const float*>(b);
         float* xf = static_cast<float*>(x);
+        if (zero_guess && marches<float>(c, level, bf, xf)) CK(launch_zero_boundary<float>(c->lev[level].g, xf, s));
         return fused_level<float>(c, level) ? smooth_fused<float>(c, level, bf, xf, zero_guess != 0, nullptr, s)
                                             : smooth<float>(c, level, bf, xf, zero_guess != 0, s);
     }

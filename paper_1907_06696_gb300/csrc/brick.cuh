@@ -416,6 +416,16 @@ cudaError_t tc_build_table(void* table, int* flag, cudaStream_t s);
 // the cell kernel); the epilogue kernels of launch_level_op consume it.
 cudaError_t launch_cell_tc(const BrickArgs<float>& a, float* acc, const TcArgs& t, cudaStream_t s);
 
+// FP32: A src with its epilogue in one launch (march.cu); 16-byte aligned vectors. Entries on the upper
+// sides of the domain boundary are left as they are, those on the lower sides too or written as the
+// epilogue of a zero product (EPI_PLAIN: 0). EPI_PLAIN: dst = A src; EPI_RESID: dst = b - A src;
+// EPI_CHEB: d = c1 d + c2 dinv (b - A src), dst = src + d (dst is not src). Levels of
+// at least 20 cells per axis.
+constexpr int kMarchKernel = 4;
+cudaError_t launch_march(int epi, const LevelGeom& g, const float* mu, const float* src, float* dst, const float* b,
+                         const float* dinv, float* d, double c1, double c2, cudaStream_t s);
+cudaError_t march_configure();   // shared-memory opt-in; once before any launch or capture
+
 // A x with an epilogue (EPI_PLAIN: dst = A x; EPI_RESID: dst = b - A x;
 // EPI_CHEB: d = c1 d + c2 dinv (b - A x), src += d in place).
 // kernel 0, 64, 128, 256: one thread per cell (blocks of 128, 64, 128, 256 threads) with atomic
@@ -424,6 +434,7 @@ cudaError_t launch_cell_tc(const BrickArgs<float>& a, float* acc, const TcArgs& 
 // kernel 3: FP32: the cell kernel's accumulation with three threads per cell (one per output
 //           component), the same consumer kernels; FP64: kernel 128;
 // kernel 1: the brick-tiled kernel with the epilogue fused (slots: brick_layout(n).total entries);
+// kernel 4: FP32: the marching kernel, EPI_PLAIN and EPI_RESID (EPI_CHEB is out of place: launch_march);
 // kernel 2: FP32: the cell products on the tensor cores, accumulated like kernel 0 (tc must be
 //           given); FP64: kernel 128.
 template <typename T>

@@ -78,7 +78,7 @@ __host__ __device__ __forceinline__ void interpT(T* x) {
 //   int u v   = w w'/36 + d d'/12 + e e'/45,   int u' v' = d d' + 4/3 e e',
 //   int u v'  = w d'/6 + d e'/3,
 // so the element operator is a diagonal plus 12 products per pair of components, and its cost is
-// that of the transforms (4 and 5 operations a line): about 960 operations per cell against 2,633
+// that of the transforms (4 operations a line each way): about 880 operations per cell against 2,633
 // for sweeps through the Gauss points, with half their rounding error (the first and second
 // differences of the nodal values are formed directly). The FP32 product at 128^3 takes 229 us, at
 // 64^3 37 us (320 and 50 us through the Gauss points: gather and atomic adds bound it now), the FP64
@@ -95,7 +95,9 @@ __host__ __device__ constexpr double mode_diag(int c, int i, int j, int k) {
            (c == 2 ? 2.0 : 1.0) * mode_mass(i) * mode_mass(j) * mode_stiff(k);
 }
 
-// Nodal values <-> modes along AX, in place: to_modes x <- (w, d, e), from_modes its transpose.
+// Nodal values <-> modes along AX, in place: to_modes x <- (w, d, e), from_modes its transpose, which
+// takes e twice (rows of the tables carry the factor 2 per index E, mode_out: w + e/2 and 4 w - e are
+// one multiply-add each).
 template <int AX, typename T>
 __host__ __device__ __forceinline__ void to_modes(T* x) {
 #pragma unroll
@@ -116,9 +118,9 @@ __host__ __device__ __forceinline__ void from_modes(T* x) {
 #pragma unroll
         for (int o1 = 0; o1 < 3; ++o1) {
             const T w = x[lin<AX>(MODE_W, o1, o2)], d = x[lin<AX>(MODE_D, o1, o2)], e = x[lin<AX>(MODE_E, o1, o2)];
-            const T t = w + e;
+            const T t = w + T(0.5) * e;
             x[lin<AX>(0, o1, o2)] = t - d;
-            x[lin<AX>(1, o1, o2)] = T(4) * w - T(2) * e;
+            x[lin<AX>(1, o1, o2)] = T(4) * w - e;
             x[lin<AX>(2, o1, o2)] = t + d;
         }
 }
@@ -126,6 +128,10 @@ template <typename T>
 __host__ __device__ __forceinline__ void to_modes3(T* x) { to_modes<0>(x); to_modes<1>(x); to_modes<2>(x); }
 template <typename T>
 __host__ __device__ __forceinline__ void from_modes3(T* x) { from_modes<2>(x); from_modes<1>(x); from_modes<0>(x); }
+
+__host__ __device__ constexpr double mode_out(int i, int j, int k) {
+    return (i == 2 ? 2.0 : 1.0) * (j == 2 ? 2.0 : 1.0) * (k == 2 ? 2.0 : 1.0);
+}
 
 // Contribution of column component D to mode (i,j,k) of row component C (C != D):
 // int d_C u_D d_D v_C couples v's mode a along C with u's a + 1, and v's b along D with u's b - 1.
@@ -142,7 +148,7 @@ __host__ __device__ constexpr double mode_cross(int i, int j, int k) {
     return mode_grad(m[C]) * mode_grad(m[D] - 1) * mode_mass(m[3 - C - D]);
 }
 
-// Modes of row component C of the velocity operator: w = (A U)_C without the factor mu h, U1 and U2
+// Modes of row component C of the velocity operator (times mode_out): w = (A U)_C without mu h, U1 and U2
 // the modes of components (C + 1) % 3 and (C + 2) % 3.
 template <int C, typename T>
 __host__ __device__ __forceinline__ void modes_A(const T* U, const T* U1, const T* U2, T* w) {
@@ -155,10 +161,10 @@ __host__ __device__ __forceinline__ void modes_A(const T* U, const T* U1, const 
             for (int i = 0; i < 3; ++i) {
                 const int m = i + 3 * j + 9 * k;
                 T v = T(0);
-                if (m != 0) v = T(mode_diag(C, i, j, k)) * U[m];
+                if (m != 0) v = T(mode_diag(C, i, j, k) * mode_out(i, j, k)) * U[m];
                 const int p1 = mode_partner<C, D1>(i, j, k), p2 = mode_partner<C, D2>(i, j, k);
-                if (p1 >= 0) v += T(mode_cross<C, D1>(i, j, k)) * U1[p1 < 0 ? 0 : p1];
-                if (p2 >= 0) v += T(mode_cross<C, D2>(i, j, k)) * U2[p2 < 0 ? 0 : p2];
+                if (p1 >= 0) v += T(mode_cross<C, D1>(i, j, k) * mode_out(i, j, k)) * U1[p1 < 0 ? 0 : p1];
+                if (p2 >= 0) v += T(mode_cross<C, D2>(i, j, k) * mode_out(i, j, k)) * U2[p2 < 0 ? 0 : p2];
                 w[m] = v;
             }
 }
@@ -226,7 +232,7 @@ __host__ __device__ __forceinline__ void modes_BT(const T (&P)[8], T* w) {
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
                 const int q = mode_pressure<C>(i, j, k);
-                if (q >= 0) w[i + 3 * j + 9 * k] += T(mode_moment<C>(i, j, k)) * P[q < 0 ? 0 : q];
+                if (q >= 0) w[i + 3 * j + 9 * k] += T(mode_moment<C>(i, j, k) * mode_out(i, j, k)) * P[q < 0 ? 0 : q];
             }
 }
 template <int C, typename T>
