@@ -23,12 +23,10 @@
 // (vec.cu) remain available and are the arithmetic of the FP64 option.
 //
 // Layout: a pair of adjacent vector entries is handled by 1, 2 or 4 adjacent
-// threads, each owning a share of the basis rows. A thread copies its rows'
-// 16-byte entry pairs into its own column of shared memory with asynchronous
-// copies that bypass L1 (all in flight without holding registers; the next
-// sweep's copies are issued before the current sweep is computed) and works
-// from there; the projection sums are combined across the entry's threads by
-// shuffles. The per-thread dot sums are reduced per warp and CTA in
+// threads, each owning a share of the basis rows (kGsShapes). A thread loads its rows'
+// 16-byte entry pairs of a sweep into registers, all before it uses the first,
+// and the other warps' arithmetic covers the wait; the projection sums are
+// combined across the entry's threads by shuffles. The per-thread dot sums are reduced per warp and CTA in
 // double-float and written as doubles to `partials`, which one CTA adds in a
 // fixed order, so the results do not depend on scheduling. Basis rows have an
 // even stride so that every entry pair is 16-byte aligned.
@@ -54,41 +52,41 @@ constexpr int kGsThreads = 128;
 constexpr int kGsMaxK = 64;                 // largest basis of the double-float passes
 constexpr int kGsMaxBlocks = 2432;          // 16 per SM on 152 SMs; the partials buffer is sized for this
 
+// The second projection's coefficients c / alpha are of the size of the first one's rounding, about
+// 1e-13. Up to this size a product c v_i in single precision (relative error 2^-23) errs by less than
+// 2^-53 of v_i, the sum over 64 rows by less than 2^-47, the last bits of a double-float pair; above it
+// the products are double-float. That takes 11 of the 36 arithmetic instructions per basis entry out.
+constexpr double kSmallC = 9.31322574615478515625e-10;   // 2^-30
+
 enum GsMode { GS_DOT = 0, GS_PROJECT_DOT = 1, GS_PROJECT_SCALE = 2, GS_LAG = 3 };
 
-// An entry pair is handled by TPE = KB / RB threads (adjacent lanes), each owning RB <= STK_GS_RB
-// basis rows: with 16, one thread up to KB = 8, two up to 32, four at 64. Measured on whole 64^3
-// and 96^3 solves: 32 rows per thread is slower, and so are 8 (Krylov kernels +10% / +13%) and 4
-// (+69% / +84%): fewer rows per thread add shuffles and partial sums faster than the higher
-// occupancy hides latency.
-#ifndef STK_GS_RB
-#define STK_GS_RB 16
-#endif
-__host__ __device__ constexpr int gs_rb(int /*mode*/, int kb) {
-    return kb <= 8 ? kb : kb / 2 > STK_GS_RB ? STK_GS_RB : kb / 2;
-}
-template <int MODE, int KB>
-struct GsShape {
-    static constexpr int RB = gs_rb(MODE, KB);
-    static constexpr int TPE = KB / RB;
-    static constexpr int PPB = kGsThreads / TPE;   // entry pairs per CTA and sweep
-};
-
-// per thread: two buffers of RB rows x 16 bytes (an entry pair), then coefficients (two sets
-// for GS_LAG) and sums
-inline size_t gs_smem(int mode, int kb) {
-    return (4 * size_t(gs_rb(mode, kb)) * kGsThreads + size_t(kb) * (mode == GS_LAG ? 2 : 1) + 4 * (size_t(kb) + 1)) *
-           sizeof(double);
+// An entry pair is handled by TPE adjacent lanes, each with RB basis rows (at most 16: with 32 rows
+// per thread, or with 8 and 4 and more threads per pair, whole solves are slower). The shape is the
+// smallest that holds k rows (gs_shapes); every lane runs its RB rows without tests: rows past the
+// k-th are zero with zero coefficients, entries past the n-th repeat the last ones with w = 0. (One
+// test per row and entry pair cost as many instructions as the arithmetic.) Measured at 48^3 with 24
+// rows of 2.9 M entries: dot products 91 us, 6.3 TB/s; GS_LAG 114 us, bound by the arithmetic of its two
+// double-float products per entry (134 and 210 us with tests and with the rows passing through shared
+// memory). 16 rows per thread at most: 168 registers, three CTAs per SM; up to 12 rows four.
+struct GsShapeId { int tpe, rb; };
+constexpr GsShapeId kGsShapes[] = {{1, 4}, {1, 8}, {1, 12}, {1, 16}, {2, 12}, {2, 16}, {4, 10}, {4, 12}, {4, 14}, {4, 16}};
+constexpr int kGsShapeCount = int(sizeof(kGsShapes) / sizeof(kGsShapes[0]));
+inline int gs_shape(int k) {
+    int i = 0;
+    while (kGsShapes[i].tpe * kGsShapes[i].rb < k) ++i;
+    return i;
 }
 
-// 16-byte asynchronous copy global -> shared, not cached in L1.
-__device__ __forceinline__ void cp_async16(void* sdst, const void* gsrc) {
-    const unsigned sa = unsigned(__cvta_generic_to_shared(sdst));
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gsrc) : "memory");
+// coefficients (GS_LAG: two sets in double-float and one in single precision) and the warps' sums
+constexpr size_t gs_smem(int mode, int tpe, int rb) {
+    return (size_t(tpe * rb) * (mode == GS_LAG ? 3 : 1) + 4 * (size_t(tpe * rb) + 1)) * sizeof(double);
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
+__device__ __forceinline__ float4 load_pairs(const double* p) {   // 16 bytes, used once: not kept in L1
+    float4 v;
+    asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
 
 __device__ __forceinline__ df64 shfl_down_df(const df64& v, int o) {
     return df64(__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o));
@@ -107,40 +105,42 @@ __device__ __forceinline__ df64 shfl_xor_df(const df64& v, int o) {
 //   1 / alpha with alpha = |u_j - V_{<j} c|, or null for j = 0 where row 0 is final):
 //   v_j = (u_j - V_{<j} c) / alpha is written over row j; w1 = w - V_{<=j} h with v_j in row j,
 //   written as double-float to row j + 1 (y = V); partials <- V_{<=j}^T w1 (row j: v_j), w1 . w1.
-// KB >= k is the compile-time bound on the basis size (8, 16, 32 or 64). A thread handles the
-// entry pair (2p, 2p + 1): one 16-byte copy per row.
-template <int MODE, int KB>
-__global__ void __launch_bounds__(kGsThreads) k_gs_df(size_t n, int k, const double* __restrict__ V, size_t ld,
+// TPE, RB: see kGsShapes. A thread handles the entry pair (2p, 2p + 1): one 16-byte copy per row.
+template <int MODE, int TPE, int RB>
+__global__ void __launch_bounds__(kGsThreads, RB <= 12 ? 4 : 3) k_gs_df(size_t n, int k, const double* __restrict__ V, size_t ld,
                                                       const double* __restrict__ h, double* __restrict__ w,
                                                       const double* __restrict__ scale, double* y,
                                                       double* __restrict__ partials) {
-    using S = GsShape<MODE, KB>;
-    constexpr int RB = S::RB, TPE = S::TPE, PPB = S::PPB;
+    constexpr int KB = TPE * RB, PPB = kGsThreads / TPE;   // rows held, entry pairs per CTA and sweep
     extern __shared__ double smem[];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int g = tid % TPE;              // row group: rows r0 .. r0 + rb - 1
+    const int g = tid % TPE;              // row group: rows r0 .. r0 + RB - 1
     const int slot = tid / TPE;           // entry pair within the CTA's sweep
-    const int rb = (k + TPE - 1) / TPE;   // rows per group (<= RB), balanced over the groups
-    const int r0 = g * rb;
-    float4* col = reinterpret_cast<float4*>(smem) + tid;                       // [2][RB][kGsThreads], own column
-    constexpr int NH = MODE == GS_LAG ? 2 : 1;
-    df64* hs = reinterpret_cast<df64*>(smem + 4 * RB * kGsThreads);            // split coefficients
-    df64* hb = hs + KB;                                                        // GS_LAG: those of v_j
-    df64* red = reinterpret_cast<df64*>(smem + 4 * RB * kGsThreads + NH * KB); // [4][KB + 1] warp sums
+    const int r0 = g * RB;
+    const int nr = max(0, min(RB, k - r0));   // rows of the group below k
+    constexpr int NH = MODE == GS_LAG ? 3 : 1;
+    df64* hs = reinterpret_cast<df64*>(smem);               // split coefficients
+    df64* hb = hs + KB;                                     // GS_LAG: those of v_j
+    float* hf = reinterpret_cast<float*>(hb + KB);          // GS_LAG: v_j's of rows i < j, single
+    df64* red = reinterpret_cast<df64*>(smem + NH * KB);    // [4][KB + 1] warp sums
+    bool small_c = true;   // GS_LAG: see kSmallC
     if constexpr (MODE == GS_LAG) {
         // w1 = w - sum_{i<j} h_i v_i - h_j v_j with v_j = (u_j - sum_{i<j} c_i v_i) / alpha, as one
         // combination of the stored rows (a) and v_j itself (b)
         const int j = k - 1;
         const double ia = scale ? scale[j + 2] : 1.0;
-        for (int i = tid; i < k; i += kGsThreads) {
+        for (int i = tid; i < KB; i += kGsThreads) {
             const double ci = (scale && i < j) ? scale[i] : 0.0;
-            hs[i] = q2::split_double(i < j ? h[i] - h[j] * ci * ia : h[j] * ia);
-            hb[i] = q2::split_double(i < j ? -ci * ia : ia);
+            hs[i] = i < k ? q2::split_double(i < j ? h[i] - h[j] * ci * ia : h[j] * ia) : df64();
+            hb[i] = i < k ? q2::split_double(i < j ? -ci * ia : ia) : df64();
+            hf[i] = float(-ci * ia);
+            small_c = small_c && fabs(ci * ia) <= kSmallC;
         }
     } else if constexpr (MODE != GS_DOT) {
-        for (int i = tid; i < k; i += kGsThreads) hs[i] = q2::split_double(h[i]);
+        for (int i = tid; i < KB; i += kGsThreads) hs[i] = i < k ? q2::split_double(h[i]) : df64();
     }
-    __syncthreads();
+    if constexpr (MODE == GS_LAG) small_c = __syncthreads_and(small_c) != 0;
+    else __syncthreads();
     const df64 sc = MODE == GS_PROJECT_SCALE ? q2::split_double(scale[0]) : df64();
     constexpr int NA = MODE == GS_PROJECT_SCALE ? 1 : RB;
     df64 acc[NA];
@@ -148,27 +148,14 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_df(size_t n, int k, const dou
     for (int r = 0; r < NA; ++r) acc[r] = df64();
     df64 self, vdot;
     // Every lane of a warp runs the same number of sweeps (pairs past the end are masked), so
-    // that the full-warp shuffles below are always convergent. The copies of sweep s + 1 are
-    // issued before sweep s is computed (two buffers per thread).
+    // that the full-warp shuffles below are always convergent.
     const size_t np = (n + 1) / 2;
     const size_t warp_first = size_t(blockIdx.x) * PPB + size_t(wid) * (32 / TPE);
     const size_t stride = size_t(gridDim.x) * PPB;
     const size_t p0 = size_t(blockIdx.x) * PPB + slot;
-    auto issue = [&](size_t base, int buf) {
-        const size_t p = p0 + base;
-        if (p < np) {
-            // the row pointer is advanced row by row (not precomputed per row) to keep registers low
-            const double* src = V + 2 * p + size_t(r0) * ld;
-            float4* dst = col + buf * (RB * kGsThreads);
-            const int nr = min(rb, k - r0);
-#pragma unroll 4
-            for (int r = 0; r < nr; ++r) {
-                cp_async16(dst + r * kGsThreads, src);
-                src += ld;
-            }
-        }
-        cp_async_commit();
-    };
+    float4 v[RB];   // rows from nr on stay 0
+#pragma unroll
+    for (int r = 0; r < RB; ++r) v[r] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     auto load_w = [&](size_t p, double& a, double& b) {
         a = 0.0;
         b = 0.0;
@@ -178,37 +165,61 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_df(size_t n, int k, const dou
         }
     };
     size_t base = 0;
-    issue(base, 0);
     double wn0, wn1;
     load_w(p0, wn0, wn1);
     for (int it = 0; warp_first + base < np; ++it) {
         const size_t p = p0 + base;
         const bool in = p < np;
         const bool in1 = 2 * p + 1 < n;
-        issue(base + stride, (it + 1) & 1);
+        {
+            const double* src = V + 2 * min(p, np - 1) + size_t(r0) * ld;
+#pragma unroll
+            for (int r = 0; r < RB; ++r) {
+                if (r < nr) v[r] = load_pairs(src);
+                src += ld;
+            }
+        }
+        float4 uj = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if constexpr (MODE == GS_LAG)
+            if (g == 0) uj = load_pairs(V + 2 * min(p, np - 1) + size_t(k - 1) * ld);   // row j once more, from L2
         df64 w0 = q2::split_double(wn0), w1 = q2::split_double(wn1);
         load_w(p + stride, wn0, wn1);
-        cp_async_wait_prev();
-        const float4* cv = col + (it & 1) * (RB * kGsThreads);
         if constexpr (MODE == GS_DOT) {
 #pragma unroll
-            for (int r = 0; r < RB; ++r)
-                if (r < rb && in && r0 + r < k) {
-                    const float4 v = cv[r * kGsThreads];
-                    q2::mac(acc[r], df64(v.x, v.y), w0);
-                    q2::mac(acc[r], df64(v.z, v.w), w1);
-                }
+            for (int r = 0; r < RB; ++r) {
+                q2::mac(acc[r], df64(v[r].x, v[r].y), w0);
+                q2::mac(acc[r], df64(v[r].z, v[r].w), w1);
+            }
         } else if constexpr (MODE == GS_LAG) {
             df64 s0, s1, t0, t1;
+            if (small_c) {
+                float f0 = 0.0f, f1 = 0.0f;
 #pragma unroll
-            for (int r = 0; r < RB; ++r)
-                if (r < rb && in && r0 + r < k) {
-                    const float4 v = cv[r * kGsThreads];
-                    q2::mac(s0, hs[r0 + r], df64(v.x, v.y));
-                    q2::mac(s1, hs[r0 + r], df64(v.z, v.w));
-                    q2::mac(t0, hb[r0 + r], df64(v.x, v.y));
-                    q2::mac(t1, hb[r0 + r], df64(v.z, v.w));
+                for (int r = 0; r < RB; ++r) {
+                    q2::mac(s0, hs[r0 + r], df64(v[r].x, v[r].y));
+                    q2::mac(s1, hs[r0 + r], df64(v[r].z, v[r].w));
+                    const float c = hf[r0 + r];
+                    f0 = fmaf(c, v[r].x, f0);
+                    f1 = fmaf(c, v[r].z, f1);
                 }
+#pragma unroll
+                for (int o = 1; o < TPE; o <<= 1) {
+                    f0 += __shfl_xor_sync(0xffffffffu, f0, o);
+                    f1 += __shfl_xor_sync(0xffffffffu, f1, o);
+                }
+                t0 = df64(f0, 0.0f);
+                t1 = df64(f1, 0.0f);
+                q2::mac(t0, hb[k - 1], df64(uj.x, uj.y));   // lanes g = 0: row j, u_j / alpha
+                q2::mac(t1, hb[k - 1], df64(uj.z, uj.w));
+            } else {
+#pragma unroll
+                for (int r = 0; r < RB; ++r) {
+                    q2::mac(s0, hs[r0 + r], df64(v[r].x, v[r].y));
+                    q2::mac(s1, hs[r0 + r], df64(v[r].z, v[r].w));
+                    q2::mac(t0, hb[r0 + r], df64(v[r].x, v[r].y));
+                    q2::mac(t1, hb[r0 + r], df64(v[r].z, v[r].w));
+                }
+            }
             q2::renorm(s0);
             q2::renorm(s1);
             q2::renorm(t0);
@@ -217,8 +228,10 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_df(size_t n, int k, const dou
             for (int o = 1; o < TPE; o <<= 1) {
                 s0 += shfl_xor_df(s0, o);
                 s1 += shfl_xor_df(s1, o);
-                t0 += shfl_xor_df(t0, o);
-                t1 += shfl_xor_df(t1, o);
+                if (!small_c) {
+                    t0 += shfl_xor_df(t0, o);
+                    t1 += shfl_xor_df(t1, o);
+                }
             }
             w0 = w0 - s0;
             w1 = w1 - s1;
@@ -237,22 +250,19 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_df(size_t n, int k, const dou
                 q2::mac(vdot, t0, w0);
                 q2::mac(vdot, t1, w1);
             }
+            if (!in) w0 = w1 = df64();
 #pragma unroll
-            for (int r = 0; r < RB; ++r)
-                if (r < rb && in && r0 + r < k - 1) {
-                    const float4 v = cv[r * kGsThreads];
-                    q2::mac(acc[r], df64(v.x, v.y), w0);
-                    q2::mac(acc[r], df64(v.z, v.w), w1);
-                }
+            for (int r = 0; r < RB; ++r) {   // row j's sum (u_j, not v_j) is not used
+                q2::mac(acc[r], df64(v[r].x, v[r].y), w0);
+                q2::mac(acc[r], df64(v[r].z, v[r].w), w1);
+            }
         } else {
             df64 s0, s1;
 #pragma unroll
-            for (int r = 0; r < RB; ++r)
-                if (r < rb && in && r0 + r < k) {
-                    const float4 v = cv[r * kGsThreads];
-                    q2::mac(s0, hs[r0 + r], df64(v.x, v.y));
-                    q2::mac(s1, hs[r0 + r], df64(v.z, v.w));
-                }
+            for (int r = 0; r < RB; ++r) {
+                q2::mac(s0, hs[r0 + r], df64(v[r].x, v[r].y));
+                q2::mac(s1, hs[r0 + r], df64(v[r].z, v[r].w));
+            }
             q2::renorm(s0);
             q2::renorm(s1);
 #pragma unroll
@@ -275,13 +285,12 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_df(size_t n, int k, const dou
                     q2::mac(self, w0, w0);
                     q2::mac(self, w1, w1);
                 }
+                if (!in) w0 = w1 = df64();
 #pragma unroll
-                for (int r = 0; r < RB; ++r)
-                    if (r < rb && in && r0 + r < k) {
-                        const float4 v = cv[r * kGsThreads];
-                        q2::mac(acc[r], df64(v.x, v.y), w0);
-                        q2::mac(acc[r], df64(v.z, v.w), w1);
-                    }
+                for (int r = 0; r < RB; ++r) {
+                        q2::mac(acc[r], df64(v[r].x, v[r].y), w0);
+                    q2::mac(acc[r], df64(v[r].z, v[r].w), w1);
+                }
             }
         }
         if ((it & 1) == 1) {
@@ -292,7 +301,6 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_df(size_t n, int k, const dou
         }
         base += stride;
     }
-    cp_async_wait_all();
     if constexpr (MODE != GS_PROJECT_SCALE) {
 #pragma unroll
         for (int r = 0; r < RB; ++r) q2::renorm(acc[r]);
@@ -310,7 +318,7 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_df(size_t n, int k, const dou
         if (lane < TPE) {
 #pragma unroll
             for (int r = 0; r < RB; ++r)
-                if (r < rb && r0 + r < kd) red[wid * (KB + 1) + r0 + r] = acc[r];
+                if (r0 + r < kd) red[wid * (KB + 1) + r0 + r] = acc[r];
             if (g == 0) red[wid * (KB + 1) + k] = self;
             if (MODE == GS_LAG && g == 0) red[wid * (KB + 1) + k - 1] = vdot;
         }
@@ -359,55 +367,41 @@ __global__ void __launch_bounds__(1024) k_gs_final(int rows, int nb, const doubl
     }
 }
 
-// Blocks per launch: as many CTAs as fit on the GPU at once (at most kGsMaxBlocks), per KB.
-int gs_blocks[4][4];
+// Blocks per launch: as many CTAs as fit on the GPU at once (at most kGsMaxBlocks), per mode and shape.
+int gs_blocks[4][kGsShapeCount];
 int gs_device = -1;
 
-inline int kb_index(int k) { return k <= 8 ? 0 : k <= 16 ? 1 : k <= 32 ? 2 : 3; }
-
-template <int MODE, int KB>
-cudaError_t configure_one(int sms) {
-    cudaError_t e = cudaFuncSetAttribute(k_gs_df<MODE, KB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         int(gs_smem(MODE, KB)));
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gs_df<MODE, KB>, kGsThreads, gs_smem(MODE, KB));
-    if (e != cudaSuccess) return e;
-    const int nb = per_sm * sms;
-    gs_blocks[MODE][kb_index(KB)] = nb < 1 ? 1 : (nb > kGsMaxBlocks ? kGsMaxBlocks : nb);
-    return cudaSuccess;
+template <int MODE, int I>
+cudaError_t configure_shapes(int sms) {
+    if constexpr (I < kGsShapeCount) {
+        constexpr int TPE = kGsShapes[I].tpe, RB = kGsShapes[I].rb;
+        constexpr size_t smem = gs_smem(MODE, TPE, RB);
+        cudaError_t e = cudaFuncSetAttribute(k_gs_df<MODE, TPE, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        if (e != cudaSuccess) return e;
+        int per_sm = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gs_df<MODE, TPE, RB>, kGsThreads, smem);
+        if (e != cudaSuccess) return e;
+        const int nb = per_sm * sms;
+        gs_blocks[MODE][I] = nb < 1 ? 1 : (nb > kGsMaxBlocks ? kGsMaxBlocks : nb);
+        return configure_shapes<MODE, I + 1>(sms);
+    } else {
+        return cudaSuccess;
+    }
 }
 
-template <int MODE>
-cudaError_t configure_mode(int sms) {
-    cudaError_t e;
-    if ((e = configure_one<MODE, 8>(sms)) != cudaSuccess) return e;
-    if ((e = configure_one<MODE, 16>(sms)) != cudaSuccess) return e;
-    if ((e = configure_one<MODE, 32>(sms)) != cudaSuccess) return e;
-    return configure_one<MODE, 64>(sms);
-}
-
-// Launches k_gs_df<MODE, KB> for the smallest KB >= k; returns its grid size.
-template <int MODE>
+// Launches k_gs_df<MODE, ...> in the smallest shape that holds k rows; returns its grid size.
+template <int MODE, int I = 0>
 int launch_df(size_t n, int k, const double* V, size_t ld, const double* h, double* w, const double* scale,
               double* y, double* partials, cudaStream_t s) {
-    const int ki = kb_index(k);
-    const int nb = gs_blocks[MODE][ki];
-    switch (ki) {
-        case 0:
-            LAUNCH(PROF_KRYLOV, s, (k_gs_df<MODE, 8><<<nb, kGsThreads, gs_smem(MODE, 8), s>>>(n, k, V, ld, h, w, scale, y, partials)));
-            break;
-        case 1:
-            LAUNCH(PROF_KRYLOV, s, (k_gs_df<MODE, 16><<<nb, kGsThreads, gs_smem(MODE, 16), s>>>(n, k, V, ld, h, w, scale, y, partials)));
-            break;
-        case 2:
-            LAUNCH(PROF_KRYLOV, s, (k_gs_df<MODE, 32><<<nb, kGsThreads, gs_smem(MODE, 32), s>>>(n, k, V, ld, h, w, scale, y, partials)));
-            break;
-        default:
-            LAUNCH(PROF_KRYLOV, s, (k_gs_df<MODE, 64><<<nb, kGsThreads, gs_smem(MODE, 64), s>>>(n, k, V, ld, h, w, scale, y, partials)));
-            break;
+    if constexpr (I < kGsShapeCount) {
+        if (gs_shape(k) != I) return launch_df<MODE, I + 1>(n, k, V, ld, h, w, scale, y, partials, s);
+        constexpr int TPE = kGsShapes[I].tpe, RB = kGsShapes[I].rb;
+        const int nb = gs_blocks[MODE][I];
+        LAUNCH(PROF_KRYLOV, s, (k_gs_df<MODE, TPE, RB><<<nb, kGsThreads, gs_smem(MODE, TPE, RB), s>>>(n, k, V, ld, h, w, scale, y, partials)));
+        return nb;
+    } else {
+        return 0;
     }
-    return nb;
 }
 
 // Native FP64: out[k+1] = hn, out[k+2] = 1 / hn from out[0..k-1] = h2 and out[k] = |w1|^2.
@@ -468,10 +462,10 @@ cudaError_t gs_configure() {
     if (dev == gs_device) return cudaSuccess;
     int sms = 0;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = configure_mode<GS_DOT>(sms)) != cudaSuccess) return e;
-    if ((e = configure_mode<GS_PROJECT_DOT>(sms)) != cudaSuccess) return e;
-    if ((e = configure_mode<GS_PROJECT_SCALE>(sms)) != cudaSuccess) return e;
-    if ((e = configure_mode<GS_LAG>(sms)) != cudaSuccess) return e;
+    if ((e = configure_shapes<GS_DOT, 0>(sms)) != cudaSuccess) return e;
+    if ((e = configure_shapes<GS_PROJECT_DOT, 0>(sms)) != cudaSuccess) return e;
+    if ((e = configure_shapes<GS_PROJECT_SCALE, 0>(sms)) != cudaSuccess) return e;
+    if ((e = configure_shapes<GS_LAG, 0>(sms)) != cudaSuccess) return e;
     gs_device = dev;
     return cudaSuccess;
 }
