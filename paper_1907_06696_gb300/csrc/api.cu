@@ -190,7 +190,6 @@ struct stokes_ctx {
     double* mp_scale = nullptr;                 // h^3 / mu per finest cell
     // preconditioner / operator work (N_u)
     double* tu = nullptr;
-    float *stage_in = nullptr, *stage_out = nullptr;   // FP32 V-cycle input / output
     // coarse level
     int nf = 0;
     int* free_idx = nullptr;
@@ -699,8 +698,7 @@ stokes_status apply_stokes(stokes_ctx* c, const double* src, double* dst, cudaSt
         return STOKES_OK;
     }
     if (native) prof_override(PROF_RESID_F64);
-    const cudaError_t e = launch_stokes_blocks(F.g, F.v64.mu, src, src + F.g.n_u, dst, dst + F.g.n_u, true, true,
-                                               true, c->opt.outer_arith >= 1 && !native, s);
+    const cudaError_t e = launch_stokes_blocks(F.g, F.v64.mu, src, src + F.g.n_u, dst, dst + F.g.n_u, true, true, true, s);
     prof_override(-1);
     CK(e);
     return STOKES_OK;
@@ -713,38 +711,48 @@ stokes_status apply_stokes(stokes_ctx* c, const double* src, double* dst, cudaSt
 // with the recursion in between.
 enum PrecPart { PREC_ALL = 0, PREC_PRE = 1, PREC_POST = 2 };
 
+// The V-cycle's right-hand side into the finest level, r_u - B^T z_p or (P_D) r_u; its boundary
+// entries are 0 there and stay 0.
+template <typename T>
+stokes_status precondition_head(stokes_ctx* c, const double* r, double* z, cudaStream_t s) {
+    Level& F = c->lev[c->L - 1];
+    const size_t nu = F.g.n_u;
+    double* zp = z + nu;
+    CKS(schur_inverse(c, r + nu, zp, s));
+    if (c->opt.precond_kind != 1) {
+        CK(launch_axpby(F.g.n_p, -1.0, zp, 0.0, zp, s));                      // z_p = -S^-1 r_p
+        CK(launch_bt_resid<T>(F.g, zp, r, vecs<T>(F).b, s));
+        return STOKES_OK;
+    }   // else P_D: z_p = S_hat^-1 r_p, z_u = A_hat^-1 r_u
+    if constexpr (sizeof(T) == 4) CK(launch_cast_d2f(nu, r, F.v32.b, s));
+    else CK(cudaMemcpyAsync(F.v64.b, r, nu * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    CK(launch_zero_boundary<T>(F.g, vecs<T>(F).b, s));
+    return STOKES_OK;
+}
+
+// z_u from the finest level's result; boundary rows are the identity.
+template <typename T>
+stokes_status precondition_tail(stokes_ctx* c, const double* r, double* z, cudaStream_t s) {
+    Level& F = c->lev[c->L - 1];
+    if constexpr (sizeof(T) == 4) CK(launch_cast_f2d(F.g.n_u, F.v32.x, z, s));
+    else CK(cudaMemcpyAsync(z, F.v64.x, F.g.n_u * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    CK(launch_copy_boundary<double>(F.g, r, z, s));
+    return STOKES_OK;
+}
+
+template <typename T>
+stokes_status precondition_uniform(stokes_ctx* c, const double* r, double* z, cudaStream_t s, int part) {
+    if (part != PREC_POST) CKS(precondition_head<T>(c, r, z, s));
+    if (part == PREC_ALL) CKS(run_levels<T>(c, s));
+    if (part != PREC_PRE) CKS(precondition_tail<T>(c, r, z, s));
+    return STOKES_OK;
+}
+
 stokes_status precondition(stokes_ctx* c, int prec, const double* r, double* z, cudaStream_t s,
                            int part = PREC_ALL) {
     if (c->oct) return oct_precondition(c, prec, r, z, s);
-    Level& F = c->lev[c->L - 1];
-    const size_t nu = F.g.n_u, np = F.g.n_p;
-    double* zp = z + nu;
-    const double* rin = c->opt.precond_kind == 1 ? r : c->tu;   // the V-cycle's right-hand side
-    if (part == PREC_POST) {   // the tail of vcycle<float>, then back to FP64
-        CK(cudaMemcpyAsync(c->stage_out, F.v32.x, nu * sizeof(float), cudaMemcpyDeviceToDevice, s));
-        CK(launch_copy_boundary<float>(F.g, c->stage_in, c->stage_out, s));
-        CK(launch_cast_f2d(nu, c->stage_out, z, s));
-        CK(launch_copy_boundary<double>(F.g, rin, z, s));
-        return STOKES_OK;
-    }
-    CKS(schur_inverse(c, r + nu, zp, s));
-    if (c->opt.precond_kind != 1) {
-        CK(launch_axpby(np, -1.0, zp, 0.0, zp, s));                           // z_p = -S^-1 r_p
-        CK(launch_stokes_blocks(F.g, F.v64.mu, nullptr, zp, c->tu, nullptr, false, true, false,
-                                c->opt.outer_arith >= 1, s));
-        CK(launch_axpby(nu, 1.0, r, -1.0, c->tu, s));                        // t = r_u - B^T z_p
-    }   // else P_D: z_p = S_hat^-1 r_p, z_u = A_hat^-1 r_u
-    if (prec == STOKES_FP64) return vcycle<double>(c, rin, z, s);
-    CK(launch_cast_d2f(nu, rin, c->stage_in, s));
-    if (part == PREC_PRE) {    // the head of vcycle<float>
-        CK(cudaMemcpyAsync(F.v32.b, c->stage_in, nu * sizeof(float), cudaMemcpyDeviceToDevice, s));
-        CK(launch_zero_boundary<float>(F.g, F.v32.b, s));
-        return STOKES_OK;
-    }
-    CKS(vcycle<float>(c, c->stage_in, c->stage_out, s));
-    CK(launch_cast_f2d(nu, c->stage_out, z, s));
-    CK(launch_copy_boundary<double>(F.g, rin, z, s));
-    return STOKES_OK;
+    return prec == STOKES_FP64 ? precondition_uniform<double>(c, r, z, s, part)
+                               : precondition_uniform<float>(c, r, z, s, part);
 }
 
 stokes_status ensure_krylov(stokes_ctx* c) {
@@ -1808,8 +1816,6 @@ stokes_status setup_impl(const stokes_mesh* mesh, const stokes_mu* mu, const sto
     CKS(dalloc(c, &c->sp_d2, gf.n_p));
     CKS(dalloc(c, &c->mp_scale, gf.cells));
     CKS(dalloc(c, &c->tu, gf.n_u));
-    CKS(dalloc(c, &c->stage_in, gf.n_u));
-    CKS(dalloc(c, &c->stage_out, gf.n_u));
     CKS(dalloc(c, &c->partials, size_t(std::max(multidot_blocks(), gs_partials_blocks())) * (o.restart + 8)));
     CKS(dalloc(c, &c->dots, size_t(o.restart + 8)));
     CK(cudaMallocHost(&c->dots_host, size_t(3 * (o.restart + 8)) * sizeof(double)));
@@ -1917,6 +1923,9 @@ stokes_status setup_impl(const stokes_mesh* mesh, const stokes_mu* mu, const sto
             CK(cudaMemcpyAsync(c->Ainv, Ainv.data(), sizeof(double) * nf * nf, cudaMemcpyHostToDevice, s));
         }
     }
+    // the finest right-hand sides' boundary entries: the preconditioner writes the others only
+    CK(cudaMemsetAsync(c->lev[L - 1].v64.b, 0, gf.n_u * sizeof(double), s));
+    CK(cudaMemsetAsync(c->lev[L - 1].v32.b, 0, gf.n_u * sizeof(float), s));
     CK(cudaStreamSynchronize(s));
     return STOKES_OK;
 }
@@ -2481,10 +2490,10 @@ stokes_status stokes_vmult(stokes_ctx* c, int level, int block, int prec, const 
     double* dd = static_cast<double*>(dst);
     switch (block) {
         case STOKES_BLOCK_B:
-            CK(launch_stokes_blocks(Lv.g, Lv.v64.mu, sd, nullptr, nullptr, dd, false, false, true, c->opt.outer_arith >= 1, s));
+            CK(launch_stokes_blocks(Lv.g, Lv.v64.mu, sd, nullptr, nullptr, dd, false, false, true, s));
             return STOKES_OK;
         case STOKES_BLOCK_BT:
-            CK(launch_stokes_blocks(Lv.g, Lv.v64.mu, nullptr, sd, dd, nullptr, false, true, false, c->opt.outer_arith >= 1, s));
+            CK(launch_stokes_blocks(Lv.g, Lv.v64.mu, nullptr, sd, dd, nullptr, false, true, false, s));
             return STOKES_OK;
         case STOKES_BLOCK_MP:
             CK(launch_mass_p(Lv.g, Lv.v64.mu, sd, dd, s));

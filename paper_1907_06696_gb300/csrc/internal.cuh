@@ -35,10 +35,8 @@ inline LevelGeom make_geom(int n) {
 // Finest-level FP64 blocks. Flags select the parts of [[A, B^T], [B, 0]]:
 // the u-part of dst gets A u (DO_A) + B^T p (DO_BT), the p-part gets B u (DO_B).
 // src_u / src_p may be null when unused; dst parts are overwritten.
-// bt_df64: B^T alone may be formed in double-float (launch_bt_gather); every other block is to FP64 accuracy.
 cudaError_t launch_stokes_blocks(const LevelGeom& g, const double* mu, const double* src_u, const double* src_p,
-                                 double* dst_u, double* dst_p, bool do_a, bool do_bt, bool do_b, bool bt_df64,
-                                 cudaStream_t s);
+                                 double* dst_u, double* dst_p, bool do_a, bool do_bt, bool do_b, cudaStream_t s);
 // The same blocks added to dst in fixed point, one velocity component per thread (outer.cu); boundary
 // rows get nothing.
 cudaError_t launch_outer_fix(const LevelGeom& g, const double* mu, const double* src_u, const double* src_p,
@@ -54,8 +52,10 @@ cudaError_t launch_outer_tc(const LevelGeom& g, const double* mu, const double* 
                             unsigned long long wait_ns, cudaStream_t s);
 // dst = M_p src (weighted pressure mass, FP64).
 cudaError_t launch_mass_p(const LevelGeom& g, const double* mu, const double* src, double* dst, cudaStream_t s);
-// out = B^T p on the uniform mesh (velocity boundary nodes 0), gathered per node pair; no atomics
-cudaError_t launch_bt_gather(const LevelGeom& g, const double* p, double* out, cudaStream_t s);
+// out = r - B^T p on the uniform mesh's free nodes (boundary entries of out left as they are), gathered, no
+// atomics; T = float: the product in double-float, one rounding at the end.
+template <typename T>
+cudaError_t launch_bt_resid(const LevelGeom& g, const double* p, const double* r, T* out, cudaStream_t s);
 // scale[cell] = h^3 / mu[cell]
 cudaError_t launch_mass_scale(const LevelGeom& g, const double* mu, double* scale, cudaStream_t s);
 // One Chebyshev step of S_hat^-1 with M_p gathered per vertex (double-float products):

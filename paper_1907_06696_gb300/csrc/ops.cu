@@ -69,36 +69,71 @@ __global__ void k_mass_p(int n, double h, const double* __restrict__ mu, const d
     }
 }
 
-// ---- B^T on the uniform mesh as a gather (pressure.cuh). Block (line (J, K), component c):
-// threads 0..8 put the line's weights, thread e then t_e into shared memory; thread e writes the
-// x-nodes 2e and 2e + 1. No atomics.
-template <int C>
-__device__ __forceinline__ void bt_line(int n, double s, const double* __restrict__ p, double* __restrict__ out,
-                                        int J, int K, q2::df64* t, q2::df64* w) {
-    const int P = n + 1, M = 2 * n + 1;
-    const int e = int(threadIdx.x);
-    double* o = out + size_t(C) * size_t(M) * M * M + size_t(M) * (J + size_t(M) * K);
-    if (J == 0 || J == M - 1 || K == 0 || K == M - 1) {   // boundary rows
-        for (int i = e; i < M; i += int(blockDim.x)) o[i] = 0.0;
-        return;
-    }
-    if (e < 9) w[e] = bt_weight<C>(J, K, e);
-    __syncthreads();
-    if (e < P) t[e] = bt_t<C>(n, p, J, K, e, w);
-    __syncthreads();
-    if (e < P) bt_out<C>(n, s, o, e, t);
+// ---- B^T on the uniform mesh as a gather, one thread per cell (e, f, g) and its 8 nodes of lower or odd
+// index (pressure.cuh bt_nodes); nodes on the domain boundary are left as they are.
+// BT_PLAIN: out = B^T p;  BT_RESID: out = r - B^T p (the V-cycle's right-hand side), TO = double in FP64,
+// TO = float in double-float without an FP64 instruction, rounded once at the end.
+// Bound by memory (r read, out written) and, in FP64, by its ~3 FP64 instructions per node. At 64^3 the
+// fused FP32 right-hand side takes 38 us; one thread per vertex of a line and component, with the moments
+// as double-float weights, took 101 us for B^T p alone, 49 us for the FP64 block now.
+enum BtMode { BT_PLAIN = 0, BT_RESID = 1 };
+
+template <typename TO> struct BtArith;
+template <> struct BtArith<double> {
+    using type = double;
+    static __device__ __forceinline__ double in(double v) { return v; }
+    static __device__ __forceinline__ double out(double v) { return v; }
+};
+template <> struct BtArith<float> {
+    using type = q2::df64;
+    static __device__ __forceinline__ q2::df64 in(double v) { return q2::split_double(v); }
+    static __device__ __forceinline__ float out(const q2::df64& v) { return v.hi; }
+};
+
+template <int C, int MODE, typename TO>
+__device__ __forceinline__ void bt_store(const typename BtArith<TO>::type (&v)[3][3][3], double h, int e, int f, int g, int M,
+                                         const double* __restrict__ r, TO* __restrict__ out) {
+    using A = BtArith<TO>;
+    using T = typename A::type;
+    T b[8];
+    bt_nodes<C>(v, b);
+    const size_t base = size_t(C) * M * M * M + size_t(2 * e) + size_t(M) * (size_t(2 * f) + size_t(M) * size_t(2 * g));
+    const T even = A::in(-h * h * bt_factor<0>(0, 0, 0)), odd = A::in(-h * h * bt_factor<0>(1, 0, 0));
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                if ((i == 0 && e == 0) || (j == 0 && f == 0) || (k == 0 && g == 0)) continue;
+                const size_t at = base + size_t(i + M * (j + M * k));
+                const T y = b[i + 2 * j + 4 * k] * ((C == 0 ? i : (C == 1 ? j : k)) != 0 ? odd : even);
+                out[at] = A::out(MODE == BT_RESID ? A::in(r[at]) - y : y);
+            }
 }
 
-__global__ void k_bt_gather(int n, double h, const double* __restrict__ p, double* __restrict__ out) {
-    extern __shared__ __align__(16) unsigned char bt_smem[];
-    q2::df64* t = reinterpret_cast<q2::df64*>(bt_smem);   // n + 1 entries
-    q2::df64* w = t + (n + 1);                             // 9 entries
-    const int M = 2 * n + 1;
-    const int J = int(blockIdx.x % unsigned(M)), K = int(blockIdx.x / unsigned(M)), c = int(blockIdx.y);
-    const double s = -h * h;
-    if (c == 0) bt_line<0>(n, s, p, out, J, K, t, w);
-    else if (c == 1) bt_line<1>(n, s, p, out, J, K, t, w);
-    else bt_line<2>(n, s, p, out, J, K, t, w);
+template <int MODE, typename TO>
+__global__ void __launch_bounds__(128) k_bt(int n, double h, const double* __restrict__ p, const double* __restrict__ r,
+                                            TO* __restrict__ out) {
+    using A = BtArith<TO>;
+    const size_t cell = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (cell >= size_t(n) * n * n) return;
+    const int e = int(cell % n), f = int((cell / n) % n), g = int(cell / (size_t(n) * n));
+    const int P = n + 1, M = 2 * n + 1;
+    typename A::type v[3][3][3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                if ((i == 0) + (j == 0) + (k == 0) > 1) continue;   // not used by any component
+                const int a = max(e - 1 + i, 0), b = max(f - 1 + j, 0), c = max(g - 1 + k, 0);
+                v[k][j][i] = A::in(p[size_t(a) + size_t(P) * (b + size_t(P) * c)]);
+            }
+    bt_store<0, MODE, TO>(v, h, e, f, g, M, r, out);
+    bt_store<1, MODE, TO>(v, h, e, f, g, M, r, out);
+    bt_store<2, MODE, TO>(v, h, e, f, g, M, r, out);
 }
 
 // s_K = h^3 / mu_K per cell: the factor of the cell's pressure mass matrix (Section 2.2.2, the
@@ -299,12 +334,12 @@ template cudaError_t launch_zero_boundary<float>(const LevelGeom&, float*, cudaS
 template cudaError_t launch_zero_boundary<double>(const LevelGeom&, double*, cudaStream_t);
 
 cudaError_t launch_stokes_blocks(const LevelGeom& g, const double* mu, const double* src_u, const double* src_p,
-                                 double* dst_u, double* dst_p, bool do_a, bool do_bt, bool do_b, bool bt_df64,
-                                 cudaStream_t s) {
+                                 double* dst_u, double* dst_p, bool do_a, bool do_bt, bool do_b, cudaStream_t s) {
     cudaError_t e;
-    // B^T alone (the preconditioner's) in double-float: the gather writes every velocity entry, no
-    // clear needed; its blocks hold one thread per vertex of a line (n + 1 <= 1024)
-    if (bt_df64 && !do_a && do_bt && !do_b && g.n + 1 <= 1024) return launch_bt_gather(g, src_p, dst_u, s);
+    if (!do_a && do_bt && !do_b) {   // B^T alone: the gather, and the boundary rows
+        LAUNCH(PROF_BT_F64, s, (k_bt<BT_PLAIN, double><<<blocks_for(g.cells, 128), 128, 0, s>>>(g.n, g.h, src_p, nullptr, dst_u)));
+        return launch_zero_boundary<double>(g, dst_u, s);
+    }
     if (do_a || do_bt) {
         e = cudaMemsetAsync(dst_u, 0, g.n_u * sizeof(double), s);
         if (e != cudaSuccess) return e;
@@ -329,14 +364,13 @@ cudaError_t launch_mass_p(const LevelGeom& g, const double* mu, const double* sr
     return cudaGetLastError();
 }
 
-cudaError_t launch_bt_gather(const LevelGeom& g, const double* p, double* out, cudaStream_t s) {
-    // one block per (line, component), one thread per vertex of the line (x-nodes 2e, 2e + 1)
-    const unsigned threads = unsigned((g.n + 1 + 31) / 32 * 32);
-    const size_t smem = size_t(g.n + 1 + 9) * sizeof(q2::df64);
-    const dim3 grid(unsigned(size_t(g.M) * g.M), 3);
-    LAUNCH(PROF_BT_F64, s, k_bt_gather<<<grid, threads, smem, s>>>(g.n, g.h, p, out));
+template <typename T>
+cudaError_t launch_bt_resid(const LevelGeom& g, const double* p, const double* r, T* out, cudaStream_t s) {
+    LAUNCH(PROF_BT_F64, s, (k_bt<BT_RESID, T><<<blocks_for(g.cells, 128), 128, 0, s>>>(g.n, g.h, p, r, out)));
     return cudaGetLastError();
 }
+template cudaError_t launch_bt_resid<float>(const LevelGeom&, const double*, const double*, float*, cudaStream_t);
+template cudaError_t launch_bt_resid<double>(const LevelGeom&, const double*, const double*, double*, cudaStream_t);
 
 cudaError_t launch_mass_scale(const LevelGeom& g, const double* mu, double* scale, cudaStream_t s) {
     LAUNCH(PROF_MASS_P, s, k_mass_scale<<<blocks_for(g.cells, 256), 256, 0, s>>>(g.cells, g.h, mu, scale));

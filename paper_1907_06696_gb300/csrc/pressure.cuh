@@ -1,8 +1,8 @@
 // pressure.cuh -- per-thread bodies of the pressure-side gathers of the preconditioner on uniform
-// meshes (ops.cu kernels k_bt_gather and k_schur_cheb): B^T p as a tensor product of assembled 1D
+// meshes (ops.cu kernels k_bt and k_schur_cheb): B^T p as a tensor product of assembled 1D
 // moment operators (Section 2.1, definition of B), and one Jacobi-Chebyshev step of S_hat^-1 on
-// the 1/mu-weighted pressure mass matrix (Section 2.2.2) with M_p gathered per vertex. Both run
-// their products in double-float on the FP32 pipes. Plain functions of the thread's indices, so
+// the 1/mu-weighted pressure mass matrix (Section 2.2.2) with M_p gathered per vertex, its
+// products in double-float on the FP32 pipes. Plain functions of the thread's indices, so
 // that a host program can run them node by node and vertex by vertex.
 #pragma once
 
@@ -19,6 +19,47 @@ namespace stk {
 // (J, K) of component C: t_e = sum X_1[J][b] X_2[K][k] p(e, b, k), then the x-nodes 2e and 2e+1
 // from t_{e-1}, t_e, t_{e+1}; boundary nodes get 0, as in the cell kernels.
 
+// Evaluated, the rows are (1, 0, -1)/6 and (4, -4)/6 along axis c and (0, 2, 0)/6 and (2, 2)/6 along the
+// others: sums and differences of neighbouring vertices, one factor per node. bt_nodes forms the 8 nodes
+// (2e, 2e + 1) x (2f, 2f + 1) x (2g, 2g + 1) of component C from the 3 x 3 x 3 vertices around (e, f, g)
+// (v[k][j][i] at e - 1 + i, ...; nodes with an even index 0 are boundary nodes, whatever v holds
+// there): out[i + 2 j + 4 k] without the factor -h^2 bt_factor. 16 additions for 8 nodes.
+template <int C>
+__host__ __device__ constexpr double bt_factor(int i, int j, int k) {   // i, j, k: node parity (1: odd)
+    return ((C == 0 ? i : (C == 1 ? j : k)) != 0 ? 2.0 / 3.0 : 1.0 / 6.0) / 9.0;
+}
+template <int C, typename T>
+__host__ __device__ __forceinline__ void bt_nodes(const T (&v)[3][3][3], T (&out)[8]) {
+    auto at = [&v](int d, int a, int b) -> const T& {   // d along C, then the other two axes in order
+        return C == 0 ? v[1 + b][1 + a][1 + d] : (C == 1 ? v[1 + b][1 + d][1 + a] : v[1 + d][1 + b][1 + a]);
+    };
+    T x[2][2][2];   // [parity along C][a][b]
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            x[0][a][b] = at(-1, a, b) - at(1, a, b);
+            x[1][a][b] = at(0, a, b) - at(1, a, b);
+        }
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+#pragma unroll
+        for (int b = 0; b < 2; ++b) x[d][1][b] = x[d][0][b] + x[d][1][b];   // now parity along a
+#pragma unroll
+        for (int a = 0; a < 2; ++a) x[d][a][1] = x[d][a][0] + x[d][a][1];   // and along b
+    }
+#pragma unroll
+    for (int d = 0; d < 2; ++d)
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                const int i = C == 0 ? d : a, j = C == 0 ? a : (C == 1 ? d : b), k = C == 2 ? d : b;
+                out[i + 2 * j + 4 * k] = x[d][a][b];
+            }
+}
+
+// The same per x-line of nodes, with the moments as weights in double-float (host comparison).
 // entry of X_0 (axis 0) in row i at vertex a, for the rows of vertex e (i = 2e, 2e + 1)
 template <int C>
 __host__ __device__ __forceinline__ double bt_x_row(int i, int a, int e) {
