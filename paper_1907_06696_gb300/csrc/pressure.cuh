@@ -139,55 +139,69 @@ __host__ __device__ __forceinline__ void bt_out(int n, double s, double* __restr
 // ---- S_hat^-1 step at pressure vertex vtx:
 //   d' = c1 d + c2 D^-1 (r - M_p z),  z' = z + d'   (into the other buffers of the pairs).
 // (M_p z)_v sums the element products of the up to 8 cells around v, s_K sum_w m(v, w) z_w with
-// s_K = h^3 / mu_K and m = M1 x M1 x M1 (M1 the 1D Q1 mass matrix on [0,1]); the 27 neighbouring
-// values are split once. In FP64 the 64 multiply-adds per vertex would bind the kernel to the FP64
-// pipe (1/72 of the FP32 rate).
+// s_K = h^3 / mu_K and m = M1 x M1 x M1, M1 = (2, 1; 1, 2)/6 on [0,1]: the sums of the 8 cells are formed
+// together axis by axis (2 z_v + z_w towards each side: 38 additions for 64 products), the factor
+// 1/216 at the end. In double-float: in FP64 the additions would bind the kernel to the FP64 pipe.
+// z(i, j, k) is the vertex value at offset i - 1, j - 1, k - 1 from v, scale(i, j, k) the s_K of the cell towards
+// side i, j, k (0: lower), 0 outside the mesh.
+template <typename Z, typename S>
+__host__ __device__ __forceinline__ double schur_sum(const Z& z, const S& scale) {
+    using q2::df64;
+    auto side = [](const df64& own, const df64& other) { return df64(own.hi + own.hi, own.lo + own.lo) + other; };
+    df64 c[3][2][2];   // [k][side along y][side along x]
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        df64 a[3][2];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const df64 own = z(1, j, k);
+            a[j][0] = side(own, z(0, j, k));
+            a[j][1] = side(own, z(2, j, k));
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            c[k][0][i] = side(a[1][i], a[0][i]);
+            c[k][1][i] = side(a[1][i], a[2][i]);
+        }
+    }
+    df64 acc;
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) acc = acc + scale(i, j, k) * side(c[1][j][i], c[2 * k][j][i]);
+    return acc.to_double() * (1.0 / 216.0);
+}
+__host__ __device__ __forceinline__ void schur_update(double mz, const double* __restrict__ r, const double* __restrict__ dinv,
+                                                      const double* __restrict__ z, const double* __restrict__ d,
+                                                      double* __restrict__ z_new, double* __restrict__ d_new, double c1,
+                                                      double c2, size_t vtx) {
+    const double dn = (c1 != 0.0 ? c1 * d[vtx] : 0.0) + c2 * (dinv[vtx] * (r[vtx] - mz));
+    d_new[vtx] = dn;
+    z_new[vtx] = z[vtx] + dn;
+}
+// The values that the step at one vertex needs, in double-float, 0 outside the mesh.
+__host__ __device__ __forceinline__ q2::df64 schur_z(int n, const double* __restrict__ z, int i, int j, int k) {
+    const int P = n + 1;
+    return i >= 0 && j >= 0 && k >= 0 && i < P && j < P && k < P ? q2::split_double(z[size_t(i) + size_t(P) * (j + size_t(P) * k)])
+                                                                 : q2::df64();
+}
+__host__ __device__ __forceinline__ q2::df64 schur_scale(int n, const double* __restrict__ scale, int i, int j, int k) {
+    return i >= 0 && j >= 0 && k >= 0 && i < n && j < n && k < n ? q2::split_double(scale[size_t(i) + size_t(n) * (j + size_t(n) * k)])
+                                                                 : q2::df64();
+}
+// One vertex on its own (k_schur_cheb runs the same with the values of a tile in shared memory).
 __host__ __device__ __forceinline__ void schur_vertex(int n, const double* __restrict__ scale,
                                                       const double* __restrict__ r, const double* __restrict__ dinv,
                                                       const double* __restrict__ z, const double* __restrict__ d,
                                                       double* __restrict__ z_new, double* __restrict__ d_new,
                                                       double c1, double c2, size_t vtx) {
-    using q2::df64;
     const int P = n + 1;
     const int vi = int(vtx % P), vj = int((vtx / P) % P), vk = int(vtx / (size_t(P) * P));
-    df64 zz[3][3][3];   // [k][j][i], the vertex (vi + i - 1, vj + j - 1, vk + k - 1)
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                const int wi = vi + i - 1, wj = vj + j - 1, wk = vk + k - 1;
-                const bool in = wi >= 0 && wj >= 0 && wk >= 0 && wi < P && wj < P && wk < P;
-                zz[k][j][i] = in ? q2::split_double(z[size_t(wi) + size_t(P) * (wj + size_t(P) * wk)]) : df64();
-            }
-    df64 acc;
-#pragma unroll
-    for (int ck = 0; ck < 2; ++ck)
-#pragma unroll
-        for (int cj = 0; cj < 2; ++cj)
-#pragma unroll
-            for (int ci = 0; ci < 2; ++ci) {
-                // cell (vi - 1 + ci, ...): v is its local corner (1 - ci, 1 - cj, 1 - ck)
-                const int gi = vi - 1 + ci, gj = vj - 1 + cj, gk = vk - 1 + ck;
-                if (gi < 0 || gj < 0 || gk < 0 || gi >= n || gj >= n || gk >= n) continue;
-                df64 inner;
-#pragma unroll
-                for (int wk = 0; wk < 2; ++wk)
-#pragma unroll
-                    for (int wj = 0; wj < 2; ++wj)
-#pragma unroll
-                        for (int wi = 0; wi < 2; ++wi) {
-                            const double m = q2::M1(1 - ci, wi) * q2::M1(1 - cj, wj) * q2::M1(1 - ck, wk);
-                            q2::mac(inner, df64(m), zz[ck + wk][cj + wj][ci + wi]);
-                        }
-                q2::renorm(inner);
-                acc = acc + q2::split_double(scale[size_t(gi) + size_t(n) * (gj + size_t(n) * gk)]) * inner;
-            }
-    const double mz = acc.to_double();
-    const double dn = (c1 != 0.0 ? c1 * d[vtx] : 0.0) + c2 * (dinv[vtx] * (r[vtx] - mz));
-    d_new[vtx] = dn;
-    z_new[vtx] = z[vtx] + dn;
+    const double mz = schur_sum([&](int i, int j, int k) { return schur_z(n, z, vi + i - 1, vj + j - 1, vk + k - 1); },
+                                [&](int i, int j, int k) { return schur_scale(n, scale, vi + i - 1, vj + j - 1, vk + k - 1); });
+    schur_update(mz, r, dinv, z, d, z_new, d_new, c1, c2, vtx);
 }
 
 }  // namespace stk
