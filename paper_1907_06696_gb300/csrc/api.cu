@@ -293,22 +293,26 @@ double tridiag_max_eig(const std::vector<double>& a, const std::vector<double>& 
 }
 
 // Level-operator selector for launch_level_op: 1 = brick kernel, 2 = tensor-core brick kernel,
-// 3 = component-split kernel (FP32 levels), else the cell kernel's block size. By default the
-// FP32 levels of at most kSplitMaxN^3 cells take the component-split kernel: there a level
-// operator is one short wave and its time one thread's serial work, which the split divides by 3.
-constexpr int kSplitMaxN = 16;
-// From this size up the FP32 level operator marches over layers with the epilogue in the same launch:
-// a degree-4 smoothing takes 197 / 528 / 1,196 us at 64^3 / 96^3 / 128^3 (cell kernel and vector
-// passes 208 / 702 / 1,624 us); below, its layers are too few to hide one layer's latency (48^3: 90 and
-// 92 us, 32^3: equal, and slower inside the captured V-cycle).
-constexpr int kMarchMinN = 64;
+// 3 = component-split kernel (FP32 levels), else the cell kernel's block size. By default the smallest and the
+// largest FP32 levels take the operators with the epilogue in the same launch:
+// - at most kBlockMaxN cells per axis: blocks of 4 x 4 x 4 cells (block.cu). A degree-4 smoothing takes 24.7 / 26.0
+//   us at 8^3 / 16^3 (component-split kernel and vector passes 32.8 / 32.8 us); at 24^3 both take 41 us, at
+//   32^3 65.6 and 57.4 us: its blocks compute two cells for each that they own;
+// - from kMarchMinN up: tiles that march over layers (march.cu), 197 / 528 / 1,196 us at 64^3 / 96^3 / 128^3 (cell
+//   kernel and vector passes 208 / 702 / 1,624 us); below, the layers are too few to hide one layer's latency;
+// - between them the cell kernel and vector passes.
+constexpr int kBlockMaxN = 16, kMarchMinN = 64;
 
 template <typename T>
 int level_kernel(const stokes_ctx* c, int l) {
     const int k = c->opt.vmult_kernel;
     if (k == 1 || k == 2 || k == 3) return k;
-    if (sizeof(T) == 4 && c->lev[l].g.n <= kSplitMaxN) return 3;
-    if (sizeof(T) == 4 && c->opt.fused_smoother == 0 && c->lev[l].g.n >= kMarchMinN) return kMarchKernel;
+    const int n = c->lev[l].g.n;
+    if (sizeof(T) == 4 && c->opt.fused_smoother == 0) {
+        if (n <= kBlockMaxN) return kBlockKernel;
+        if (n >= kMarchMinN) return kMarchKernel;
+    }
+    if (sizeof(T) == 4 && n <= kBlockMaxN) return 3;   // steps carried by the products (fused_smoother)
     return c->cell_block;
 }
 
@@ -317,16 +321,18 @@ int level_kernel(const stokes_ctx* c, int l) {
 template <typename... P>
 bool aligned16(const P*... p) { return ((reinterpret_cast<uintptr_t>(p) | ...) & 15u) == 0; }
 
+// Whether a smoothing step on level l with these vectors writes its iterate beside the old one.
 template <typename T>
-bool marches(const stokes_ctx* c, int l, const T* a, const T* b) {
-    return level_kernel<T>(c, l) == kMarchKernel && aligned16(a, b);
+bool out_of_place(const stokes_ctx* c, int l, const T* a, const T* b) {
+    const int k = level_kernel<T>(c, l);
+    return k == kBlockKernel || (k == kMarchKernel && aligned16(a, b));
 }
 
 template <typename T>
 stokes_status vmult_level(stokes_ctx* c, int l, const T* src, T* dst, cudaStream_t s) {
     Level& L = c->lev[l];
     int k = level_kernel<T>(c, l);
-    if (k == kMarchKernel && !marches<T>(c, l, src, dst)) k = c->cell_block;
+    if (k == kMarchKernel && !aligned16(src, dst)) k = c->cell_block;
     CK(launch_level_op<T>(k, L.g, L.planes, EPI_PLAIN, vecs<T>(L).mu, src, dst, nullptr, nullptr, nullptr, 0.0, 0.0,
                           slots<T>(L), vecs<T>(L).acc, s, &c->tc));
     return STOKES_OK;
@@ -352,19 +358,26 @@ stokes_status smooth(stokes_ctx* c, int l, const T* b, T* x, bool zero_guess, cu
     const double sigma = theta / delta;
     double rho = 1.0 / sigma;
     const size_t n = L.g.n_u;
-    // the marching operator writes the new iterate beside the old one (its neighbours read that): the
-    // iterates alternate between x and the level's x2, starting where the last step ends in x
-    const bool march = marches<T>(c, l, b, x);
+    // the operators with the epilogue inside write the new iterate beside the old one (its neighbours
+    // read that): the iterates alternate between x and the level's x2, starting where the last step
+    // ends in x
+    const bool apart = out_of_place<T>(c, l, b, x), block = level_kernel<T>(c, l) == kBlockKernel;
     T* X[2] = {x, v.x2};
-    int cur = march ? (c->opt.cheb_degree - (zero_guess ? 1 : 0)) & 1 : 0;
+    int cur = apart ? (c->opt.cheb_degree - (zero_guess ? 1 : 0)) & 1 : 0;
+    bool pending = false;   // the first step from zero, left to the block kernel's gather
     auto step = [&](double c1, double c2) -> stokes_status {
-        if (!march) return cheb_step<T>(c, l, b, x, c1, c2, s);
-        if constexpr (sizeof(T) == 4)
-            CK(launch_march(EPI_CHEB, L.g, v.mu, X[cur], X[cur ^ 1], b, v.dinv, v.d, c1, c2, s));
+        if (!apart) return cheb_step<T>(c, l, b, x, c1, c2, s);
+        if constexpr (sizeof(T) == 4) {
+            if (block) CK(launch_block(EPI_CHEB, L.g, v.mu, pending ? nullptr : X[cur], X[cur ^ 1], b, v.dinv, v.d, 1.0 / theta, c1, c2, s));
+            else CK(launch_march(EPI_CHEB, L.g, v.mu, X[cur], X[cur ^ 1], b, v.dinv, v.d, c1, c2, s));
+        }
+        pending = false;
         cur ^= 1;
         return STOKES_OK;
     };
-    if (zero_guess) {
+    if (zero_guess && apart && block && c->opt.cheb_degree > 1) {
+        pending = true;
+    } else if (zero_guess) {
         CK(launch_cheb_update<T>(n, b, nullptr, v.dinv, v.d, X[cur], 0.0, 1.0 / theta, false, s));
     } else {
         if (cur == 1) CK(cudaMemcpyAsync(v.x2, x, n * sizeof(T), cudaMemcpyDeviceToDevice, s));
@@ -1784,7 +1797,7 @@ stokes_status setup_impl(const stokes_mesh* mesh, const stokes_mu* mu, const sto
             CKS(dalloc(c, p, nu));
         CK(cudaMemsetAsync(Lv.v64.acc, 0, nu * sizeof(double), s));
         CK(cudaMemsetAsync(Lv.v32.acc, 0, nu * sizeof(float), s));
-        if (level_kernel<float>(c, l) == kMarchKernel) {   // it leaves the boundary entries as they are: zero
+        if (level_kernel<float>(c, l) == kMarchKernel || level_kernel<float>(c, l) == kBlockKernel) {   // they leave the boundary entries as they are: zero
             CKS(dalloc(c, &Lv.v32.x2, nu));
             for (float* p : {Lv.v32.x, Lv.v32.r, Lv.v32.x2}) CK(cudaMemsetAsync(p, 0, nu * sizeof(float), s));
         }
@@ -2863,7 +2876,7 @@ stokes_status stokes_smooth(stokes_ctx* c, int level, int prec, const void* b, v
     if (prec == STOKES_FP32) {
         const float* bf = static_cast<const float*>(b);
         float* xf = static_cast<float*>(x);
-        if (zero_guess && marches<float>(c, level, bf, xf)) CK(launch_zero_boundary<float>(c->lev[level].g, xf, s));
+        if (zero_guess && out_of_place<float>(c, level, bf, xf)) CK(launch_zero_boundary<float>(c->lev[level].g, xf, s));
         return fused_level<float>(c, level) ? smooth_fused<float>(c, level, bf, xf, zero_guess != 0, nullptr, s)
                                             : smooth<float>(c, level, bf, xf, zero_guess != 0, s);
     }

@@ -629,10 +629,12 @@ template <typename T>
 cudaError_t launch_level_op(int kernel, const LevelGeom& g, const PlaneLayout& L, int epi, const T* mu, const T* src,
                             T* dst, const T* b, const T* dinv, T* d, double c1, double c2, T* slots, T* acc,
                             cudaStream_t s, const TcArgs* tc) {
-    if (kernel == kMarchKernel) {
+    if (kernel == kMarchKernel || kernel == kBlockKernel) {
         if constexpr (sizeof(T) == 4) {
             if (epi == EPI_CHEB) return cudaErrorInvalidValue;
-            const cudaError_t e = launch_march(epi, g, mu, src, dst, b, nullptr, nullptr, 0.0, 0.0, s);
+            const cudaError_t e = kernel == kMarchKernel
+                                      ? launch_march(epi, g, mu, src, dst, b, nullptr, nullptr, 0.0, 0.0, s)
+                                      : launch_block(epi, g, mu, src, dst, b, nullptr, nullptr, 0.0, 0.0, 0.0, s);
             return e != cudaSuccess || epi != EPI_PLAIN ? e : launch_copy_boundary<T>(g, src, dst, s);
         } else {
             return cudaErrorInvalidValue;

@@ -424,6 +424,12 @@ cudaError_t launch_cell_tc(const BrickArgs<float>& a, float* acc, const TcArgs& 
 constexpr int kMarchKernel = 4;
 cudaError_t launch_march(int epi, const LevelGeom& g, const float* mu, const float* src, float* dst, const float* b,
                          const float* dinv, float* d, double c1, double c2, cudaStream_t s);
+// The same on levels of any size in blocks of 4 x 4 x 4 cells (block.cu), no alignment asked; entries on the
+// domain boundary are left as they are. EPI_CHEB with src null: the first step from zero is pending,
+// src = d = c0 dinv b.
+constexpr int kBlockKernel = 5;
+cudaError_t launch_block(int epi, const LevelGeom& g, const float* mu, const float* src, float* dst, const float* b,
+                         const float* dinv, float* d, double c0, double c1, double c2, cudaStream_t s);
 cudaError_t march_configure();   // shared-memory opt-in; once before any launch or capture
 
 // A x with an epilogue (EPI_PLAIN: dst = A x; EPI_RESID: dst = b - A x;
@@ -434,7 +440,7 @@ cudaError_t march_configure();   // shared-memory opt-in; once before any launch
 // kernel 3: FP32: the cell kernel's accumulation with three threads per cell (one per output
 //           component), the same consumer kernels; FP64: kernel 128;
 // kernel 1: the brick-tiled kernel with the epilogue fused (slots: brick_layout(n).total entries);
-// kernel 4: FP32: the marching kernel, EPI_PLAIN and EPI_RESID (EPI_CHEB is out of place: launch_march);
+// kernel 4, 5: FP32: the marching and the block kernel, EPI_PLAIN and EPI_RESID (EPI_CHEB is out of place);
 // kernel 2: FP32: the cell products on the tensor cores, accumulated like kernel 0 (tc must be
 //           given); FP64: kernel 128.
 template <typename T>
