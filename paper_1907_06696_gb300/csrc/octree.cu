@@ -27,9 +27,14 @@ inline unsigned blocks_for(size_t n, int t) {
     return unsigned(b == 0 ? 1 : b);
 }
 
-// Quadratic Lagrange basis on {0, 1/2, 1} at positions 0, 1/4, 1/2, 3/4, 1 of a parent cell.
-__constant__ double c_q2_at[5][3] = {{1, 0, 0}, {0.375, 0.75, -0.125}, {0, 1, 0}, {-0.125, 0.75, 0.375}, {0, 0, 1}};
-__device__ __forceinline__ double q2_at(int p, int m) { return c_q2_at[p][m]; }
+// Quadratic Lagrange basis on {0, 1/2, 1} at position p/4 of a parent cell: the three weights of an axis.
+// They and their products over the axes are exact in either precision.
+template <typename T>
+__device__ __forceinline__ void q2_at(int p, T (&w)[3]) {
+    w[0] = p == 0 ? T(1) : (p == 1 ? T(0.375) : (p == 3 ? T(-0.125) : T(0)));
+    w[1] = p == 1 || p == 3 ? T(0.75) : (p == 2 ? T(1) : T(0));
+    w[2] = p == 4 ? T(1) : (p == 1 ? T(-0.125) : (p == 3 ? T(0.375) : T(0)));
+}
 
 // Is entry v, read at position `at` of table t, below `bound`? STOKES_DEBUG builds check and record
 // the first failure (flag, table + 1, position); release builds return true without a test.
@@ -119,12 +124,18 @@ __global__ void k_oct_prolongate(OctLevelDev F, OctLevelDev C, const T* __restri
     T v[3] = {T(0), T(0), T(0)};
     if (idx_ok(F.dbg, OCT_PARENT, par, C.n_cells, n) && idx_ok(F.dbg, OCT_POS, p, 125, n)) {
         const int32_t* cn = C.cell_nodes + size_t(par) * 27;
+        T wx[3], wy[3], wz[3];
+        q2_at(px, wx);
+        q2_at(py, wy);
+        q2_at(pz, wz);
+#pragma unroll
         for (int b = 0; b < 27; ++b) {
-            const double w = q2_at(px, b % 3) * q2_at(py, (b / 3) % 3) * q2_at(pz, b / 9);
-            if (w == 0.0) continue;
+            const T w = wx[b % 3] * wy[b / 3 % 3] * wz[b / 9];
+            if (w == T(0)) continue;
             const int32_t node = cn[b];
             if (!idx_ok(C.dbg, OCT_CELL_NODES, node, (long long)C.nn, size_t(par) * 27 + b)) continue;
-            for (int c = 0; c < 3; ++c) v[c] += T(w) * coarse[c * C.nn + node];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) v[c] += w * coarse[c * C.nn + node];
         }
     }
     for (int c = 0; c < 3; ++c) fine[c * F.nn + n] = (add ? fine[c * F.nn + n] : T(0)) + v[c];
@@ -139,13 +150,19 @@ __global__ void k_oct_restrict_add(OctLevelDev F, OctLevelDev C, const T* __rest
     if (!idx_ok(F.dbg, OCT_PARENT, par, C.n_cells, n) || !idx_ok(F.dbg, OCT_POS, p, 125, n)) return;
     const int32_t* cn = C.cell_nodes + size_t(par) * 27;
     const T f[3] = {fine[n], fine[F.nn + n], fine[2 * F.nn + n]};
+    T wx[3], wy[3], wz[3];
+    q2_at(px, wx);
+    q2_at(py, wy);
+    q2_at(pz, wz);
+#pragma unroll
     for (int b = 0; b < 27; ++b) {
-        const double w = q2_at(px, b % 3) * q2_at(py, (b / 3) % 3) * q2_at(pz, b / 9);
-        if (w == 0.0) continue;
+        const T w = wx[b % 3] * wy[b / 3 % 3] * wz[b / 9];
+        if (w == T(0)) continue;
         const int32_t node = cn[b];
         if (!idx_ok(C.dbg, OCT_CELL_NODES, node, (long long)C.nn, size_t(par) * 27 + b)) continue;
         if (C.flags[node] & 1) continue;
-        for (int c = 0; c < 3; ++c) atomicAdd(coarse + c * C.nn + node, T(w) * f[c]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) atomicAdd(coarse + c * C.nn + node, w * f[c]);
     }
 }
 
