@@ -7,6 +7,7 @@
 // Every kernel takes one cell (or one node) per thread. Level vectors are component-blocked
 // [3][nn]; the active velocity vector is [3][nu] and the active pressure vector [np].
 #include "octree.cuh"
+#include "outer.cuh"
 #include "prof.cuh"
 #include "q2_basis.cuh"
 
@@ -259,40 +260,67 @@ __device__ __forceinline__ void scatter_p(const OctActiveDev& a, double* dst, in
     }
 }
 
+// One velocity component per thread, 32 leaves per CTA, in the fixed-point arithmetic of the uniform
+// outer operator (outer.cuh): warp c gathers component c through the leaf's references and scatters it the same
+// way. 3,431 leaves: 168 -> 133 us (one thread per leaf with FP64 instructions in the
+// modes); 79,080 leaves: 385 -> 383 us, bound by the hanging nodes, whose terms every lane waits for.
 template <bool DO_A, bool DO_BT, bool DO_B>
-__global__ void __launch_bounds__(128) k_oct_active(OctActiveDev a, const double* __restrict__ src_u,
-                                                    const double* __restrict__ src_p, double* __restrict__ dst_u,
-                                                    double* __restrict__ dst_p) {
-    const int leaf = blockIdx.x * blockDim.x + threadIdx.x;
-    if (leaf >= a.n_leaves) return;
-    const int32_t* ru = a.leaf_u + size_t(leaf) * 27;
-    const int32_t* rp = a.leaf_p + size_t(leaf) * 8;
+__global__ void __launch_bounds__(kOuterThreads, 5) k_oct_active(OctActiveDev a, const double* __restrict__ src_u,
+                                                                 const double* __restrict__ src_p, double* __restrict__ dst_u,
+                                                                 double* __restrict__ dst_p) {
+    __shared__ OuterShared sh;
+    const int C = int(threadIdx.x) / kOuterCells, g = int(threadIdx.x) % kOuterCells;
+    const int leaf = int(blockIdx.x) * kOuterCells + g;
+    const bool valid = leaf < a.n_leaves;
+    const int32_t* ru = a.leaf_u + size_t(valid ? leaf : 0) * 27;
+    const int32_t* rp = a.leaf_p + size_t(valid ? leaf : 0) * 8;
+    // strides of the own frame's axes in the leaf's 27 nodes
+    const int q0 = C == 0 ? 1 : (C == 1 ? 3 : 9), q1 = C == 0 ? 3 : (C == 1 ? 9 : 1), q2 = C == 0 ? 9 : (C == 1 ? 1 : 3);
+    {
+        double T[27];
+        if (DO_A || DO_B) {
+            int e = 0;
+#pragma unroll
+            for (int m = 0; m < 27; ++m) {
+                const int at = (m % 3) * q0 + (m / 3 % 3) * q1 + (m / 9) * q2;
+                T[m] = valid ? gather_u(a, src_u, C, ru[at], size_t(leaf) * 27 + at) : 0.0;
+                e = max(e, exp_of(__double_as_longlong(T[m])));
+            }
+            sh.eu[C][g] = e;
+        }
+        if (DO_BT) {
+            int e = 0;
+            for (int v = C; v < 8; v += 3) {
+                const long long b = __double_as_longlong(valid ? gather_p(a, src_p, rp[v], size_t(leaf) * 8 + v) : 0.0);
+                e = max(e, exp_of(b));
+                sh.P[v][g] = b;
+            }
+            sh.ep[C][g] = e;
+        }
+        __syncthreads();
+        outer_modes<DO_A || DO_B, DO_BT>(C, g, sh, T);
+    }
+    __syncthreads();
+    if (!valid) return;
     const double h = ldexp(1.0, -int(a.level[leaf]));
-    const double s = -h * h;
-    double u[3][27], w[3][27], p8[8], pb[8];
-    if (DO_A || DO_B) {
-#pragma unroll
-        for (int m = 0; m < 27; ++m) {
-            const int32_t r = ru[m];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) u[c][m] = gather_u(a, src_u, c, r, size_t(leaf) * 27 + m);
+    if (DO_B) {
+        long long b[8];
+        const double s = outer_pressure(C, g, sh, h, b);
+        const int v1 = 1 << C, v6 = 7 - v1;   // as in outer_phase2: each vertex by one warp
+        scatter_p(a, dst_p, rp[v1], fix_out(b[1], s), size_t(leaf) * 8 + v1);
+        scatter_p(a, dst_p, rp[v6], fix_out(b[6], s), size_t(leaf) * 8 + v6);
+        if (C < 2) {
+            const int v = C == 0 ? 0 : 7;
+            scatter_p(a, dst_p, rp[v], fix_out(C == 0 ? b[0] : b[7], s), size_t(leaf) * 8 + v);
         }
     }
-    if (DO_BT) {
-#pragma unroll
-        for (int v = 0; v < 8; ++v) p8[v] = s * gather_p(a, src_p, rp[v], size_t(leaf) * 8 + v);
-    }
-    q2::cell_stokes<DO_A, DO_BT, DO_B>(u, p8, DO_A ? a.mu[leaf] * h : 0.0, w, pb);
-    if (DO_B) {
-#pragma unroll
-        for (int v = 0; v < 8; ++v) scatter_p(a, dst_p, rp[v], s * pb[v], size_t(leaf) * 8 + v);
-    }
     if (DO_A || DO_BT) {
+        long long Y[27];
+        const double s = outer_velocity<DO_A, DO_BT>(C, g, sh, a.mu[leaf], h, Y);
 #pragma unroll
         for (int m = 0; m < 27; ++m) {
-            const int32_t r = ru[m];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) scatter_u(a, dst_u, c, r, w[c][m], size_t(leaf) * 27 + m);
+            const int at = (m % 3) * q0 + (m / 3 % 3) * q1 + (m / 9) * q2;
+            scatter_u(a, dst_u, C, ru[at], fix_out(Y[m], s), size_t(leaf) * 27 + at);
         }
     }
 }
@@ -392,12 +420,12 @@ cudaError_t launch_oct_active(const OctActiveDev& a, const double* src_u, const 
     cudaError_t e;
     if ((do_a || do_bt) && (e = cudaMemsetAsync(dst_u, 0, 3 * a.nu_nodes * sizeof(double), s)) != cudaSuccess) return e;
     if (do_b && (e = cudaMemsetAsync(dst_p, 0, a.np * sizeof(double), s)) != cudaSuccess) return e;
-    const unsigned g = blocks_for(a.n_leaves, 128);
+    const unsigned g = blocks_for(a.n_leaves, kOuterCells);
     const int cls = do_a ? PROF_STOKES_F64 : (do_bt ? PROF_BT_F64 : PROF_STOKES_F64);
-    if (do_a && do_bt && do_b) LAUNCH(cls, s, (k_oct_active<true, true, true><<<g, 128, 0, s>>>(a, src_u, src_p, dst_u, dst_p)));
-    else if (do_a && !do_bt && !do_b) LAUNCH(cls, s, (k_oct_active<true, false, false><<<g, 128, 0, s>>>(a, src_u, src_p, dst_u, dst_p)));
-    else if (!do_a && do_bt && !do_b) LAUNCH(cls, s, (k_oct_active<false, true, false><<<g, 128, 0, s>>>(a, src_u, src_p, dst_u, dst_p)));
-    else if (!do_a && !do_bt && do_b) LAUNCH(cls, s, (k_oct_active<false, false, true><<<g, 128, 0, s>>>(a, src_u, src_p, dst_u, dst_p)));
+    if (do_a && do_bt && do_b) LAUNCH(cls, s, (k_oct_active<true, true, true><<<g, kOuterThreads, 0, s>>>(a, src_u, src_p, dst_u, dst_p)));
+    else if (do_a && !do_bt && !do_b) LAUNCH(cls, s, (k_oct_active<true, false, false><<<g, kOuterThreads, 0, s>>>(a, src_u, src_p, dst_u, dst_p)));
+    else if (!do_a && do_bt && !do_b) LAUNCH(cls, s, (k_oct_active<false, true, false><<<g, kOuterThreads, 0, s>>>(a, src_u, src_p, dst_u, dst_p)));
+    else if (!do_a && !do_bt && do_b) LAUNCH(cls, s, (k_oct_active<false, false, true><<<g, kOuterThreads, 0, s>>>(a, src_u, src_p, dst_u, dst_p)));
     else return cudaErrorInvalidValue;
     if (do_a) LAUNCH(cls, s, (k_oct_active_boundary<<<blocks_for(a.nu_nodes, 256), 256, 0, s>>>(a, src_u, dst_u)));
     return cudaGetLastError();

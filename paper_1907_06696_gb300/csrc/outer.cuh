@@ -182,7 +182,6 @@ __host__ __device__ __forceinline__ void fix_from_modes(long long* x) {
 struct OuterFrame {
     int C;            // velocity component of this thread
     size_t sn[3];     // global node strides of local axes 0, 1, 2
-    int sv[3];        // global Q1-vertex bits (1, 2, 4 rotated)
     int cl[3];        // cell coordinates along the local axes
     int ci, cj, ck;   // global cell coordinates
 };
@@ -198,7 +197,6 @@ __host__ __device__ __forceinline__ OuterFrame outer_frame(const OuterArgs& a, i
     for (int d = 0; d < 3; ++d) {   // selects, not indexed arrays: those would live in local memory
         const int ax = (C + d) % 3;
         f.sn[d] = ax == 0 ? 1 : (ax == 1 ? M : M * M);
-        f.sv[d] = 1 << ax;
         f.cl[d] = ax == 0 ? f.ci : (ax == 1 ? f.cj : f.ck);
     }
     return f;
@@ -256,11 +254,11 @@ __host__ __device__ __forceinline__ int max3(const int (&e)[3][kOuterCells], int
     return m > e[2][g] ? m : e[2][g];
 }
 
-// Phase 1b (after a barrier): fixed point against the cell's largest magnitude, and the modes.
-template <bool DO_A, bool DO_B = true, bool DO_BT = true, typename V>
-__host__ __device__ __forceinline__ void outer_phase1b(const OuterArgs&, int C, int, int g, OuterShared& sh,
-                                                       const V (&T)[27]) {
-    if (DO_A || DO_B) {
+// This thread's component (raw FP64 bits T) in fixed point against the cell's largest magnitude, and its
+// modes; every third pressure value (sh.P) in fixed point. After the barrier behind sh.eu and sh.ep.
+template <bool DO_U, bool DO_P, typename V>
+__host__ __device__ __forceinline__ void outer_modes(int C, int g, OuterShared& sh, const V (&T)[27]) {
+    if (DO_U) {
         const int e = max3(sh.eu, g);
         long long X[27];
 #pragma unroll
@@ -275,43 +273,32 @@ __host__ __device__ __forceinline__ void outer_phase1b(const OuterArgs&, int C, 
 #pragma unroll
         for (int m = 0; m < 27; ++m) sh.U[C][m][g] = X[m];
     }
-    if (DO_BT) {
+    if (DO_P) {
         const int e = max3(sh.ep, g);
         for (int v = C; v < 8; v += 3) sh.P[v][g] = fix_round(sh.P[v][g], e);
     }
 }
 
-// Phase 2 (after a barrier): the element matrix in the modes, the transposed transform and the
-// scatter into the velocity output; B u at this warp's vertices.
-template <bool DO_A, bool DO_BT, bool DO_B = true, typename V>
-__host__ __device__ __forceinline__ void outer_phase2(const OuterArgs& a, int C, int blk, int g, const OuterShared& sh,
-                                                      V (&W)[27]) {
-    (void)W;
-    const size_t cells = size_t(a.n) * a.n * a.n;
-    const size_t cell = size_t(blk) * kOuterCells + g;
-    if (cell >= cells) return;
-    const OuterFrame f = outer_frame(a, C, cell);
-    const int D1 = (C + 1) % 3, D2 = (C + 2) % 3;
-    const int eu = DO_A || DO_B ? max3(sh.eu, g) : 0;
-    if (DO_B) {
-        long long b[8];
+// B u of a cell of side h at its vertices (warp C's frame: bit d of the index along global axis C + d), as
+// b scale. After the barrier behind outer_modes.
+__host__ __device__ __forceinline__ double outer_pressure(int C, int g, const OuterShared& sh, double h, long long (&b)[8]) {
+    const int D1 = (C + 1) % 3, D2 = (C + 2) % 3, eu = max3(sh.eu, g);
 #pragma unroll
-        for (int v = 0; v < 8; ++v) {
-            const int i = v & 1, j = (v >> 1) & 1, k = v >> 2;
-            b[v] = ((3 - i) * sh.U[C][(i + 1) + 3 * j + 9 * k][g] >> 2) + ((3 - j) * sh.U[D1][(j + 1) + 3 * k + 9 * i][g] >> 2) +
-                   ((3 - k) * sh.U[D2][(k + 1) + 3 * i + 9 * j][g] >> 2);
-        }
-        q2::from_pressure_modes(b);
-        const double s = fix_scale(-a.h * a.h / 864.0, eu - 1022 - kFixBits + 2, eu < kFixMinExp, eu == 0x7FF);
-        // the vertex one step along the own axis and its opposite; the two that no rotation moves
-        // go to warps 0 and 1
-        outer_atomic_add(a.dst_p + outer_vertex(a, f, f.sv[0]), fix_out(b[1], s));
-        outer_atomic_add(a.dst_p + outer_vertex(a, f, 7 - f.sv[0]), fix_out(b[6], s));
-        if (C < 2) outer_atomic_add(a.dst_p + outer_vertex(a, f, C == 0 ? 0 : 7), fix_out(C == 0 ? b[0] : b[7], s));
+    for (int v = 0; v < 8; ++v) {
+        const int i = v & 1, j = (v >> 1) & 1, k = v >> 2;
+        b[v] = ((3 - i) * sh.U[C][(i + 1) + 3 * j + 9 * k][g] >> 2) + ((3 - j) * sh.U[D1][(j + 1) + 3 * k + 9 * i][g] >> 2) +
+               ((3 - k) * sh.U[D2][(k + 1) + 3 * i + 9 * j][g] >> 2);
     }
-    if (!(DO_A || DO_BT)) return;
-    const double mu = a.mu[cell];
-    long long Y[27];
+    q2::from_pressure_modes(b);
+    return fix_scale(-h * h / 864.0, eu - 1022 - kFixBits + 2, eu < kFixMinExp, eu == 0x7FF);
+}
+
+// Component C of A u + B^T p of a cell of side h and viscosity mu, in warp C's frame, as Y scale.
+template <bool DO_A, bool DO_BT>
+__host__ __device__ __forceinline__ double outer_velocity(int C, int g, const OuterShared& sh, double mu, double h,
+                                                          long long (&Y)[27]) {
+    const int D1 = (C + 1) % 3, D2 = (C + 2) % 3;
+    const int eu = DO_A ? max3(sh.eu, g) : 0;
 #pragma unroll
     for (int k = 0; k < 3; ++k)
 #pragma unroll
@@ -334,14 +321,14 @@ __host__ __device__ __forceinline__ void outer_phase2(const OuterArgs& a, int C,
         // may exceed |u| by 2^10 before its share of the result is the larger one
         const int ep = max3(sh.ep, g);
         if (ep >= kFixMinExp) {
-            const long long kb = (long long)q2::dbl_bits(112.5 * a.h / mu);
+            const long long kb = (long long)q2::dbl_bits(112.5 * h / mu);
             const long long km = ((kb & 0xFFFFFFFFFFFFFLL) | (1LL << 52)) << 10;
             const int epk = ep + exp_of(kb) - 1022;
             E = E > epk - 10 ? E : epk - 10;
             long long P[8];
 #pragma unroll
             for (int v = 0; v < 8; ++v)
-                P[v] = sh.P[(v & 1) * f.sv[0] + ((v >> 1) & 1) * f.sv[1] + (v >> 2) * f.sv[2]][g];
+                P[v] = sh.P[((v & 1) << C) + (((v >> 1) & 1) << D1) + ((v >> 2) << D2)][g];
             q2::to_pressure_modes(P);
             const int sp = E - epk + 16 < 63 ? E - epk + 16 : 63;
             const int sa = DO_A ? (E - eu < 63 ? E - eu : 63) : 0;
@@ -360,7 +347,38 @@ __host__ __device__ __forceinline__ void outer_phase2(const OuterArgs& a, int C,
     fix_from_modes<2>(Y);
     fix_from_modes<1>(Y);
     fix_from_modes<0>(Y);
-    const double s = fix_scale(mu * a.h * (1.0 / 97200.0), E - 1022 - kFixBits + kFixMid, E == 0, bad);
+    return fix_scale(mu * h * (1.0 / 97200.0), E - 1022 - kFixBits + kFixMid, E == 0, bad);
+}
+
+// Phase 1b (after a barrier): fixed point and modes.
+template <bool DO_A, bool DO_B = true, bool DO_BT = true, typename V>
+__host__ __device__ __forceinline__ void outer_phase1b(const OuterArgs&, int C, int, int g, OuterShared& sh,
+                                                       const V (&T)[27]) {
+    outer_modes<DO_A || DO_B, DO_BT>(C, g, sh, T);
+}
+
+// Phase 2 (after a barrier): the element matrix in the modes, the transposed transform and the
+// scatter into the velocity output; B u at this warp's vertices.
+template <bool DO_A, bool DO_BT, bool DO_B = true, typename V>
+__host__ __device__ __forceinline__ void outer_phase2(const OuterArgs& a, int C, int blk, int g, const OuterShared& sh,
+                                                      V (&W)[27]) {
+    (void)W;
+    const size_t cells = size_t(a.n) * a.n * a.n;
+    const size_t cell = size_t(blk) * kOuterCells + g;
+    if (cell >= cells) return;
+    const OuterFrame f = outer_frame(a, C, cell);
+    if (DO_B) {
+        long long b[8];
+        const double s = outer_pressure(C, g, sh, a.h, b);
+        // the vertex one step along the own axis and its opposite; the two that no rotation moves
+        // go to warps 0 and 1
+        outer_atomic_add(a.dst_p + outer_vertex(a, f, 1 << C), fix_out(b[1], s));
+        outer_atomic_add(a.dst_p + outer_vertex(a, f, 7 - (1 << C)), fix_out(b[6], s));
+        if (C < 2) outer_atomic_add(a.dst_p + outer_vertex(a, f, C == 0 ? 0 : 7), fix_out(C == 0 ? b[0] : b[7], s));
+    }
+    if (!(DO_A || DO_BT)) return;
+    long long Y[27];
+    const double s = outer_velocity<DO_A, DO_BT>(C, g, sh, a.mu[cell], a.h, Y);
     double* dst = a.dst_u + size_t(C) * a.nodes +
                   (size_t(2 * f.ci) + size_t(a.M) * (size_t(2 * f.cj) + size_t(a.M) * size_t(2 * f.ck)));
 #pragma unroll
