@@ -166,6 +166,7 @@ struct OctCtx {
     OctActiveDev act;
     std::vector<OctLevel> lev;
     double* leaf_mu = nullptr;
+    double* vx = nullptr;         // output of the captured V-cycle (3 nu_nodes)
 };
 
 template <typename T> LevelVecs<T>& ovecs(OctLevel& L);
@@ -503,12 +504,11 @@ stokes_status vcycle_level(stokes_ctx* c, int l, cudaStream_t s) {
     return STOKES_OK;
 }
 
-// The level recursion of one V-cycle. It touches only the context's level buffers, so it is
-// captured once per precision as a CUDA graph and replayed on the library stream (ordered
-// after and before the caller's stream by events). Profiling runs it launch by launch.
-template <typename T>
-stokes_status run_levels(stokes_ctx* c, cudaStream_t s) {
-    if (!c->opt.graphs || prof_enabled()) return vcycle_level<T>(c, c->L - 1, s);
+// The launches of body(stream), captured on first use as the graph of precision T and replayed on the
+// library stream, ordered after and before the caller's stream by events. body touches only the
+// context's own buffers.
+template <typename T, typename Body>
+stokes_status run_graph(stokes_ctx* c, cudaStream_t s, Body body) {
     const int p = sizeof(T) == 4 ? 1 : 0;
     if (!c->gstream) {
         CK(cudaStreamCreateWithFlags(&c->gstream, cudaStreamNonBlocking));
@@ -521,7 +521,7 @@ stokes_status run_levels(stokes_ctx* c, cudaStream_t s) {
         cudaGraph_t graph = nullptr;
         const long long before = launch_total();
         CK(cudaStreamBeginCapture(c->gstream, cudaStreamCaptureModeThreadLocal));
-        stokes_status st = vcycle_level<T>(c, c->L - 1, c->gstream);
+        stokes_status st = body(c->gstream);
         cudaError_t e = cudaStreamEndCapture(c->gstream, &graph);
         if (st != STOKES_OK) {
             if (graph) cudaGraphDestroy(graph);
@@ -538,6 +538,13 @@ stokes_status run_levels(stokes_ctx* c, cudaStream_t s) {
     CK(cudaEventRecord(c->gev_out, c->gstream));
     CK(cudaStreamWaitEvent(s, c->gev_out, 0));
     return STOKES_OK;
+}
+
+// The level recursion of one V-cycle. Profiling runs it launch by launch.
+template <typename T>
+stokes_status run_levels(stokes_ctx* c, cudaStream_t s) {
+    if (!c->opt.graphs || prof_enabled()) return vcycle_level<T>(c, c->L - 1, s);
+    return run_graph<T>(c, s, [c](cudaStream_t g) { return vcycle_level<T>(c, c->L - 1, g); });
 }
 
 template <typename T>
@@ -615,10 +622,9 @@ stokes_status oct_vcycle_level(stokes_ctx* c, int li, cudaStream_t s) {
     return STOKES_OK;
 }
 
-// x = V(rhs) on the active velocity space (FP64 vectors, V-cycle arithmetic T); Dirichlet
-// rows act as the identity.
+// All launches of x = V(rhs) but the copies of the caller's vectors.
 template <typename T>
-stokes_status oct_vcycle(stokes_ctx* c, const double* rhs, double* x, cudaStream_t s) {
+stokes_status oct_vcycle_body(stokes_ctx* c, const double* rhs, double* x, cudaStream_t s) {
     OctCtx& o = *c->oct;
     const size_t nu = o.act.nu_nodes;
     for (OctLevel& L : o.lev) {
@@ -629,6 +635,24 @@ stokes_status oct_vcycle(stokes_ctx* c, const double* rhs, double* x, cudaStream
     for (OctLevel& L : o.lev)
         CK(launch_oct_copy_from_level<T>(L.n_copy, L.copy_a, L.copy_l, nu, L.g.nn, ovecs<T>(L).x, x, L.g.dbg, s));
     CK(launch_oct_identity_rows(o.act, rhs, x, s));
+    return STOKES_OK;
+}
+
+// x = V(rhs) on the active velocity space (FP64 vectors, V-cycle arithmetic T); Dirichlet
+// rows act as the identity. As on uniform meshes the launches are replayed as a graph: its input is
+// c->tu, its output oct->vx, so that no pointer of the caller's is in it. The copies cost 2 us at the
+// 3,431 leaves of the shell mesh. A caller that captures its own stream, profiling and graphs = 0 get the
+// launches one by one.
+template <typename T>
+stokes_status oct_vcycle(stokes_ctx* c, const double* rhs, double* x, cudaStream_t s) {
+    OctCtx& o = *c->oct;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(s, &cap));
+    if (!c->opt.graphs || prof_enabled() || cap != cudaStreamCaptureStatusNone) return oct_vcycle_body<T>(c, rhs, x, s);
+    const size_t bytes = 3 * o.act.nu_nodes * sizeof(double);
+    if (rhs != c->tu) CK(cudaMemcpyAsync(c->tu, rhs, bytes, cudaMemcpyDeviceToDevice, s));
+    CKS(run_graph<T>(c, s, [c, &o](cudaStream_t g) { return oct_vcycle_body<T>(c, c->tu, o.vx, g); }));
+    CK(cudaMemcpyAsync(x, o.vx, bytes, cudaMemcpyDeviceToDevice, s));
     return STOKES_OK;
 }
 
@@ -2054,6 +2078,7 @@ stokes_status oct_setup_impl(const stokes_octree* mesh, const stokes_mu* mu, con
     CKS(dalloc(c, &c->sp_d, np));
     CKS(dalloc(c, &c->sp_t, np));
     CKS(dalloc(c, &c->tu, nu));
+    CKS(dalloc(c, &c->oct->vx, nu));
     CKS(dalloc(c, &c->partials, size_t(std::max(multidot_blocks(), gs_partials_blocks())) * (o.restart + 8)));
     CKS(dalloc(c, &c->dots, size_t(o.restart + 8)));
     CK(cudaMallocHost(&c->dots_host, size_t(3 * (o.restart + 8)) * sizeof(double)));
