@@ -56,13 +56,14 @@ __device__ __forceinline__ bool idx_ok(const OctDebug& d, int t, long long v, lo
 #endif
 }
 
-template <typename T>
-__global__ void __launch_bounds__(128) k_oct_cells(OctLevelDev L, const T* __restrict__ mu, const T* __restrict__ src,
-                                                   T* __restrict__ acc) {
+// acc += A_l src over the cells of an FP32 level, one thread per cell. (Three threads per cell, one component
+// each, measured slower: FP32 V-cycle on 79,000 leaves 680 -> 732 us.)
+__global__ void __launch_bounds__(128) k_oct_cells(OctLevelDev L, const float* __restrict__ mu, const float* __restrict__ src,
+                                                   float* __restrict__ acc) {
     const int cell = blockIdx.x * blockDim.x + threadIdx.x;
     if (cell >= L.n_cells) return;
     const int32_t* cn = L.cell_nodes + size_t(cell) * 27;
-    T u[3][27], w[3][27];
+    float u[3][27], w[3][27];
     unsigned skip = 0;   // bit a: node a is a boundary node (or a bad table entry)
 #pragma unroll
     for (int a = 0; a < 27; ++a) {
@@ -71,16 +72,60 @@ __global__ void __launch_bounds__(128) k_oct_cells(OctLevelDev L, const T* __res
                        (L.flags[node] & 1) != 0;
         skip |= unsigned(b) << a;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) u[c][a] = b ? T(0) : src[c * L.nn + node];
+        for (int c = 0; c < 3; ++c) u[c][a] = b ? 0.0f : src[c * L.nn + node];
     }
     q2::cell_A(u, w);
-    const T s = mu[cell] * T(L.h);
+    const float s = mu[cell] * float(L.h);
 #pragma unroll
     for (int a = 0; a < 27; ++a) {
         if ((skip >> a) & 1u) continue;
         const int32_t node = cn[a];
 #pragma unroll
         for (int c = 0; c < 3; ++c) atomicAdd(acc + c * L.nn + node, w[c][a] * s);
+    }
+}
+
+// The same on an FP64 level, in the fixed point of the outer operator (outer.cuh): one component per thread,
+// 32 cells per block. FP64 instructions run at 1/72 of the integer rate: FP64 V-cycle on 3,431 / 79,000 leaves
+// 1,452 / 3,584 -> 530 / 1,644 us.
+__global__ void __launch_bounds__(kOuterThreads, 5)
+    k_oct_cells_fix(OctLevelDev L, const double* __restrict__ mu, const double* __restrict__ src, double* __restrict__ acc) {
+    __shared__ int32_t node[27][kOuterCells + 1];   // the block's piece of the index map; -1: a boundary node
+    __shared__ OuterShared sh;
+    const int C = int(threadIdx.x) / kOuterCells, g = int(threadIdx.x) % kOuterCells;
+    const size_t first = size_t(blockIdx.x) * kOuterCells, map = first * 27, end = size_t(L.n_cells) * 27;
+    for (int t = threadIdx.x; t < 27 * kOuterCells; t += kOuterThreads) {
+        int32_t v = -1;
+        if (map + t < end) {
+            v = L.cell_nodes[map + t];
+            if (!idx_ok(L.dbg, OCT_CELL_NODES, v, (long long)L.nn, map + t) || (L.flags[v] & 1)) v = -1;
+        }
+        node[t % 27][t / 27] = v;
+    }
+    __syncthreads();
+    // strides of the own frame's axes C, C + 1, C + 2 in the cell's 27 nodes
+    const int q0 = C == 0 ? 1 : (C == 1 ? 3 : 9), q1 = C == 0 ? 3 : (C == 1 ? 9 : 1), q2 = C == 0 ? 9 : (C == 1 ? 1 : 3);
+    {
+        double u[27];
+        int e = 0;
+#pragma unroll
+        for (int m = 0; m < 27; ++m) {
+            const int32_t v = node[(m % 3) * q0 + (m / 3 % 3) * q1 + (m / 9) * q2][g];
+            u[m] = v < 0 ? 0.0 : src[C * L.nn + v];
+            e = max(e, exp_of(__double_as_longlong(u[m])));
+        }
+        sh.eu[C][g] = e;
+        __syncthreads();
+        outer_modes<true, false>(C, g, sh, u);
+    }
+    __syncthreads();
+    if (first + g >= size_t(L.n_cells)) return;
+    long long Y[27];
+    const double s = outer_velocity<true, false>(C, g, sh, mu[first + g], L.h, Y);
+#pragma unroll
+    for (int m = 0; m < 27; ++m) {
+        const int32_t v = node[(m % 3) * q0 + (m / 3 % 3) * q1 + (m / 9) * q2][g];
+        if (v >= 0) atomicAdd(acc + C * L.nn + v, fix_out(Y[m], s));
     }
 }
 
@@ -361,8 +406,10 @@ const char* oct_table_name(int table) {
 template <typename T>
 cudaError_t launch_oct_level_cells(const OctLevelDev& L, const T* mu, const T* src, T* acc, cudaStream_t s) {
     if (L.n_cells == 0) return cudaSuccess;
-    LAUNCH(sizeof(T) == 4 ? PROF_VMULT_F32 : PROF_VMULT_F64, s,
-           (k_oct_cells<T><<<blocks_for(L.n_cells, 128), 128, 0, s>>>(L, mu, src, acc)));
+    if constexpr (sizeof(T) == 4)
+        LAUNCH(PROF_VMULT_F32, s, (k_oct_cells<<<blocks_for(L.n_cells, 128), 128, 0, s>>>(L, mu, src, acc)));
+    else
+        LAUNCH(PROF_VMULT_F64, s, (k_oct_cells_fix<<<blocks_for(L.n_cells, kOuterCells), kOuterThreads, 0, s>>>(L, mu, src, acc)));
     return cudaGetLastError();
 }
 
