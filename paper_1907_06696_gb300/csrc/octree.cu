@@ -235,42 +235,30 @@ __global__ void k_oct_copy_from_level(size_t n, const int32_t* __restrict__ ai, 
 }
 
 // ---- active blocks with hanging-node constraints
-// A reference r read at position `at` of leaf_u / leaf_p is a node (r >= 0) or constraint -r-1.
-__device__ __forceinline__ double gather_u(const OctActiveDev& a, const double* src, int c, int32_t r, size_t at) {
-    if (r >= 0) {
-        if (!idx_ok(a.dbg, OCT_LEAF_U, r, (long long)a.nu_nodes, at)) return 0.0;
-        return a.ubnd[r] ? 0.0 : src[c * a.nu_nodes + r];
-    }
-    const long long k = -(long long)r - 1;
-    if (!idx_ok(a.dbg, OCT_LEAF_U, k, (long long)a.n_ucon, at)) return 0.0;
+// A reference r read from leaf_u / leaf_p is a node (r >= 0) or constraint -r-1. The terms of a constraint are
+// loaded together, unused ones (-1) as zero: their addresses do not depend on one another.
+__device__ __forceinline__ double con_gather_u(const OctActiveDev& a, const double* src, int c, long long k) {
     const int32_t* nd = a.ucon_node + size_t(k) * kOctUCon;
     const double* wt = a.ucon_w + size_t(k) * kOctUCon;
     double v = 0.0;
-#pragma unroll 1
+#pragma unroll
     for (int t = 0; t < kOctUCon; ++t) {
         const int32_t node = nd[t];
-        if (node < 0) break;
-        if (!idx_ok(a.dbg, OCT_UCON_NODE, node, (long long)a.nu_nodes, size_t(k) * kOctUCon + t)) continue;
-        if (!a.ubnd[node]) v += wt[t] * src[c * a.nu_nodes + node];
+        const bool on = node >= 0 && idx_ok(a.dbg, OCT_UCON_NODE, node, (long long)a.nu_nodes, size_t(k) * kOctUCon + t);
+        const bool free = on && !a.ubnd[on ? node : 0];
+        const double x = src[c * a.nu_nodes + (on ? node : 0)];
+        if (free) v += wt[t] * x;
     }
     return v;
 }
-__device__ __forceinline__ void scatter_u(const OctActiveDev& a, double* dst, int c, int32_t r, double v, size_t at) {
-    if (r >= 0) {
-        if (!idx_ok(a.dbg, OCT_LEAF_U, r, (long long)a.nu_nodes, at)) return;
-        if (!a.ubnd[r]) atomicAdd(dst + c * a.nu_nodes + r, v);
-        return;
-    }
-    const long long k = -(long long)r - 1;
-    if (!idx_ok(a.dbg, OCT_LEAF_U, k, (long long)a.n_ucon, at)) return;
+__device__ __forceinline__ void con_scatter_u(const OctActiveDev& a, double* dst, int c, long long k, double v) {
     const int32_t* nd = a.ucon_node + size_t(k) * kOctUCon;
     const double* wt = a.ucon_w + size_t(k) * kOctUCon;
-#pragma unroll 1
+#pragma unroll
     for (int t = 0; t < kOctUCon; ++t) {
         const int32_t node = nd[t];
-        if (node < 0) break;
-        if (!idx_ok(a.dbg, OCT_UCON_NODE, node, (long long)a.nu_nodes, size_t(k) * kOctUCon + t)) continue;
-        if (!a.ubnd[node]) atomicAdd(dst + c * a.nu_nodes + node, wt[t] * v);
+        const bool on = node >= 0 && idx_ok(a.dbg, OCT_UCON_NODE, node, (long long)a.nu_nodes, size_t(k) * kOctUCon + t);
+        if (on && !a.ubnd[node]) atomicAdd(dst + c * a.nu_nodes + node, wt[t] * v);
     }
 }
 __device__ __forceinline__ double gather_p(const OctActiveDev& a, const double* src, int32_t r, size_t at) {
@@ -280,11 +268,12 @@ __device__ __forceinline__ double gather_p(const OctActiveDev& a, const double* 
     const int32_t* nd = a.pcon_node + size_t(k) * kOctPCon;
     const double* wt = a.pcon_w + size_t(k) * kOctPCon;
     double v = 0.0;
-#pragma unroll 1
+#pragma unroll
     for (int t = 0; t < kOctPCon; ++t) {
-        if (nd[t] < 0) break;
-        if (!idx_ok(a.dbg, OCT_PCON_NODE, nd[t], (long long)a.np, size_t(k) * kOctPCon + t)) continue;
-        v += wt[t] * src[nd[t]];
+        const int32_t node = nd[t];
+        const bool on = node >= 0 && idx_ok(a.dbg, OCT_PCON_NODE, node, (long long)a.np, size_t(k) * kOctPCon + t);
+        const double x = src[on ? node : 0];
+        if (on) v += wt[t] * x;
     }
     return v;
 }
@@ -297,38 +286,73 @@ __device__ __forceinline__ void scatter_p(const OctActiveDev& a, double* dst, in
     if (!idx_ok(a.dbg, OCT_LEAF_P, k, (long long)a.n_pcon, at)) return;
     const int32_t* nd = a.pcon_node + size_t(k) * kOctPCon;
     const double* wt = a.pcon_w + size_t(k) * kOctPCon;
-#pragma unroll 1
+#pragma unroll
     for (int t = 0; t < kOctPCon; ++t) {
-        if (nd[t] < 0) break;
-        if (!idx_ok(a.dbg, OCT_PCON_NODE, nd[t], (long long)a.np, size_t(k) * kOctPCon + t)) continue;
-        atomicAdd(dst + nd[t], wt[t] * v);
+        const int32_t node = nd[t];
+        if (node >= 0 && idx_ok(a.dbg, OCT_PCON_NODE, node, (long long)a.np, size_t(k) * kOctPCon + t))
+            atomicAdd(dst + node, wt[t] * v);
     }
 }
 
+// The block's references to velocity nodes: a node, kNoRow (a Dirichlet row, a bad entry or no leaf: reads 0,
+// writes nothing) or constraint -r-1; and the places of the constrained ones, at * kOuterCells + leaf.
+constexpr int32_t kNoRow = INT32_MIN;
+struct OctRefs {
+    int32_t u[27][kOuterCells + 1];
+    uint16_t hang[27 * kOuterCells];
+    int n_hang;
+};
+
 // One velocity component per thread, 32 leaves per CTA, in the fixed-point arithmetic of the uniform
 // outer operator (outer.cuh): warp c gathers component c through the leaf's references and scatters it the same
-// way. 3,431 leaves: 168 -> 133 us (one thread per leaf with FP64 instructions in the
-// modes); 79,080 leaves: 385 -> 383 us, bound by the hanging nodes, whose terms every lane waits for.
+// way. A hanging node's value is a chain of dependent loads (constraint, nodes, Dirichlet flags, values). Taken
+// where the leaf comes to it, the whole warp waits for the chain at each of the 27 nodes, so the block first
+// lists its hanging nodes, one lane takes one of them, and the values go through the (then unused) space of
+// the modes in shared memory. 79,080 leaves (with the
+// clearing of the output): 406 -> 170 us, of which the uniform operator on as many cells takes some 60.
 template <bool DO_A, bool DO_BT, bool DO_B>
 __global__ void __launch_bounds__(kOuterThreads, 5) k_oct_active(OctActiveDev a, const double* __restrict__ src_u,
                                                                  const double* __restrict__ src_p, double* __restrict__ dst_u,
                                                                  double* __restrict__ dst_p) {
     __shared__ OuterShared sh;
+    __shared__ OctRefs ref;
     const int C = int(threadIdx.x) / kOuterCells, g = int(threadIdx.x) % kOuterCells;
     const int leaf = int(blockIdx.x) * kOuterCells + g;
     const bool valid = leaf < a.n_leaves;
-    const int32_t* ru = a.leaf_u + size_t(valid ? leaf : 0) * 27;
     const int32_t* rp = a.leaf_p + size_t(valid ? leaf : 0) * 8;
     // strides of the own frame's axes in the leaf's 27 nodes
     const int q0 = C == 0 ? 1 : (C == 1 ? 3 : 9), q1 = C == 0 ? 3 : (C == 1 ? 9 : 1), q2 = C == 0 ? 9 : (C == 1 ? 1 : 3);
+    if (threadIdx.x == 0) ref.n_hang = 0;
+    __syncthreads();
+    const size_t map = size_t(blockIdx.x) * kOuterCells * 27, end = size_t(a.n_leaves) * 27;
+#pragma unroll
+    for (int t = threadIdx.x; t < 27 * kOuterCells; t += kOuterThreads) {
+        int32_t r = kNoRow;
+        if (map + t < end) {
+            r = a.leaf_u[map + t];
+            const bool ok = r >= 0 ? idx_ok(a.dbg, OCT_LEAF_U, r, (long long)a.nu_nodes, map + t)
+                                   : idx_ok(a.dbg, OCT_LEAF_U, -(long long)r - 1, (long long)a.n_ucon, map + t);
+            if (!ok || (r >= 0 && a.ubnd[r])) r = kNoRow;
+        }
+        ref.u[t % 27][t / 27] = r;
+        if (r < 0 && r != kNoRow) ref.hang[atomicAdd(&ref.n_hang, 1)] = uint16_t(t % 27 * kOuterCells + t / 27);
+    }
+    __syncthreads();
+    const int n_hang = ref.n_hang;
     {
         double T[27];
         if (DO_A || DO_B) {
+            for (int i = g; i < n_hang; i += kOuterCells) {
+                const int at = ref.hang[i] / kOuterCells, l = ref.hang[i] % kOuterCells;
+                sh.U[C][at][l] = __double_as_longlong(con_gather_u(a, src_u, C, -(long long)ref.u[at][l] - 1));
+            }
+            __syncwarp();
             int e = 0;
 #pragma unroll
             for (int m = 0; m < 27; ++m) {
                 const int at = (m % 3) * q0 + (m / 3 % 3) * q1 + (m / 9) * q2;
-                T[m] = valid ? gather_u(a, src_u, C, ru[at], size_t(leaf) * 27 + at) : 0.0;
+                const int32_t r = ref.u[at][g];
+                T[m] = r >= 0 ? src_u[C * a.nu_nodes + r] : (r == kNoRow ? 0.0 : __longlong_as_double(sh.U[C][at][g]));
                 e = max(e, exp_of(__double_as_longlong(T[m])));
             }
             sh.eu[C][g] = e;
@@ -346,9 +370,8 @@ __global__ void __launch_bounds__(kOuterThreads, 5) k_oct_active(OctActiveDev a,
         outer_modes<DO_A || DO_B, DO_BT>(C, g, sh, T);
     }
     __syncthreads();
-    if (!valid) return;
-    const double h = ldexp(1.0, -int(a.level[leaf]));
-    if (DO_B) {
+    const double h = valid ? ldexp(1.0, -int(a.level[leaf])) : 1.0;
+    if (DO_B && valid) {
         long long b[8];
         const double s = outer_pressure(C, g, sh, h, b);
         const int v1 = 1 << C, v6 = 7 - v1;   // as in outer_phase2: each vertex by one warp
@@ -361,11 +384,20 @@ __global__ void __launch_bounds__(kOuterThreads, 5) k_oct_active(OctActiveDev a,
     }
     if (DO_A || DO_BT) {
         long long Y[27];
-        const double s = outer_velocity<DO_A, DO_BT>(C, g, sh, a.mu[leaf], h, Y);
+        const double s = outer_velocity<DO_A, DO_BT>(C, g, sh, valid ? a.mu[leaf] : 1.0, h, Y);
+        __syncthreads();   // every warp has read the modes
 #pragma unroll
         for (int m = 0; m < 27; ++m) {
             const int at = (m % 3) * q0 + (m / 3 % 3) * q1 + (m / 9) * q2;
-            scatter_u(a, dst_u, C, ru[at], fix_out(Y[m], s), size_t(leaf) * 27 + at);
+            const int32_t r = ref.u[at][g];
+            const double y = fix_out(Y[m], s);
+            if (r >= 0) atomicAdd(dst_u + C * a.nu_nodes + r, y);
+            else if (r != kNoRow) sh.U[C][at][g] = __double_as_longlong(y);
+        }
+        __syncwarp();
+        for (int i = g; i < n_hang; i += kOuterCells) {
+            const int at = ref.hang[i] / kOuterCells, l = ref.hang[i] % kOuterCells;
+            con_scatter_u(a, dst_u, C, -(long long)ref.u[at][l] - 1, __longlong_as_double(sh.U[C][at][l]));
         }
     }
 }
@@ -376,23 +408,19 @@ __global__ void k_oct_active_boundary(OctActiveDev a, const double* __restrict__
     for (int c = 0; c < 3; ++c) dst_u[c * a.nu_nodes + n] = src_u[c * a.nu_nodes + n];
 }
 
-__global__ void k_oct_mass_p(OctActiveDev a, const double* __restrict__ src, double* __restrict__ dst) {
-    const int leaf = blockIdx.x * blockDim.x + threadIdx.x;
-    if (leaf >= a.n_leaves) return;
-    const int32_t* rp = a.leaf_p + size_t(leaf) * 8;
+// M_p: one thread per vertex of a leaf, the element matrix (2, 1; 1, 2)/6 per axis by exchanges within the leaf's
+// 8 lanes. With it and k_oct_active a solve on 3,431 leaves took 97
+// instead of 128 ms (one thread per leaf, the 64 products of the matrix).
+__global__ void __launch_bounds__(256) k_oct_mass_p(OctActiveDev a, const double* __restrict__ src, double* __restrict__ dst) {
+    const size_t t = size_t(blockIdx.x) * blockDim.x + threadIdx.x, end = size_t(a.n_leaves) * 8;
+    const int32_t r = t < end ? a.leaf_p[t] : 0;
+    double p = t < end ? gather_p(a, src, r, t) * (1.0 / 216.0) : 0.0;
+#pragma unroll
+    for (int d = 1; d < 8; d <<= 1) p = 2.0 * p + __shfl_xor_sync(0xffffffffu, p, d);
+    if (t >= end) return;
+    const size_t leaf = t / 8;
     const double h = ldexp(1.0, -int(a.level[leaf]));
-    const double sc = h * h * h / a.mu[leaf];
-    double p[8];
-    for (int v = 0; v < 8; ++v) p[v] = gather_p(a, src, rp[v], size_t(leaf) * 8 + v);
-    for (int v = 0; v < 8; ++v) {
-        double o = 0.0;
-        for (int q = 0; q < 8; ++q) {
-            double m = 1.0;
-            for (int d = 0; d < 3; ++d) m *= (((v >> d) & 1) == ((q >> d) & 1)) ? (1.0 / 3.0) : (1.0 / 6.0);
-            o += m * p[q];
-        }
-        scatter_p(a, dst, rp[v], sc * o, size_t(leaf) * 8 + v);
-    }
+    scatter_p(a, dst, r, h * h * h / a.mu[leaf] * p, t);
 }
 
 }  // namespace
@@ -486,7 +514,7 @@ cudaError_t launch_oct_identity_rows(const OctActiveDev& a, const double* src_u,
 cudaError_t launch_oct_mass_p(const OctActiveDev& a, const double* src, double* dst, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(dst, 0, a.np * sizeof(double), s);
     if (e != cudaSuccess) return e;
-    LAUNCH(PROF_MASS_P, s, (k_oct_mass_p<<<blocks_for(a.n_leaves, 128), 128, 0, s>>>(a, src, dst)));
+    LAUNCH(PROF_MASS_P, s, (k_oct_mass_p<<<blocks_for(size_t(a.n_leaves) * 8, 256), 256, 0, s>>>(a, src, dst)));
     return cudaGetLastError();
 }
 
