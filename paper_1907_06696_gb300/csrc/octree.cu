@@ -155,6 +155,24 @@ __global__ void k_oct_dinv(OctLevelDev L, const double* __restrict__ diag, doubl
     for (int c = 0; c < 3; ++c) dinv[c * L.nn + n] = skip ? 0.0 : 1.0 / diag[c * L.nn + n];
 }
 
+// The parent's 27 nodes, -1 where the weight is 0 (or the entry is bad). All loads before the first use: a transfer
+// that looks at one node after the other waits for up to 27 pairs of dependent loads. FP32 V-cycle on 3,431 leaves
+// 339 -> 328 us, 79,080 leaves 681 -> 679 us. FP64 levels look at one node after the other: there the products
+// with weights of 0 cost more (1,660 -> 1,684 us on 79,080 leaves).
+template <typename T>
+__device__ __forceinline__ void parent_nodes(const OctLevelDev& C, uint32_t par, const T (&wx)[3], const T (&wy)[3],
+                                             const T (&wz)[3], int32_t (&node)[27]) {
+    const int32_t* cn = C.cell_nodes + size_t(par) * 27;
+#pragma unroll
+    for (int b = 0; b < 27; ++b) {
+        const bool on = wx[b % 3] != T(0) && wy[b / 3 % 3] != T(0) && wz[b / 9] != T(0);
+        node[b] = on ? cn[b] : -1;
+    }
+#pragma unroll
+    for (int b = 0; b < 27; ++b)
+        if (node[b] >= 0 && !idx_ok(C.dbg, OCT_CELL_NODES, node[b], (long long)C.nn, size_t(par) * 27 + b)) node[b] = -1;
+}
+
 template <typename T>
 __global__ void k_oct_prolongate(OctLevelDev F, OctLevelDev C, const T* __restrict__ coarse, T* __restrict__ fine,
                                  bool add) {
@@ -169,19 +187,33 @@ __global__ void k_oct_prolongate(OctLevelDev F, OctLevelDev C, const T* __restri
     const int p = F.pos[n], px = p % 5, py = (p / 5) % 5, pz = p / 25;
     T v[3] = {T(0), T(0), T(0)};
     if (idx_ok(F.dbg, OCT_PARENT, par, C.n_cells, n) && idx_ok(F.dbg, OCT_POS, p, 125, n)) {
-        const int32_t* cn = C.cell_nodes + size_t(par) * 27;
         T wx[3], wy[3], wz[3];
         q2_at(px, wx);
         q2_at(py, wy);
         q2_at(pz, wz);
+        if constexpr (sizeof(T) == 8) {
+            const int32_t* cn = C.cell_nodes + size_t(par) * 27;
 #pragma unroll
-        for (int b = 0; b < 27; ++b) {
-            const T w = wx[b % 3] * wy[b / 3 % 3] * wz[b / 9];
-            if (w == T(0)) continue;
-            const int32_t node = cn[b];
-            if (!idx_ok(C.dbg, OCT_CELL_NODES, node, (long long)C.nn, size_t(par) * 27 + b)) continue;
+            for (int b = 0; b < 27; ++b) {
+                const T w = wx[b % 3] * wy[b / 3 % 3] * wz[b / 9];
+                if (w == T(0)) continue;
+                const int32_t node = cn[b];
+                if (!idx_ok(C.dbg, OCT_CELL_NODES, node, (long long)C.nn, size_t(par) * 27 + b)) continue;
 #pragma unroll
-            for (int c = 0; c < 3; ++c) v[c] += w * coarse[c * C.nn + node];
+                for (int c = 0; c < 3; ++c) v[c] += w * coarse[c * C.nn + node];
+            }
+        } else {
+            int32_t node[27];
+            parent_nodes(C, par, wx, wy, wz, node);
+#pragma unroll
+            for (int b = 0; b < 27; ++b) {
+                const T w = wx[b % 3] * wy[b / 3 % 3] * wz[b / 9];
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const T x = node[b] >= 0 ? coarse[c * C.nn + node[b]] : T(0);
+                    v[c] += w * x;
+                }
+            }
         }
     }
     for (int c = 0; c < 3; ++c) fine[c * F.nn + n] = (add ? fine[c * F.nn + n] : T(0)) + v[c];
@@ -194,21 +226,39 @@ __global__ void k_oct_restrict_add(OctLevelDev F, OctLevelDev C, const T* __rest
     const uint32_t par = F.parent[n];
     const int p = F.pos[n], px = p % 5, py = (p / 5) % 5, pz = p / 25;
     if (!idx_ok(F.dbg, OCT_PARENT, par, C.n_cells, n) || !idx_ok(F.dbg, OCT_POS, p, 125, n)) return;
-    const int32_t* cn = C.cell_nodes + size_t(par) * 27;
     const T f[3] = {fine[n], fine[F.nn + n], fine[2 * F.nn + n]};
     T wx[3], wy[3], wz[3];
     q2_at(px, wx);
     q2_at(py, wy);
     q2_at(pz, wz);
+    if constexpr (sizeof(T) == 8) {
+        const int32_t* cn = C.cell_nodes + size_t(par) * 27;
 #pragma unroll
-    for (int b = 0; b < 27; ++b) {
-        const T w = wx[b % 3] * wy[b / 3 % 3] * wz[b / 9];
-        if (w == T(0)) continue;
-        const int32_t node = cn[b];
-        if (!idx_ok(C.dbg, OCT_CELL_NODES, node, (long long)C.nn, size_t(par) * 27 + b)) continue;
-        if (C.flags[node] & 1) continue;
+        for (int b = 0; b < 27; ++b) {
+            const T w = wx[b % 3] * wy[b / 3 % 3] * wz[b / 9];
+            if (w == T(0)) continue;
+            const int32_t node = cn[b];
+            if (!idx_ok(C.dbg, OCT_CELL_NODES, node, (long long)C.nn, size_t(par) * 27 + b)) continue;
+            if (C.flags[node] & 1) continue;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) atomicAdd(coarse + c * C.nn + node, w * f[c]);
+            for (int c = 0; c < 3; ++c) atomicAdd(coarse + c * C.nn + node, w * f[c]);
+        }
+    } else {
+        int32_t node[27];
+        parent_nodes(C, par, wx, wy, wz, node);
+        uint32_t skip = 0;
+#pragma unroll
+        for (int b = 0; b < 27; ++b) {
+            const unsigned flag = node[b] >= 0 ? C.flags[node[b]] : 1u;
+            skip |= (flag & 1u) << b;
+        }
+#pragma unroll
+        for (int b = 0; b < 27; ++b) {
+            if ((skip >> b) & 1u) continue;
+            const T w = wx[b % 3] * wy[b / 3 % 3] * wz[b / 9];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) atomicAdd(coarse + c * C.nn + node[b], w * f[c]);
+        }
     }
 }
 
