@@ -2047,9 +2047,14 @@ stokes_status oct_setup_impl(const stokes_octree* mesh, const stokes_mu* mu, con
             std::copy(H.leaf_u.begin() + o * 27, H.leaf_u.begin() + o * 27 + 27, zu.begin() + n * 27);
             std::copy(H.leaf_p.begin() + o * 8, H.leaf_p.begin() + o * 8 + 8, zp.begin() + n * 8);
         }
+        for (int32_t& r : zu)
+            if (r >= 0 && H.ubnd[r]) r = kOctNoRow;
+        std::vector<int32_t> un_free(H.ucon_node);
+        for (int32_t& r : un_free)
+            if (r >= 0 && H.ubnd[r]) r = -1;
         CKS(upload(c, &lu, zu, s));
         CKS(upload(c, &lp, zp, s));
-        CKS(upload(c, &un, H.ucon_node, s));
+        CKS(upload(c, &un, un_free, s));
         CKS(upload(c, &uw, H.ucon_w, s));
         CKS(upload(c, &pn, H.pcon_node, s));
         CKS(upload(c, &pw, H.pcon_w, s));

@@ -285,8 +285,9 @@ __global__ void k_oct_copy_from_level(size_t n, const int32_t* __restrict__ ai, 
 }
 
 // ---- active blocks with hanging-node constraints
-// A reference r read from leaf_u / leaf_p is a node (r >= 0) or constraint -r-1. The terms of a constraint are
-// loaded together, unused ones (-1) as zero: their addresses do not depend on one another.
+// A reference r read from leaf_u / leaf_p is a node (r >= 0), constraint -r-1 or (velocity) kOctNoRow. The terms of a
+// constraint are loaded together, unused ones (-1: no term, or a Dirichlet row) as zero: their addresses do
+// not depend on one another.
 __device__ __forceinline__ double con_gather_u(const OctActiveDev& a, const double* src, int c, long long k) {
     const int32_t* nd = a.ucon_node + size_t(k) * kOctUCon;
     const double* wt = a.ucon_w + size_t(k) * kOctUCon;
@@ -295,9 +296,8 @@ __device__ __forceinline__ double con_gather_u(const OctActiveDev& a, const doub
     for (int t = 0; t < kOctUCon; ++t) {
         const int32_t node = nd[t];
         const bool on = node >= 0 && idx_ok(a.dbg, OCT_UCON_NODE, node, (long long)a.nu_nodes, size_t(k) * kOctUCon + t);
-        const bool free = on && !a.ubnd[on ? node : 0];
         const double x = src[c * a.nu_nodes + (on ? node : 0)];
-        if (free) v += wt[t] * x;
+        if (on) v += wt[t] * x;
     }
     return v;
 }
@@ -308,7 +308,7 @@ __device__ __forceinline__ void con_scatter_u(const OctActiveDev& a, double* dst
     for (int t = 0; t < kOctUCon; ++t) {
         const int32_t node = nd[t];
         const bool on = node >= 0 && idx_ok(a.dbg, OCT_UCON_NODE, node, (long long)a.nu_nodes, size_t(k) * kOctUCon + t);
-        if (on && !a.ubnd[node]) atomicAdd(dst + c * a.nu_nodes + node, wt[t] * v);
+        if (on) atomicAdd(dst + c * a.nu_nodes + node, wt[t] * v);
     }
 }
 __device__ __forceinline__ double gather_p(const OctActiveDev& a, const double* src, int32_t r, size_t at) {
@@ -344,9 +344,7 @@ __device__ __forceinline__ void scatter_p(const OctActiveDev& a, double* dst, in
     }
 }
 
-// The block's references to velocity nodes: a node, kNoRow (a Dirichlet row, a bad entry or no leaf: reads 0,
-// writes nothing) or constraint -r-1; and the places of the constrained ones, at * kOuterCells + leaf.
-constexpr int32_t kNoRow = INT32_MIN;
+// The block's references to velocity nodes, and the places of the constrained ones, at * kOuterCells + leaf.
 struct OctRefs {
     int32_t u[27][kOuterCells + 1];
     uint16_t hang[27 * kOuterCells];
@@ -355,20 +353,24 @@ struct OctRefs {
 
 // One velocity component per thread, 32 leaves per CTA, in the fixed-point arithmetic of the uniform
 // outer operator (outer.cuh): warp c gathers component c through the leaf's references and scatters it the same
-// way. A hanging node's value is a chain of dependent loads (constraint, nodes, Dirichlet flags, values). Taken
+// way. A hanging node's value is a chain of dependent loads (constraint, nodes, values). Taken
 // where the leaf comes to it, the whole warp waits for the chain at each of the 27 nodes, so the block first
 // lists its hanging nodes, one lane takes one of them, and the values go through the (then unused) space of
-// the modes in shared memory. 79,080 leaves (with the
-// clearing of the output): 406 -> 170 us, of which the uniform operator on as many cells takes some 60.
-template <bool DO_A, bool DO_BT, bool DO_B>
-__global__ void __launch_bounds__(kOuterThreads, 5) k_oct_active(OctActiveDev a, const double* __restrict__ src_u,
-                                                                 const double* __restrict__ src_p, double* __restrict__ dst_u,
-                                                                 double* __restrict__ dst_p) {
+// the modes in shared memory. 79,080 leaves (with the clearing of the output): 406 -> 170 us, of which the uniform
+// operator on as many cells takes some 60.
+// On meshes of at most one block per SM the time is that of the block with the most hanging nodes (up to 600,
+// 20 rounds of 32 lanes): there GROUPS - 1 more warps per component take part in those rounds alone. Stokes operator on 3,431
+// leaves 49.2 -> 32.8 us, with the Dirichlet flags folded into the tables; that alone on 79,080 leaves 149 -> 132 us.
+template <bool DO_A, bool DO_BT, bool DO_B, int GROUPS>
+__global__ void __launch_bounds__(kOuterThreads * GROUPS, GROUPS == 1 ? 5 : 1)
+    k_oct_active(OctActiveDev a, const double* __restrict__ src_u, const double* __restrict__ src_p, double* __restrict__ dst_u,
+                 double* __restrict__ dst_p) {
     __shared__ OuterShared sh;
     __shared__ OctRefs ref;
-    const int C = int(threadIdx.x) / kOuterCells, g = int(threadIdx.x) % kOuterCells;
+    const int C = int(threadIdx.x) / kOuterCells % 3, g = int(threadIdx.x) % kOuterCells;
+    const int group = int(threadIdx.x) / kOuterThreads;
     const int leaf = int(blockIdx.x) * kOuterCells + g;
-    const bool valid = leaf < a.n_leaves;
+    const bool main = GROUPS == 1 || group == 0, valid = main && leaf < a.n_leaves;
     const int32_t* rp = a.leaf_p + size_t(valid ? leaf : 0) * 8;
     // strides of the own frame's axes in the leaf's 27 nodes
     const int q0 = C == 0 ? 1 : (C == 1 ? 3 : 9), q1 = C == 0 ? 3 : (C == 1 ? 9 : 1), q2 = C == 0 ? 9 : (C == 1 ? 1 : 3);
@@ -376,38 +378,41 @@ __global__ void __launch_bounds__(kOuterThreads, 5) k_oct_active(OctActiveDev a,
     __syncthreads();
     const size_t map = size_t(blockIdx.x) * kOuterCells * 27, end = size_t(a.n_leaves) * 27;
 #pragma unroll
-    for (int t = threadIdx.x; t < 27 * kOuterCells; t += kOuterThreads) {
-        int32_t r = kNoRow;
+    for (int t = threadIdx.x; t < 27 * kOuterCells; t += kOuterThreads * GROUPS) {
+        int32_t r = kOctNoRow;
         if (map + t < end) {
             r = a.leaf_u[map + t];
-            const bool ok = r >= 0 ? idx_ok(a.dbg, OCT_LEAF_U, r, (long long)a.nu_nodes, map + t)
-                                   : idx_ok(a.dbg, OCT_LEAF_U, -(long long)r - 1, (long long)a.n_ucon, map + t);
-            if (!ok || (r >= 0 && a.ubnd[r])) r = kNoRow;
+            if (r != kOctNoRow && !(r >= 0 ? idx_ok(a.dbg, OCT_LEAF_U, r, (long long)a.nu_nodes, map + t)
+                                           : idx_ok(a.dbg, OCT_LEAF_U, -(long long)r - 1, (long long)a.n_ucon, map + t)))
+                r = kOctNoRow;
         }
         ref.u[t % 27][t / 27] = r;
-        if (r < 0 && r != kNoRow) ref.hang[atomicAdd(&ref.n_hang, 1)] = uint16_t(t % 27 * kOuterCells + t / 27);
+        if (r < 0 && r != kOctNoRow) ref.hang[atomicAdd(&ref.n_hang, 1)] = uint16_t(t % 27 * kOuterCells + t / 27);
     }
     __syncthreads();
     const int n_hang = ref.n_hang;
     {
         double T[27];
         if (DO_A || DO_B) {
-            for (int i = g; i < n_hang; i += kOuterCells) {
+            for (int i = g + kOuterCells * group; i < n_hang; i += kOuterCells * GROUPS) {
                 const int at = ref.hang[i] / kOuterCells, l = ref.hang[i] % kOuterCells;
                 sh.U[C][at][l] = __double_as_longlong(con_gather_u(a, src_u, C, -(long long)ref.u[at][l] - 1));
             }
-            __syncwarp();
-            int e = 0;
+            if (GROUPS == 1) __syncwarp();
+            else __syncthreads();
+            if (main) {
+                int e = 0;
 #pragma unroll
-            for (int m = 0; m < 27; ++m) {
-                const int at = (m % 3) * q0 + (m / 3 % 3) * q1 + (m / 9) * q2;
-                const int32_t r = ref.u[at][g];
-                T[m] = r >= 0 ? src_u[C * a.nu_nodes + r] : (r == kNoRow ? 0.0 : __longlong_as_double(sh.U[C][at][g]));
-                e = max(e, exp_of(__double_as_longlong(T[m])));
+                for (int m = 0; m < 27; ++m) {
+                    const int at = (m % 3) * q0 + (m / 3 % 3) * q1 + (m / 9) * q2;
+                    const int32_t r = ref.u[at][g];
+                    T[m] = r >= 0 ? src_u[C * a.nu_nodes + r] : (r == kOctNoRow ? 0.0 : __longlong_as_double(sh.U[C][at][g]));
+                    e = max(e, exp_of(__double_as_longlong(T[m])));
+                }
+                sh.eu[C][g] = e;
             }
-            sh.eu[C][g] = e;
         }
-        if (DO_BT) {
+        if (DO_BT && main) {
             int e = 0;
             for (int v = C; v < 8; v += 3) {
                 const long long b = __double_as_longlong(valid ? gather_p(a, src_p, rp[v], size_t(leaf) * 8 + v) : 0.0);
@@ -417,7 +422,7 @@ __global__ void __launch_bounds__(kOuterThreads, 5) k_oct_active(OctActiveDev a,
             sh.ep[C][g] = e;
         }
         __syncthreads();
-        outer_modes<DO_A || DO_B, DO_BT>(C, g, sh, T);
+        if (main) outer_modes<DO_A || DO_B, DO_BT>(C, g, sh, T);
     }
     __syncthreads();
     const double h = valid ? ldexp(1.0, -int(a.level[leaf])) : 1.0;
@@ -434,18 +439,22 @@ __global__ void __launch_bounds__(kOuterThreads, 5) k_oct_active(OctActiveDev a,
     }
     if (DO_A || DO_BT) {
         long long Y[27];
-        const double s = outer_velocity<DO_A, DO_BT>(C, g, sh, valid ? a.mu[leaf] : 1.0, h, Y);
+        double s = 0.0;
+        if (main) s = outer_velocity<DO_A, DO_BT>(C, g, sh, valid ? a.mu[leaf] : 1.0, h, Y);
         __syncthreads();   // every warp has read the modes
+        if (main) {
 #pragma unroll
-        for (int m = 0; m < 27; ++m) {
-            const int at = (m % 3) * q0 + (m / 3 % 3) * q1 + (m / 9) * q2;
-            const int32_t r = ref.u[at][g];
-            const double y = fix_out(Y[m], s);
-            if (r >= 0) atomicAdd(dst_u + C * a.nu_nodes + r, y);
-            else if (r != kNoRow) sh.U[C][at][g] = __double_as_longlong(y);
+            for (int m = 0; m < 27; ++m) {
+                const int at = (m % 3) * q0 + (m / 3 % 3) * q1 + (m / 9) * q2;
+                const int32_t r = ref.u[at][g];
+                const double y = fix_out(Y[m], s);
+                if (r >= 0) atomicAdd(dst_u + C * a.nu_nodes + r, y);
+                else if (r != kOctNoRow) sh.U[C][at][g] = __double_as_longlong(y);
+            }
         }
-        __syncwarp();
-        for (int i = g; i < n_hang; i += kOuterCells) {
+        if (GROUPS == 1) __syncwarp();
+        else __syncthreads();
+        for (int i = g + kOuterCells * group; i < n_hang; i += kOuterCells * GROUPS) {
             const int at = ref.hang[i] / kOuterCells, l = ref.hang[i] % kOuterCells;
             con_scatter_u(a, dst_u, C, -(long long)ref.u[at][l] - 1, __longlong_as_double(sh.U[C][at][l]));
         }
@@ -540,17 +549,31 @@ cudaError_t launch_oct_copy_from_level(size_t n_copy, const int32_t* active_idx,
     return cudaGetLastError();
 }
 
+namespace {
+
+template <bool DO_A, bool DO_BT, bool DO_B>
+void launch_active(int cls, const OctActiveDev& a, const double* src_u, const double* src_p, double* dst_u, double* dst_p,
+                   cudaStream_t s) {
+    constexpr int kWide = 4, kSms = 152;
+    const unsigned n = blocks_for(a.n_leaves, kOuterCells);
+    if (n <= kSms)
+        LAUNCH(cls, s, (k_oct_active<DO_A, DO_BT, DO_B, kWide><<<n, kWide * kOuterThreads, 0, s>>>(a, src_u, src_p, dst_u, dst_p)));
+    else
+        LAUNCH(cls, s, (k_oct_active<DO_A, DO_BT, DO_B, 1><<<n, kOuterThreads, 0, s>>>(a, src_u, src_p, dst_u, dst_p)));
+}
+
+}  // namespace
+
 cudaError_t launch_oct_active(const OctActiveDev& a, const double* src_u, const double* src_p, double* dst_u,
                               double* dst_p, bool do_a, bool do_bt, bool do_b, cudaStream_t s) {
     cudaError_t e;
     if ((do_a || do_bt) && (e = cudaMemsetAsync(dst_u, 0, 3 * a.nu_nodes * sizeof(double), s)) != cudaSuccess) return e;
     if (do_b && (e = cudaMemsetAsync(dst_p, 0, a.np * sizeof(double), s)) != cudaSuccess) return e;
-    const unsigned g = blocks_for(a.n_leaves, kOuterCells);
     const int cls = do_a ? PROF_STOKES_F64 : (do_bt ? PROF_BT_F64 : PROF_STOKES_F64);
-    if (do_a && do_bt && do_b) LAUNCH(cls, s, (k_oct_active<true, true, true><<<g, kOuterThreads, 0, s>>>(a, src_u, src_p, dst_u, dst_p)));
-    else if (do_a && !do_bt && !do_b) LAUNCH(cls, s, (k_oct_active<true, false, false><<<g, kOuterThreads, 0, s>>>(a, src_u, src_p, dst_u, dst_p)));
-    else if (!do_a && do_bt && !do_b) LAUNCH(cls, s, (k_oct_active<false, true, false><<<g, kOuterThreads, 0, s>>>(a, src_u, src_p, dst_u, dst_p)));
-    else if (!do_a && !do_bt && do_b) LAUNCH(cls, s, (k_oct_active<false, false, true><<<g, kOuterThreads, 0, s>>>(a, src_u, src_p, dst_u, dst_p)));
+    if (do_a && do_bt && do_b) launch_active<true, true, true>(cls, a, src_u, src_p, dst_u, dst_p, s);
+    else if (do_a && !do_bt && !do_b) launch_active<true, false, false>(cls, a, src_u, src_p, dst_u, dst_p, s);
+    else if (!do_a && do_bt && !do_b) launch_active<false, true, false>(cls, a, src_u, src_p, dst_u, dst_p, s);
+    else if (!do_a && !do_bt && do_b) launch_active<false, false, true>(cls, a, src_u, src_p, dst_u, dst_p, s);
     else return cudaErrorInvalidValue;
     if (do_a) LAUNCH(cls, s, (k_oct_active_boundary<<<blocks_for(a.nu_nodes, 256), 256, 0, s>>>(a, src_u, dst_u)));
     return cudaGetLastError();

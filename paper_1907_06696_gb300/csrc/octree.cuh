@@ -131,6 +131,9 @@ struct OctLevelDev {
     OctDebug dbg;
 };
 
+// In the device tables the Dirichlet rows are no references: kOctNoRow in leaf_u (reads 0, writes nothing), -1 in
+// ucon_node.
+constexpr int32_t kOctNoRow = INT32_MIN;
 struct OctActiveDev {
     int n_leaves = 0;
     size_t nu_nodes = 0, np = 0;
