@@ -56,9 +56,12 @@ __device__ __forceinline__ bool idx_ok(const OctDebug& d, int t, long long v, lo
 #endif
 }
 
-// acc += A_l src over the cells of an FP32 level, one thread per cell. (Three threads per cell, one component
-// each, measured slower: FP32 V-cycle on 79,000 leaves 680 -> 732 us.)
-__global__ void __launch_bounds__(128) k_oct_cells(OctLevelDev L, const float* __restrict__ mu, const float* __restrict__ src,
+// acc += A_l src over the cells of an FP32 level, one thread per cell. Blocks of 64: the gathers and atomic adds of a
+// block queue on its SM, and most levels have fewer blocks than the chip has SMs. V-cycle on 3,431 leaves 320 -> 297
+// us, 79,080 leaves 671 -> 654 us against blocks of 128; blocks of 32: 302 and 647 us. (Three threads per cell, one
+// component each: 328 -> 354 us and 679 -> 776 us with blocks of 128 before.)
+constexpr int kCellThreads = 64;
+__global__ void __launch_bounds__(kCellThreads) k_oct_cells(OctLevelDev L, const float* __restrict__ mu, const float* __restrict__ src,
                                                    float* __restrict__ acc) {
     const int cell = blockIdx.x * blockDim.x + threadIdx.x;
     if (cell >= L.n_cells) return;
@@ -494,7 +497,7 @@ template <typename T>
 cudaError_t launch_oct_level_cells(const OctLevelDev& L, const T* mu, const T* src, T* acc, cudaStream_t s) {
     if (L.n_cells == 0) return cudaSuccess;
     if constexpr (sizeof(T) == 4)
-        LAUNCH(PROF_VMULT_F32, s, (k_oct_cells<<<blocks_for(L.n_cells, 128), 128, 0, s>>>(L, mu, src, acc)));
+        LAUNCH(PROF_VMULT_F32, s, (k_oct_cells<<<blocks_for(L.n_cells, kCellThreads), kCellThreads, 0, s>>>(L, mu, src, acc)));
     else
         LAUNCH(PROF_VMULT_F64, s, (k_oct_cells_fix<<<blocks_for(L.n_cells, kOuterCells), kOuterThreads, 0, s>>>(L, mu, src, acc)));
     return cudaGetLastError();
