@@ -212,6 +212,7 @@ struct stokes_ctx {
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};   // [FP64, FP32]
     long long glaunches[2] = {0, 0};                 // kernel launches inside each graph
     int cell_block = 128;                            // threads per block of the cell kernel (autotuned)
+    bool cell_tuned = false;                         // FP32 levels use it once tuned, blocks of 32 before
     float *tune_x = nullptr, *tune_r = nullptr, *tune_b = nullptr;   // autotuner work (FP32, finest level)
     double* tune_up = nullptr;                                        // autotuner solution vector
     OctCtx* oct = nullptr;                           // set for octree meshes (stokes_setup_octree)
@@ -304,6 +305,14 @@ double tridiag_max_eig(const std::vector<double>& a, const std::vector<double>& 
 // - between them the cell kernel and vector passes.
 constexpr int kBlockMaxN = 16, kMarchMinN = 64;
 
+// Blocks of the cell kernel on FP32 levels unless tuned: with 32 threads its gathers and atomic adds spread over more
+// SMs (V-cycle 20^3 137 -> 131 us, 32^3 268 -> 264 us, 40^3 287 -> 273 us; product at 20^3 14.3 -> 12.1 us
+// against blocks of 128; 24^3 and 48^3 the same).
+template <typename T>
+int cell_threads(const stokes_ctx* c) {
+    return sizeof(T) == 4 && !c->cell_tuned ? 32 : c->cell_block;
+}
+
 template <typename T>
 int level_kernel(const stokes_ctx* c, int l) {
     const int k = c->opt.vmult_kernel;
@@ -314,7 +323,7 @@ int level_kernel(const stokes_ctx* c, int l) {
         if (n >= kMarchMinN) return kMarchKernel;
     }
     if (sizeof(T) == 4 && n <= kBlockMaxN) return 3;   // steps carried by the products (fused_smoother)
-    return c->cell_block;
+    return cell_threads<T>(c);
 }
 
 // The marching operator copies 16-byte units: 16-byte aligned vectors (the level's own are; a caller's
@@ -333,7 +342,7 @@ template <typename T>
 stokes_status vmult_level(stokes_ctx* c, int l, const T* src, T* dst, cudaStream_t s) {
     Level& L = c->lev[l];
     int k = level_kernel<T>(c, l);
-    if (k == kMarchKernel && !aligned16(src, dst)) k = c->cell_block;
+    if (k == kMarchKernel && !aligned16(src, dst)) k = cell_threads<T>(c);
     CK(launch_level_op<T>(k, L.g, L.planes, EPI_PLAIN, vecs<T>(L).mu, src, dst, nullptr, nullptr, nullptr, 0.0, 0.0,
                           slots<T>(L), vecs<T>(L).acc, s, &c->tc));
     return STOKES_OK;
@@ -345,7 +354,7 @@ stokes_status cheb_step(stokes_ctx* c, int l, const T* b, T* x, double c1, doubl
     Level& L = c->lev[l];
     LevelVecs<T>& v = vecs<T>(L);
     const int k = level_kernel<T>(c, l);
-    CK(launch_level_op<T>(k == kMarchKernel ? c->cell_block : k, L.g, L.planes, EPI_CHEB, v.mu, x, nullptr, b, v.dinv, v.d,
+    CK(launch_level_op<T>(k == kMarchKernel ? cell_threads<T>(c) : k, L.g, L.planes, EPI_CHEB, v.mu, x, nullptr, b, v.dinv, v.d,
                           c1, c2, slots<T>(L), v.acc, s, &c->tc));
     return STOKES_OK;
 }
@@ -2658,10 +2667,11 @@ stokes_status stokes_autotune(stokes_ctx* c, int what, void* stream, int* block_
     CK(cudaEventCreate(&e1));
     stokes_status st = STOKES_OK;
     // only the cell kernel has a block size
-    if ((what & 1) && c->opt.vmult_kernel == 0 && level_kernel<float>(c, c->L - 1) == c->cell_block) {
+    if ((what & 1) && c->opt.vmult_kernel == 0 && level_kernel<float>(c, c->L - 1) == cell_threads<float>(c)) {
         // threads per block of the cell kernel: the fastest FP32 level operator on the finest level
         float best = 1e30f;
         int best_bs = c->cell_block;
+        c->cell_tuned = true;
         for (int bs : {64, 128, 256}) {
             c->cell_block = bs;
             for (int it = 0; it < 2; ++it) st = vmult_level<float>(c, c->L - 1, c->tune_b, c->tune_r, s);

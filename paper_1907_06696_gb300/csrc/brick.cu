@@ -450,7 +450,10 @@ cudaError_t launch_cell(const BrickArgs<T>& a, T* acc, int bs, cudaStream_t s) {
     const int cls = sizeof(T) == 4 ? PROF_VMULT_F32 : PROF_VMULT_F64;
     // pair atomics need an 8-byte aligned accumulator (callers may pass offset views)
     const bool pairs = (reinterpret_cast<uintptr_t>(acc) & 7u) == 0;
-    if (bs == 64) {
+    if (bs == 32) {
+        if (pairs) LAUNCH(cls, s, (k_cell_atomic<T, 32, true><<<unsigned((cells + 31) / 32), 32, 0, s>>>(a, acc)));
+        else LAUNCH(cls, s, (k_cell_atomic<T, 32, false><<<unsigned((cells + 31) / 32), 32, 0, s>>>(a, acc)));
+    } else if (bs == 64) {
         if (pairs) LAUNCH(cls, s, (k_cell_atomic<T, 64, true><<<unsigned((cells + 63) / 64), 64, 0, s>>>(a, acc)));
         else LAUNCH(cls, s, (k_cell_atomic<T, 64, false><<<unsigned((cells + 63) / 64), 64, 0, s>>>(a, acc)));
     } else if (bs == 256) {
@@ -663,7 +666,7 @@ cudaError_t launch_level_op(int kernel, const LevelGeom& g, const PlaneLayout& L
             kernel = 128;   // no FP64 tensor-core path
         }
     }
-    if (kernel == 0 || kernel == kSplitKernel || kernel == 64 || kernel == 128 || kernel == 256)
+    if (kernel == 0 || kernel == kSplitKernel || kernel == 32 || kernel == 64 || kernel == 128 || kernel == 256)
         return launch_cell_epi<T>(a, epi, acc, g.n_u, kernel == 0 ? 128 : kernel, s);
     switch (epi) {
         case EPI_PLAIN: return launch_epi<T, EPI_PLAIN>(a, s);

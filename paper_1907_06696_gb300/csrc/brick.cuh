@@ -385,12 +385,12 @@ struct ChebGather {
     T c1, c2;
 };
 
-// acc += A x' with x' from the pending step g (kernel: 0, 64, 128, 256 the cell kernel's block
-// size, 3 the component-split kernel on FP32 levels).
+// acc += A x' with x' from the pending step g (kernel: 64, 128, 256 the cell kernel's block size, others
+// 128, 3 the component-split kernel on FP32 levels).
 template <typename T>
 cudaError_t launch_cell_cheb(int kernel, const LevelGeom& geo, const T* mu, const ChebGather<T>& g, T* acc,
                              cudaStream_t s);
-// acc += A src with the cell (kernel 0, 64, 128, 256) or component-split (3, FP32) operator.
+// acc += A src with the cell (kernel 0, 32, 64, 128, 256) or component-split (3, FP32) operator.
 template <typename T>
 cudaError_t launch_accumulate(int kernel, const LevelGeom& geo, const T* mu, const T* src, T* acc, cudaStream_t s);
 // The consumers with separate input and output (d, x) buffers (equal pointers: in place) and a
@@ -434,7 +434,7 @@ cudaError_t march_configure();   // shared-memory opt-in; once before any launch
 
 // A x with an epilogue (EPI_PLAIN: dst = A x; EPI_RESID: dst = b - A x;
 // EPI_CHEB: d = c1 d + c2 dinv (b - A x), src += d in place).
-// kernel 0, 64, 128, 256: one thread per cell (blocks of 128, 64, 128, 256 threads) with atomic
+// kernel 0, 32, 64, 128, 256: one thread per cell (blocks of 128, 32, 64, 128, 256 threads) with atomic
 //           adds into acc (n_u entries, zero on entry and on return) and a consumer kernel for the
 //           epilogue;
 // kernel 3: FP32: the cell kernel's accumulation with three threads per cell (one per output
