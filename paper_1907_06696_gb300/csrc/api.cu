@@ -297,9 +297,8 @@ double tridiag_max_eig(const std::vector<double>& a, const std::vector<double>& 
 // Level-operator selector for launch_level_op: 1 = brick kernel, 2 = tensor-core brick kernel,
 // 3 = component-split kernel (FP32 levels), else the cell kernel's block size. By default the smallest and the
 // largest FP32 levels take the operators with the epilogue in the same launch:
-// - at most kBlockMaxN cells per axis: blocks of 4 x 4 x 4 cells (block.cu). A degree-4 smoothing takes 24.7 / 26.0
-//   us at 8^3 / 16^3 (component-split kernel and vector passes 32.8 / 32.8 us); at 24^3 both take 41 us, at
-//   32^3 65.6 and 57.4 us: its blocks compute two cells for each that they own;
+// - at most kBlockMaxN cells per axis: blocks of 2 x 2 x 2 cells (block.cu). With the limit at 24 cells 20^3 takes 132
+//   instead of 125 us and 24^3 181 instead of 146: its blocks compute 27 cells for 8 that they own;
 // - from kMarchMinN up: tiles that march over layers (march.cu), 197 / 528 / 1,196 us at 64^3 / 96^3 / 128^3 (cell
 //   kernel and vector passes 208 / 702 / 1,624 us); below, the layers are too few to hide one layer's latency;
 // - between them the cell kernel and vector passes.

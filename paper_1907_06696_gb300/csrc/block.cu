@@ -2,14 +2,15 @@
 // one launch and without atomic adds: A x, b - A x, or the Jacobi-Chebyshev step of Section 2.2.1.
 //
 // On levels of a few thousand cells a launch costs more than its arithmetic, so a step is one launch and
-// the arithmetic is spread as thin as it goes: a block completes the nodes with local index 0 or 1 in 4 x 4 x 4 cells
-// and computes those cells and the ones before them along each axis (5 x 5 x 5, three threads per
-// cell, one per component). A thread transforms its component to the modes of q2_basis.cuh, leaves
+// the arithmetic is spread as thin as it goes: a block completes the nodes with local index 0 or 1 in 2 x 2 x 2 cells
+// and computes those cells and the ones before them along each axis (3 x 3 x 3, one warp per
+// component). A thread transforms its component to the modes of q2_basis.cuh, leaves
 // them in shared memory, takes the 24 that it needs of the other two, and leaves its 27 results there;
 // then a thread sums the results of up to 8 cells for four nodes and runs the epilogue, whose
 // operands it loaded first of all. The first step of a smoothing from zero, x = c0 dinv b, is formed where
-// it is gathered. A level's V-cycle takes 11 launches instead of 20: FP32 V-cycle at 8^3 150 -> 134 us, 12^3 113 -> 98 us,
-// product at 16^3 12.1 -> 10.0 us. Bound by latency: loads, two exchanges through shared memory, stores.
+// it is gathered. Bound by the instructions of the warps that share a scheduler (some 900 each), so the
+// smallest blocks are the fastest although they compute 27 cells for 8: with 4 x 4 x 4 cells and 12 warps the
+// FP32 V-cycle at 8^3 took 135 us, now 107; 12^3 100 -> 84, 16^3 181 -> 154 us.
 #include "brick.cuh"
 #include "prof.cuh"
 
@@ -25,11 +26,11 @@ namespace stk {
 
 namespace {
 
-constexpr int kOwn = 4, kSide = kOwn + 1;              // owned and computed cells per axis
-constexpr int kCells = kSide * kSide * kSide;          // 125
-constexpr int kLanes = 128;                            // threads per component
+constexpr int kOwn = 2, kSide = kOwn + 1;              // owned and computed cells per axis
+constexpr int kCells = kSide * kSide * kSide;          // 27
+constexpr int kLanes = 32;                             // threads per component
 constexpr int kBlockThreads = 3 * kLanes;
-static_assert(kBlockThreads == 2 * 3 * kOwn * kOwn * kOwn, "two threads per owned cell and component");
+static_assert(kBlockThreads >= 2 * 3 * kOwn * kOwn * kOwn, "two threads per owned cell and component");
 
 struct BlockArgs {
     int n, M;
@@ -59,7 +60,7 @@ __device__ __forceinline__ float node_sum(const float (&W)[3][27][kLanes], int c
 }
 
 template <int EPI, bool ZERO>
-__global__ void __launch_bounds__(kBlockThreads, 2) k_block(BlockArgs a) {
+__global__ void __launch_bounds__(kBlockThreads, 5) k_block(BlockArgs a) {
     __shared__ float W[3][27][kLanes];   // the cells' modes, then their results
     const int n = a.n, M = a.M, t = int(threadIdx.x);
     const int x0 = int(blockIdx.x) * kOwn, y0 = int(blockIdx.y) * kOwn, z0 = int(blockIdx.z) * kOwn;
@@ -67,7 +68,7 @@ __global__ void __launch_bounds__(kBlockThreads, 2) k_block(BlockArgs a) {
     const int k = t / (3 * kOwn * kOwn * kOwn), o = t % (3 * kOwn * kOwn * kOwn), oc = o / (kOwn * kOwn * kOwn);
     const int li = o % kOwn, lj = (o / kOwn) % kOwn, lk = (o / (kOwn * kOwn)) % kOwn;
     const int oi = x0 + li, oj = y0 + lj, ok = z0 + lk;
-    const bool own = oi < n && oj < n && ok < n && 2 * ok + k > 0;
+    const bool own = k < 2 && oi < n && oj < n && ok < n && 2 * ok + k > 0;
     const size_t obase = size_t(oc) * a.nodes + size_t(2 * oi) + size_t(M) * (size_t(2 * oj) + size_t(M) * size_t(2 * ok + k));
     bool live[4];
     float eb[4], ei[4], ed[4], ex[4];
