@@ -35,16 +35,12 @@ sys.path.insert(0, ROOT)
 
 METRIC = "vmult GDoF/s & %HBM peak; Stokes solve s to 1e-8 rel (FP32 vs FP64 GMG)"
 RTOL = 1e-8
-# Algorithmic flops per cell of the velocity operator A by sum factorisation as implemented
-# (multiply-add = 2 flops): 36 sweeps of 9 lines. Interpolations and their transposes (18
-# sweeps): 3 outputs x 3 MACs per line. Derivatives (9 sweeps): the outer outputs 3 MACs, the
-# middle one a difference times a constant (the derivative matrix at symmetric Gauss points is
-# antisymmetric, its centre 0), 2 flops. Transposed derivatives (9): 3 MACs, and a difference
-# and one MAC, 3 flops.
-A_FLOP_PER_CELL = 18 * 9 * 18 + 9 * 9 * (12 + 2) + 9 * 9 * (12 + 3)
-# Outer operator [A B^T; B 0]: B^T and B as tensor products of 3x2 moment matrices, 3
-# components x 114 MACs each.
-STOKES_FLOP_PER_CELL = A_FLOP_PER_CELL + 2 * (342 + 342)
+# Algorithmic flops per cell of the velocity operator A in the Legendre modes of each axis (an operation = 2
+# flops, as on the FMA pipe): transforms of 81 lines each way, 9 operations a line together, and about 230 products
+# of the diagonal and the component pairs.
+A_FLOP_PER_CELL = 2 * (81 * 9 + 230)
+# Outer operator [A B^T; B 0]: B^T and B in the same modes, about 300 operations.
+STOKES_FLOP_PER_CELL = A_FLOP_PER_CELL + 2 * 300
 
 
 def parse():
@@ -82,7 +78,7 @@ def parse():
     ap.add_argument("--vmult-kernel", type=int, default=None,
                     help="with --kernels: level operator (0 cell kernel, 1 brick, 2 tensor cores)")
     ap.add_argument("--outer-arith", type=int, default=None,
-                    help="with --kernels: outer operator (0 native FP64, 1 double-float, 2 tensor-core digit slices)")
+                    help="with --kernels: outer operator (0 and 1 fixed point, 2 tensor-core digit slices)")
     return ap.parse_args()
 
 
@@ -157,10 +153,9 @@ def peaks():
 # Sources that define each profiled kernel class (a recorded ncu traffic figure is used only
 # while these files are unchanged).
 KERNEL_SOURCES = {
-    "stokes_df64": ("q2_basis.cuh", "df64.cuh", "outer.cuh", "outer.cu"),
-    "stokes_df64_inst": ("q2_basis.cuh", "df64.cuh", "outer.cuh", "outer.cu"),
-    "stokes_fp64": ("q2_basis.cuh", "ops.cu"),
-    "vmult_A_fp32": ("q2_basis.cuh", "brick.cuh", "brick.cu"),
+    "stokes_fixed": ("q2_basis.cuh", "outer.cuh", "outer.cu"),
+    "stokes_fixed_inst": ("q2_basis.cuh", "outer.cuh", "outer.cu"),
+    "vmult_A_fp32": ("q2_basis.cuh", "brick.cuh", "march.cu"),
     "krylov_vec": ("krylov.cu", "vec.cu"),
 }
 
@@ -380,12 +375,12 @@ def run_ours(args):
     dopt = capi.stokes_default_options()
     line = {"metric": METRIC, "value": value, "unit": "GDoF/s", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
-            "vs_baseline": None, "dtype": "df64 outer (FP64 true residual) + f32 V-cycle", "data": "synthetic",
+            "vs_baseline": None, "dtype": "FP64-accurate fixed-point outer + f32 V-cycle", "data": "synthetic",
             "config": workload_config(prob, n_u, n_p),
             "impl_config": {"parallelism": "replicas" if world > 1 else "1 GPU", "cell_block": tuned_block,
                             "vmult_kernel": VMULT_KERNELS.get(dopt.vmult_kernel, dopt.vmult_kernel),
-                            "outer_arith": "double-float on FP32 pipes (~47-bit significand), restart and final "
-                                           "residuals native FP64" if dopt.outer_arith == 1 else "native FP64",
+                            "outer_arith": "64-bit fixed point on the integer pipes, Krylov basis in "
+                                           + ("double-float" if dopt.outer_arith == 1 else "FP64"),
                             "l2": "working set %.1f GB > L2 (no flush needed)" % (N * 8 * 103 / 1e9)},
             "solve": {"fp32_vcycle_s": ms / 1e3, "fp32_vcycle_iterations": its,
                       "fp32_true_rel_residual": true_res32},
@@ -581,29 +576,25 @@ def dominant_roofline(prof, dopt, cells, n_u, N, hbm, hbm_src, f32_peak, f64_pea
     if dom == "stokes_fp64":
         bytes_alg = (2 * N + cells) * 8
         fl = cells * STOKES_FLOP_PER_CELL
-        df = dopt.outer_arith == 1
-        r = {"kernel": "k_outer_df64<1,1,1> (outer [A B^T; B 0], double-float)" if df else
-                       "k_stokes_blocks<double,1,1,1> (outer [A B^T; B 0], FP64)",
+        r = {"kernel": "k_outer_fix<1,1,1> (outer [A B^T; B 0], 64-bit fixed point)",
              "bound": "hbm", "achieved": bytes_alg / (dms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
              "frac": bytes_alg / (dms / 1e3) / 1e9 / hbm,
-             "traffic": recorded_traffic("stokes_df64" if df else "stokes_fp64", workload),
+             "traffic": recorded_traffic("stokes_fixed", workload),
              "peak_note": hbm_src, "launch_ms": dms,
              "per_launch": "(2 (N_u + N_p) + cells) x 8 B = %d B (u, p read and written in FP64, cell viscosity)"
                            % bytes_alg}
-        alu_peak = f32_peak if df else f64_peak
+        alu_peak = f32_peak
         r["alu"] = {"method_flop_per_cell": STOKES_FLOP_PER_CELL, "achieved_gflops": fl / (dms / 1e3) / 1e9,
                     "peak_gflops": alu_peak * 1e3, "frac": fl / (dms / 1e3) / 1e9 / (alu_peak * 1e3),
-                    "peak_note": "of measured (%s probe, this run); the FP64 method flops %s"
-                                 % ("FFMA" if df else "DFMA",
-                                    "run as double-float on the FP32 pipes, several FP32 instructions each"
-                                    if df else "on the FP64 pipe")}
-        inst = recorded_traffic("stokes_df64_inst" if df else "stokes_fp64_inst", workload)
+                    "peak_note": "of measured (FFMA probe, this run); the method flops, run as "
+                                 "64-bit integer operations in the Legendre modes"}
+        inst = recorded_traffic("stokes_fixed_inst", workload)
         if inst:
             ips = inst / (dms / 1e3)
             r["issue"] = {"thread_inst_per_launch": inst, "frac": ips / (f32_peak / 2 * 1e12),
                           "note": "instructions per launch (ncu smsp__inst_executed.sum x 32) against the "
                                   "FFMA probe's instruction rate (FMA = 1 instruction): the issue efficiency "
-                                  "of the double-float code"}
+                                  "of the fixed-point code"}
         return r
     bytes_alg = (2 * n_u + cells) * 4
     return {"kernel": dom, "bound": "hbm", "achieved": bytes_alg / (dms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
@@ -639,7 +630,7 @@ def run_refinement(capi, si, torch, stream):
 def run_large(capi, si, torch, stream, hbm, hbm_src, name="cube128"):
     """The 128^3 configuration (16 sinkers, viscosity ratio 1e6, 8 levels): the standalone vmult with
     vectors far above L2 (the HBM figure) and one FP32-V-cycle FGMRES solve to 1e-8 with its true
-    residual from the native FP64 operator."""
+    residual from the FP64-accurate operator."""
     prob = si.workload(name)
     t0 = time.perf_counter()
     ctx = capi.stokes_setup_problem(prob, stream=stream)
@@ -659,7 +650,7 @@ def run_large(capi, si, torch, stream, hbm, hbm_src, name="cube128"):
              "iterations": info.iterations, "status": info.status,
              "true_rel_residual": info.rel_residual_true,
              "note": "first solve on the context (includes the V-cycle graph capture); true residual from the "
-                     "library's native FP64 operator"}
+                     "library's FP64-accurate operator"}
     ctx.close()
     del up
     torch.cuda.empty_cache()
@@ -787,7 +778,7 @@ def run_batch(args):
         seq[tag] = (e0.elapsed_time(e1), its)
     line = {"metric": METRIC, "value": ndof / (ms / 1e3) / 1e9, "unit": "GDoF/s", "n_gpus": 1, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
-            "vs_baseline": None, "dtype": "df64 outer (FP64 true residual) + f32 V-cycle", "data": "synthetic",
+            "vs_baseline": None, "dtype": "FP64-accurate fixed-point outer + f32 V-cycle", "data": "synthetic",
             "config": {"workload": args.workload, "problems": count,
                        "sizes": sorted(set(p.n for p in probs)), "total_dofs": ndof, "rtol": RTOL},
             "batch": {"fp32_batch_graphs_s": ms / 1e3, "iterations": [i.iterations for i in infos],

@@ -314,7 +314,7 @@ size_t stokes_size(const stokes_ctx* ctx, int level, int what);
  * M_p and Stokes blocks are FP64 and finest-level only. src and dst must not
  * overlap. Errors: EINVAL (bad level/block/precision, null pointer), ECUDA.
  * Octree contexts: level -1 is the active space with hanging-node constraints (FP64, all
- * blocks, native FP64 arithmetic); level li >= 0 is multigrid level li (block A, FP32 or
+ * blocks, FP64 or its accuracy); level li >= 0 is multigrid level li (block A, FP32 or
  * FP64; refinement-edge rows are ordinary rows). */
 stokes_status stokes_vmult(stokes_ctx* ctx, int level, int block, int prec,
                            const void* src_dev, void* dst_dev, void* stream);
@@ -336,7 +336,7 @@ stokes_status gmg_vcycle(stokes_ctx* ctx, int prec, const void* rhs_dev, void* x
  * block-diagonal P_D instead). rhs_dev = NULL uses the sinker right-hand side
  * [F; 0]. up_dev: in = initial guess, out = solution with zero-mean pressure.
  * Stops when the recurrence residual <= rtol ||b|| and the true residual
- * b - K x, recomputed with the native FP64 operator, is too; otherwise the
+ * b - K x, recomputed with the FP64-accurate operator, is too; otherwise the
  * method restarts from x (at most 10 times). The returned status follows that
  * true residual: OK only if it is <= rtol ||b||, NOT_CONVERGED otherwise
  * (max_it reached, or the restarts used up; up holds the last iterate and
@@ -444,7 +444,7 @@ stokes_status stokes_schur_inverse_noalloc(int n, const double* mu_dev, const do
 /* Kernel classes timed by stokes_profile: 0 velocity cell kernel FP32, 1 velocity
  * cell kernel FP64, 2 fused A+B^T+B cell kernel, 3 B^T cell kernel, 4 pressure mass
  * cell kernel, 5 transfers, 6 smoother / residual vector kernels, 7 Krylov vector
- * kernels, 8 coarse solve, 9 precision casts, 10 the outer operator applied in native FP64
+ * kernels, 8 coarse solve, 9 precision casts, 10 the outer operator applied for the solvers' residuals
  * for the solvers' restart and final residuals (uniform meshes). */
 #define STOKES_PROF_NCLASS 11
 /* enable = 1: record a CUDA event pair around every kernel launch the library

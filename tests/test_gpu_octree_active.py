@@ -1,5 +1,6 @@
 """Octree operators at the edges of their blocks, against the CPU oracle (oracle/adaptive.py): meshes with fewer
-leaves than a block of 32, without hanging nodes, and with a last block that is partly filled; the V-cycle on
+leaves than a block of 32, without hanging nodes, with a last block that is partly filled, and with
+more blocks than SMs; the V-cycle on
 hierarchies of two to five levels.
 
 Tolerances as in test_gpu_octree.py: blocks 1e-12 (same sums, another order), V-cycle FP64 1e-9, FP32 1e-4.
@@ -14,7 +15,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 # base level, coarsest level, sinkers, their levels
-MESHES = [(1, 1, 1, (2,)), (1, 1, 1, (3,)), (2, 1, 1, (2,)), (2, 2, 3, (3, 4)), (2, 1, 2, (5,))]
+MESHES = [(1, 1, 1, (2,)), (1, 1, 1, (3,)), (2, 1, 1, (2,)), (2, 2, 3, (3, 4)), (2, 1, 2, (5,)), (4, 2, 1, (6,))]
 
 
 @pytest.fixture(scope="module")
