@@ -118,18 +118,19 @@ typedef struct {
                                    tcgen05.mma with FP32 accumulation, exact because every partial sum
                                    is an integer below 2^24), recombined in double-float and written
                                    as FP64 with integer instructions; every other block and the
-                                   Krylov basis as in 1. Not yet the default: its speed is unmeasured. */
-    int vmult_kernel;           /* level operator of the V-cycle: 0 = one thread per cell with atomic adds
-                                   and a separate epilogue pass (default); 1 = brick-tiled, atomic-free
+                                   Krylov basis as in 1. Not the default: 832 us at 64^3 against 195 us for 1. */
+    int vmult_kernel;           /* level operator of the V-cycle: 0 = by level size (default): FP32 levels of at
+                                   most 16^3 cells in blocks of 2^3 cells and those from 64^3 up in tiles
+                                   that march over layers, both with the epilogue inside; between them
+                                   one thread per cell with atomic adds and a separate epilogue pass;
+                                   FP64 levels in 64-bit fixed point; 1 = brick-tiled, atomic-free
                                    and deterministic, epilogue fused; 2 = FP32 levels: the brick-tiled
                                    scatter of 1 with the cell products on the tensor cores (A_cell =
                                    mu_c h A_hat with 5400 A_hat exact in f16; each cell's values scaled
                                    by a power of two and split into two f16 terms, 22 significant bits;
                                    f32 accumulation), FP64 levels as 0; 3 = FP32 levels: three
                                    threads per cell, one per output component, cross derivatives
-                                   exchanged in shared memory (by default 0 uses it on the FP32
-                                   levels of at most 16^3 cells, where a level operator's time is
-                                   one thread's serial work), FP64 levels as 0 */
+                                   exchanged in shared memory, FP64 levels as 0 */
     int graphs;                 /* 1 = capture the V-cycle's level recursion once per precision as a CUDA
                                    graph and replay it on a library stream ordered with the caller's
                                    stream by events (default); 0 = launch kernel by kernel. The first
@@ -181,10 +182,10 @@ typedef struct {
                                    cell stores the new (d, x), and the pre-smoothing's last update
                                    rides on its residual's product, so a degree-k smoothing takes k
                                    products and one vector pass instead of k of each; 0 = a separate
-                                   vector pass after every product (default: on GB300 the products
+                                   vector pass after every product, or the pass in the products of the
+                                   small and large levels (default: on GB300 the cell products
                                    are bound by issue and latency, and gathering five vectors at every
-                                   node of every cell costs them more than the streaming pass saves:
-                                   a degree-4 smoothing at 64^3 takes 374 us fused, 268 us separate).
+                                   node of every cell costs them more than the streaming pass saves).
                                    Same arithmetic. */
 } stokes_options;
 

@@ -4,7 +4,7 @@
 // blocks with hanging-node constraints resolved in the gather and the scatter (Section 2.1,
 // with the constrained space of the adaptive meshes).
 //
-// Every kernel takes one cell (or one node) per thread. Level vectors are component-blocked
+// A thread takes one cell, one node, or (FP64 operators) one component of a cell. Level vectors are component-blocked
 // [3][nn]; the active velocity vector is [3][nu] and the active pressure vector [np].
 #include "octree.cuh"
 #include "outer.cuh"

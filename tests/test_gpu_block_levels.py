@@ -1,6 +1,6 @@
 """The FP32 operator of the small levels (csrc/block.cu): products, smoothing steps and V-cycles against the
 component-split operator with separate vector passes (vmult_kernel = 3, itself checked against the
-oracle): one cell, sizes that end inside a 4 x 4 x 4 block, every coarsest mesh, every parity of the Chebyshev
+oracle): one cell, sizes that end inside a block, every coarsest mesh, every parity of the Chebyshev
 degree from zero and from a guess; V-cycles twice, since the first leaves its buffers to the second.
 
 Tolerances: 2e-6 for a product and 2e-5 for smoothing and the V-cycle, the FP32 bounds of the parity tests:
