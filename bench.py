@@ -420,7 +420,7 @@ def run_ours(args):
     # live FMA peaks of this GPU (FMA-chain probe), for the ALU side of the roofline
     f32_peak, f64_peak = capi.stokes_probe_fma()
     line["alu_peaks_tflops"] = {"fp32": f32_peak, "fp64": f64_peak, "how": "stokes_probe_fma: 8 FMA chains/thread"}
-    line["roofline"] = dominant_roofline(prof, dopt, cells, n_u, N, hbm, hbm_src, f32_peak, f64_peak, args.workload)
+    line["roofline"] = dominant_roofline(prof, cells, N, hbm, hbm_src, f32_peak, args.workload)
 
     # class-level roofline of the FGMRES vector kernels: algorithmic bytes of their passes over
     # the profiled solve / their summed time
@@ -508,7 +508,7 @@ def run_ours(args):
     print(json.dumps(line))
 
 
-VMULT_KERNELS = {0: "k_cell_atomic (one thread per cell, FP32 pipes, atomic scatter)",
+VMULT_KERNELS = {0: "by level size: k_block, k_cell_atomic, k_march (FP32 pipes, Legendre modes)",
                  1: "k_brick + k_planes (brick-tiled, deterministic)",
                  2: "k_cell_tc (cell products on the tensor cores, tcgen05 kind::f16, shared-memory node tile)"}
 
@@ -566,42 +566,34 @@ def time_vmult(capi, ctx, n, n_u, stream, hbm, reps=(20, 5)):
     return out
 
 
-def dominant_roofline(prof, dopt, cells, n_u, N, hbm, hbm_src, f32_peak, f64_peak, workload):
-    """Roofline of the single kernel with the largest time in the profiled solve. achieved =
-    algorithmic bytes per launch / its mean launch time, against the measured HBM peak; the ALU
-    side (method flops against the FMA probe) beside it."""
-    single = ("stokes_fp64", "vmult_A_fp32")
-    dom = max(single, key=lambda k: prof.get(k, (0.0, 0))[0])
-    dms = prof[dom][0] / max(prof[dom][1], 1)
-    if dom == "stokes_fp64":
-        bytes_alg = (2 * N + cells) * 8
-        fl = cells * STOKES_FLOP_PER_CELL
-        r = {"kernel": "k_outer_fix<1,1,1> (outer [A B^T; B 0], 64-bit fixed point)",
-             "bound": "hbm", "achieved": bytes_alg / (dms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
-             "frac": bytes_alg / (dms / 1e3) / 1e9 / hbm,
-             "traffic": recorded_traffic("stokes_fixed", workload),
-             "peak_note": hbm_src, "launch_ms": dms,
-             "per_launch": "(2 (N_u + N_p) + cells) x 8 B = %d B (u, p read and written in FP64, cell viscosity)"
-                           % bytes_alg}
-        alu_peak = f32_peak
-        r["alu"] = {"method_flop_per_cell": STOKES_FLOP_PER_CELL, "achieved_gflops": fl / (dms / 1e3) / 1e9,
-                    "peak_gflops": alu_peak * 1e3, "frac": fl / (dms / 1e3) / 1e9 / (alu_peak * 1e3),
-                    "peak_note": "of measured (FFMA probe, this run); the method flops, run as "
-                                 "64-bit integer operations in the Legendre modes"}
-        inst = recorded_traffic("stokes_fixed_inst", workload)
-        if inst:
-            ips = inst / (dms / 1e3)
-            r["issue"] = {"thread_inst_per_launch": inst, "frac": ips / (f32_peak / 2 * 1e12),
-                          "note": "instructions per launch (ncu smsp__inst_executed.sum x 32) against the "
-                                  "FFMA probe's instruction rate (FMA = 1 instruction): the issue efficiency "
-                                  "of the fixed-point code"}
-        return r
-    bytes_alg = (2 * n_u + cells) * 4
-    return {"kernel": dom, "bound": "hbm", "achieved": bytes_alg / (dms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
-            "frac": bytes_alg / (dms / 1e3) / 1e9 / hbm, "traffic": recorded_traffic(dom, workload),
-            "peak_note": hbm_src, "launch_ms": dms,
-            "per_launch": "finest-level (2 N_u + cells) x 4 B = %d B (mean over the solve's levels is lower)"
-                          % bytes_alg}
+def dominant_roofline(prof, cells, N, hbm, hbm_src, f32_peak, workload):
+    """Roofline of the outer operator, the single kernel with the largest time in the profiled solve
+    (the level operator's class has more, over kernels and levels of all sizes). achieved = algorithmic
+    bytes per launch / its mean launch time, against the measured HBM peak; the ALU side (method flops
+    against the FMA probe) beside it."""
+    dms = prof["stokes_fp64"][0] / max(prof["stokes_fp64"][1], 1)
+    bytes_alg = (2 * N + cells) * 8
+    fl = cells * STOKES_FLOP_PER_CELL
+    r = {"kernel": "k_outer_fix<1,1,1> (outer [A B^T; B 0], 64-bit fixed point)",
+         "bound": "hbm", "achieved": bytes_alg / (dms / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",
+         "frac": bytes_alg / (dms / 1e3) / 1e9 / hbm,
+         "traffic": recorded_traffic("stokes_fixed", workload),
+         "peak_note": hbm_src, "launch_ms": dms,
+         "per_launch": "(2 (N_u + N_p) + cells) x 8 B = %d B (u, p read and written in FP64, cell viscosity)"
+                       % bytes_alg}
+    alu_peak = f32_peak
+    r["alu"] = {"method_flop_per_cell": STOKES_FLOP_PER_CELL, "achieved_gflops": fl / (dms / 1e3) / 1e9,
+                "peak_gflops": alu_peak * 1e3, "frac": fl / (dms / 1e3) / 1e9 / (alu_peak * 1e3),
+                "peak_note": "of measured (FFMA probe, this run); the method flops, run as "
+                             "64-bit integer operations in the Legendre modes"}
+    inst = recorded_traffic("stokes_fixed_inst", workload)
+    if inst:
+        ips = inst / (dms / 1e3)
+        r["issue"] = {"thread_inst_per_launch": inst, "frac": ips / (f32_peak / 2 * 1e12),
+                      "note": "instructions per launch (ncu smsp__inst_executed.sum x 32) against the "
+                              "FFMA probe's instruction rate (FMA = 1 instruction): the issue efficiency "
+                              "of the fixed-point code"}
+    return r
 
 
 def run_refinement(capi, si, torch, stream):
