@@ -31,6 +31,7 @@
 // fixed order, so the results do not depend on scheduling. Basis rows have an
 // even stride so that every entry pair is 16-byte aligned.
 #include "df64.cuh"
+#include "gs.cuh"
 #include "internal.cuh"
 #include "prof.cuh"
 
@@ -48,7 +49,6 @@ namespace {
 
 using q2::df64;
 
-constexpr int kGsThreads = 128;
 constexpr int kGsMaxK = 64;                 // largest basis of the double-float passes
 constexpr int kGsMaxBlocks = 2432;          // 16 per SM on 152 SMs; the partials buffer is sized for this
 
@@ -63,8 +63,8 @@ enum GsMode { GS_DOT = 0, GS_PROJECT_DOT = 1, GS_PROJECT_SCALE = 2, GS_LAG = 3 }
 // An entry pair is handled by TPE adjacent lanes, each with RB basis rows (at most 16: with 32 rows
 // per thread, or with 8 and 4 and more threads per pair, whole solves are slower). The shape is the
 // smallest that holds k rows (gs_shapes); every lane runs its RB rows without tests: rows past the
-// k-th are zero with zero coefficients, entries past the n-th repeat the last ones with w = 0. (One
-// test per row and entry pair cost as many instructions as the arithmetic.) Measured at 48^3 with 24
+// k-th are zero with zero coefficients, lanes past the last pair repeat it (GS_LAG: load nothing, gs_reads) with
+// w = 0. (One test per row and entry pair cost as many instructions as the arithmetic.) Measured at 48^3 with 24
 // rows of 2.9 M entries: dot products 91 us, 6.3 TB/s; GS_LAG 114 us, bound by the arithmetic of its two
 // double-float products per entry (134 and 210 us with tests and with the rows passing through shared
 // memory). 16 rows per thread at most: 168 registers, three CTAs per SM; up to 12 rows four.
@@ -115,7 +115,6 @@ __global__ void __launch_bounds__(kGsThreads, RB <= 12 ? 4 : 3) k_gs_df(size_t n
     extern __shared__ double smem[];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int g = tid % TPE;              // row group: rows r0 .. r0 + RB - 1
-    const int slot = tid / TPE;           // entry pair within the CTA's sweep
     const int r0 = g * RB;
     const int nr = max(0, min(RB, k - r0));   // rows of the group below k
     constexpr int NH = MODE == GS_LAG ? 3 : 1;
@@ -152,7 +151,7 @@ __global__ void __launch_bounds__(kGsThreads, RB <= 12 ? 4 : 3) k_gs_df(size_t n
     const size_t np = (n + 1) / 2;
     const size_t warp_first = size_t(blockIdx.x) * PPB + size_t(wid) * (32 / TPE);
     const size_t stride = size_t(gridDim.x) * PPB;
-    const size_t p0 = size_t(blockIdx.x) * PPB + slot;
+    const size_t p0 = gs_pair(0, blockIdx.x, tid, TPE);
     float4 v[RB];   // rows from nr on stay 0
 #pragma unroll
     for (int r = 0; r < RB; ++r) v[r] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -169,19 +168,19 @@ __global__ void __launch_bounds__(kGsThreads, RB <= 12 ? 4 : 3) k_gs_df(size_t n
     load_w(p0, wn0, wn1);
     for (int it = 0; warp_first + base < np; ++it) {
         const size_t p = p0 + base;
-        const bool in = p < np;
+        const bool in = gs_reads(p, np);
         const bool in1 = 2 * p + 1 < n;
         {
-            const double* src = V + 2 * min(p, np - 1) + size_t(r0) * ld;
+            const double* src = V + 2 * (MODE == GS_LAG ? p : min(p, np - 1)) + size_t(r0) * ld;
 #pragma unroll
             for (int r = 0; r < RB; ++r) {
-                if (r < nr) v[r] = load_pairs(src);
+                if (r < nr && (MODE != GS_LAG || in)) v[r] = load_pairs(src);
                 src += ld;
             }
         }
         float4 uj = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         if constexpr (MODE == GS_LAG)
-            if (g == 0) uj = load_pairs(V + 2 * min(p, np - 1) + size_t(k - 1) * ld);   // row j once more, from L2
+            if (g == 0 && in) uj = load_pairs(V + 2 * p + size_t(k - 1) * ld);   // row j once more, from L2
         df64 w0 = q2::split_double(wn0), w1 = q2::split_double(wn1);
         load_w(p + stride, wn0, wn1);
         if constexpr (MODE == GS_DOT) {
