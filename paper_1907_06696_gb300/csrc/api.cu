@@ -119,7 +119,7 @@ template <typename T>
 struct LevelVecs {
     T* b = nullptr;   // right-hand side of the level problem
     T* x = nullptr;   // level solution / correction
-    T* r = nullptr;   // residual
+    T* r = nullptr;   // residual; while the level smooths, the marching operator's second direction
     T* d = nullptr;   // Chebyshev direction
     T* t = nullptr;   // operator output
     T* mu = nullptr;  // cell viscosity
@@ -369,16 +369,20 @@ stokes_status smooth(stokes_ctx* c, int l, const T* b, T* x, bool zero_guess, cu
     const size_t n = L.g.n_u;
     // the operators with the epilogue inside write the new iterate beside the old one (its neighbours
     // read that): the iterates alternate between x and the level's x2, starting where the last step
-    // ends in x
+    // ends in x. The marching operator writes its direction beside the old one too, into the residual's
+    // vector, which is free while a level smooths
     const bool apart = out_of_place<T>(c, l, b, x), block = level_kernel<T>(c, l) == kBlockKernel;
-    T* X[2] = {x, v.x2};
-    int cur = apart ? (c->opt.cheb_degree - (zero_guess ? 1 : 0)) & 1 : 0;
+    T *X[2] = {x, v.x2}, *D[2] = {v.d, v.r};
+    int dir = 0, cur = apart ? (c->opt.cheb_degree - (zero_guess ? 1 : 0)) & 1 : 0;
     bool pending = false;   // the first step from zero, left to the block kernel's gather
     auto step = [&](double c1, double c2) -> stokes_status {
         if (!apart) return cheb_step<T>(c, l, b, x, c1, c2, s);
         if constexpr (sizeof(T) == 4) {
             if (block) CK(launch_block(EPI_CHEB, L.g, v.mu, pending ? nullptr : X[cur], X[cur ^ 1], b, v.dinv, v.d, 1.0 / theta, c1, c2, s));
-            else CK(launch_march(EPI_CHEB, L.g, v.mu, X[cur], X[cur ^ 1], b, v.dinv, v.d, c1, c2, s));
+            else {
+                CK(launch_march(EPI_CHEB, L.g, v.mu, X[cur], X[cur ^ 1], b, v.dinv, D[dir], D[dir ^ 1], c1, c2, s));
+                dir ^= 1;
+            }
         }
         pending = false;
         cur ^= 1;

@@ -636,7 +636,7 @@ cudaError_t launch_level_op(int kernel, const LevelGeom& g, const PlaneLayout& L
         if constexpr (sizeof(T) == 4) {
             if (epi == EPI_CHEB) return cudaErrorInvalidValue;
             const cudaError_t e = kernel == kMarchKernel
-                                      ? launch_march(epi, g, mu, src, dst, b, nullptr, nullptr, 0.0, 0.0, s)
+                                      ? launch_march(epi, g, mu, src, dst, b, nullptr, nullptr, nullptr, 0.0, 0.0, s)
                                       : launch_block(epi, g, mu, src, dst, b, nullptr, nullptr, 0.0, 0.0, 0.0, s);
             return e != cudaSuccess || epi != EPI_PLAIN ? e : launch_copy_boundary<T>(g, src, dst, s);
         } else {

@@ -419,11 +419,11 @@ cudaError_t launch_cell_tc(const BrickArgs<float>& a, float* acc, const TcArgs& 
 // FP32: A src with its epilogue in one launch (march.cu); 16-byte aligned vectors. Entries on the upper
 // sides of the domain boundary are left as they are, those on the lower sides too or written as the
 // epilogue of a zero product (EPI_PLAIN: 0). EPI_PLAIN: dst = A src; EPI_RESID: dst = b - A src;
-// EPI_CHEB: d = c1 d + c2 dinv (b - A src), dst = src + d (dst is not src). Levels of
-// at least 20 cells per axis.
+// EPI_CHEB: d_new = c1 d + c2 dinv (b - A src), dst = src + d_new (dst is not src, d_new is not d: a block's copies
+// of both reach into entries that its neighbours write; EINVAL). Levels of at least 20 cells per axis.
 constexpr int kMarchKernel = 4;
 cudaError_t launch_march(int epi, const LevelGeom& g, const float* mu, const float* src, float* dst, const float* b,
-                         const float* dinv, float* d, double c1, double c2, cudaStream_t s);
+                         const float* dinv, const float* d, float* d_new, double c1, double c2, cudaStream_t s);
 // The same on levels of any size in blocks of 4 x 4 x 4 cells (block.cu), no alignment asked; entries on the
 // domain boundary are left as they are. EPI_CHEB with src null: the first step from zero is pending,
 // src = d = c0 dinv b.

@@ -55,7 +55,8 @@ struct MarchArgs {
     float* dst;            // EPI_PLAIN: A x; EPI_RESID: b - A x; EPI_CHEB: the new x (not src)
     const float* b;
     const float* dinv;
-    float* d;              // EPI_CHEB: the direction, in place
+    const float* d;        // EPI_CHEB: the direction
+    float* d_new;          // EPI_CHEB: the new direction (not d: the copies of a row reach into the next tile's)
     float c1, c2;
 };
 
@@ -221,7 +222,7 @@ __device__ __forceinline__ void march_epilogue(const MarchArgs& a, const float* 
             const float2 di = load_pair<PARITY>(e + kNext), d = load_pair<PARITY>(e + 2 * kNext),
                          x = load_pair<PARITY>(e + 3 * kNext);
             const float2 dn = make_float2(a.c1 * d.x + a.c2 * (di.x * (b.x - ax.x)), a.c1 * d.y + a.c2 * (di.y * (b.y - ax.y)));
-            store_pair<PARITY>(a.d + i, dn);
+            store_pair<PARITY>(a.d_new + i, dn);
             store_pair<PARITY>(a.dst + i, make_float2(x.x + dn.x, x.y + dn.y));
         }
     }
@@ -417,7 +418,8 @@ cudaError_t march_configure() {
 }
 
 cudaError_t launch_march(int epi, const LevelGeom& g, const float* mu, const float* src, float* dst, const float* b,
-                         const float* dinv, float* d, double c1, double c2, cudaStream_t s) {
+                         const float* dinv, const float* d, float* d_new, double c1, double c2, cudaStream_t s) {
+    if (epi == EPI_CHEB && (dst == src || d_new == d)) return cudaErrorInvalidValue;
     MarchArgs a{};
     a.n = g.n;
     a.M = g.M;
@@ -430,6 +432,7 @@ cudaError_t launch_march(int epi, const LevelGeom& g, const float* mu, const flo
     a.b = b;
     a.dinv = dinv;
     a.d = d;
+    a.d_new = d_new;
     a.c1 = float(c1);
     a.c2 = float(c2);
     const dim3 grid(unsigned((g.n + kTileX - 1) / kTileX), unsigned((g.n + kTileY - 1) / kTileY),
