@@ -221,7 +221,9 @@ __device__ __forceinline__ void march_epilogue(const MarchArgs& a, const float* 
         } else {
             const float2 di = load_pair<PARITY>(e + kNext), d = load_pair<PARITY>(e + 2 * kNext),
                          x = load_pair<PARITY>(e + 3 * kNext);
-            const float2 dn = make_float2(a.c1 * d.x + a.c2 * (di.x * (b.x - ax.x)), a.c1 * d.y + a.c2 * (di.y * (b.y - ax.y)));
+            const bool old = a.c1 != 0.0f;   // a first step has no direction before it: d holds anything, NaN too
+            const float2 dn = make_float2((old ? a.c1 * d.x : 0.0f) + a.c2 * (di.x * (b.x - ax.x)),
+                                          (old ? a.c1 * d.y : 0.0f) + a.c2 * (di.y * (b.y - ax.y)));
             store_pair<PARITY>(a.d_new + i, dn);
             store_pair<PARITY>(a.dst + i, make_float2(x.x + dn.x, x.y + dn.y));
         }
