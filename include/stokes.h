@@ -469,7 +469,8 @@ stokes_status stokes_debug_alloc_limit(long long bytes);
  * trapped on, and recorded in the context's status words; the call that ran the kernel
  * (stokes_setup_octree, stokes_vmult, gmg_vcycle, stokes_schur_inverse, stokes_precondition,
  * stokes_solve; each synchronises its stream in such a build) then returns STOKES_EMESH and
- * stokes_last_error() names the table and the entry's position in it. */
+ * stokes_last_error() names the table and the entry's position in it. Such a build also fills every
+ * device allocation with NaN (uniform meshes too). */
 int stokes_debug_build(void);
 /* Test hook of STOKES_DEBUG builds: from now on the checks of `table` on this octree context
  * accept only entries below (true bound - cut), so that the last `cut` valid entries read as bad

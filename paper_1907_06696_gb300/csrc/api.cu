@@ -244,9 +244,13 @@ stokes_status dalloc(stokes_ctx* c, T** p, size_t count) {
         g_alloc_left -= (long long)bytes;
     }
     void* q = nullptr;
-    cudaError_t e = cudaMalloc(&q, count * sizeof(T) > 0 ? count * sizeof(T) : 16);
+    cudaError_t e = cudaMalloc(&q, bytes);
     if (e != cudaSuccess) return fail(STOKES_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
     c->allocs.push_back(q);
+#ifdef STOKES_DEBUG
+    // NaN in every float and double that is read before it is written
+    if (cudaMemset(q, 0xFF, bytes) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) return fail(STOKES_ECUDA, "cudaMemset");
+#endif
     *p = static_cast<T*>(q);
     return STOKES_OK;
 }
@@ -804,12 +808,15 @@ stokes_status precondition(stokes_ctx* c, int prec, const double* r, double* z, 
                                : precondition_uniform<float>(c, r, z, s, part);
 }
 
-stokes_status ensure_krylov(stokes_ctx* c) {
+stokes_status ensure_krylov(stokes_ctx* c, cudaStream_t s) {
     const int m = c->opt.restart;
     if (c->V && c->krylov_restart == m) return STOKES_OK;
     c->N = active_nu(c) + active_np(c);
     c->ldv = c->N + (c->N & 1);   // even row stride: 16-byte aligned entry pairs (krylov.cu)
     CKS(dalloc(c, &c->V, size_t(m + 1) * c->ldv));
+    // N odd: the passes read each row's last pair whole, and no row's writer touches the entry past the N-th
+    if (c->ldv > c->N)
+        CK(cudaMemset2DAsync(c->V + c->N, c->ldv * sizeof(double), 0, sizeof(double), size_t(m + 1), s));
     // flexible GMRES keeps the m preconditioned vectors; GMRES (outer_solver 2) one work vector
     CKS(dalloc(c, &c->Z, c->opt.outer_solver == 2 ? c->ldv : size_t(m) * c->N));
     CKS(dalloc(c, &c->w, c->N));
@@ -1109,7 +1116,7 @@ stokes_status fgmres_complete(FgmresRun& r) {
 
 stokes_status fgmres_init(FgmresRun& r, stokes_ctx* c, int prec, const double* b, double* x, double rtol,
                           int max_it, stokes_solve_info* info, cudaStream_t s) {
-    CKS(ensure_krylov(c));
+    CKS(ensure_krylov(c, s));
     r.c = c;
     r.prec = prec;
     r.b = b;
@@ -2588,7 +2595,7 @@ stokes_status stokes_solve(stokes_ctx* c, int vcycle_prec, const double* rhs, do
         c->N = active_nu(c) + active_np(c);   // MINRES vectors: minres_solve
         if (!c->bvec) CKS(dalloc(c, &c->bvec, c->N));
     } else {
-        CKS(ensure_krylov(c));
+        CKS(ensure_krylov(c, s));
     }
     const size_t nu = active_nu(c), np = active_np(c);
     const double* b = rhs;
@@ -2694,7 +2701,7 @@ stokes_status stokes_autotune(stokes_ctx* c, int what, void* stream, int* block_
         // Chebyshev degree: wall time of a short FGMRES solve (FP32 V-cycle, relative residual 1e-3,
         // zero guess, the context's own right-hand side [F; 0]) for each candidate degree
         const int keep = c->opt.cheb_degree;
-        if ((st = ensure_krylov(c)) == STOKES_OK && !c->tune_up) st = dalloc(c, &c->tune_up, c->N);
+        if ((st = ensure_krylov(c, s)) == STOKES_OK && !c->tune_up) st = dalloc(c, &c->tune_up, c->N);
         double best_t = 1e300;
         int best_deg = keep;
         const LevelGeom& g = F.g;
@@ -2753,7 +2760,7 @@ stokes_status stokes_batch_solve(int n_problems, stokes_ctx* const* ctxs, int vc
             if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) { st = fail(STOKES_ECUDA, "stream"); break; }
             own.push_back(s);
         }
-        st = ensure_krylov(c);
+        st = ensure_krylov(c, s);
         if (st != STOKES_OK) break;
         const LevelGeom& g = c->lev[c->L - 1].g;
         const double* b = rhs_devs ? rhs_devs[i] : nullptr;

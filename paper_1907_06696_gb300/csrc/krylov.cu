@@ -29,7 +29,8 @@
 // combined across the entry's threads by shuffles. The per-thread dot sums are reduced per warp and CTA in
 // double-float and written as doubles to `partials`, which one CTA adds in a
 // fixed order, so the results do not depend on scheduling. Basis rows have an
-// even stride so that every entry pair is 16-byte aligned.
+// even stride so that every entry pair is 16-byte aligned; with an odd number of entries the last
+// pair's second entry is 0 in every row (set with the allocation, written by none of the passes).
 #include "df64.cuh"
 #include "gs.cuh"
 #include "internal.cuh"
