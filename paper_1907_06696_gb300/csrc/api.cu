@@ -783,13 +783,11 @@ stokes_status precondition_head(stokes_ctx* c, const double* r, double* z, cudaS
     return STOKES_OK;
 }
 
-// z_u from the finest level's result; boundary rows are the identity.
+// z_u from the finest level's result; boundary rows are the identity (also where z is r).
 template <typename T>
 stokes_status precondition_tail(stokes_ctx* c, const double* r, double* z, cudaStream_t s) {
     Level& F = c->lev[c->L - 1];
-    if constexpr (sizeof(T) == 4) CK(launch_cast_f2d(F.g.n_u, F.v32.x, z, s));
-    else CK(cudaMemcpyAsync(z, F.v64.x, F.g.n_u * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    CK(launch_copy_boundary<double>(F.g, r, z, s));
+    CK(launch_free_rows<T>(F.g, vecs<T>(F).x, r, z, s));
     return STOKES_OK;
 }
 

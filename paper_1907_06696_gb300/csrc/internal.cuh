@@ -103,9 +103,11 @@ cudaError_t launch_zero_boundary(const LevelGeom& g, T* x, cudaStream_t s);
 // out = in on boundary nodes (identity rows).
 template <typename T>
 cudaError_t launch_copy_boundary(const LevelGeom& g, const T* in, T* out, cudaStream_t s);
-// Casts with the boundary entries zeroed (to_boundary_zero) or kept.
+// z = x on free nodes, r on boundary nodes; z may be r.
+template <typename T>
+cudaError_t launch_free_rows(const LevelGeom& g, const T* x, const double* r, double* z, cudaStream_t s);
+// out = in rounded to FP32.
 cudaError_t launch_cast_d2f(size_t n, const double* in, float* out, cudaStream_t s);
-cudaError_t launch_cast_f2d(size_t n, const float* in, double* out, cudaStream_t s);
 // Coarse solve: x[free[i]] = sum_j Ainv[i][j] b[free[j]], FP64 arithmetic; x elsewhere untouched.
 template <typename T>
 cudaError_t launch_coarse_solve(int nf, const int* free_idx, const double* Ainv, const T* b, T* x, cudaStream_t s);

@@ -43,6 +43,16 @@ __global__ void k_copy_boundary(int M, const T* __restrict__ in, T* __restrict__
     for (int c = 0; c < 3; ++c) out[c * nodes + node] = in ? in[c * nodes + node] : T(0);
 }
 
+// z = x on the free nodes, r on the domain boundary; z may be r.
+template <typename T>
+__global__ void __launch_bounds__(256) k_free_rows(int M, const T* __restrict__ x, const double* r, double* z) {
+    const size_t nodes = size_t(M) * M * M, node = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (node >= nodes) return;
+    const bool b = on_bnd(int(node % M), M) || on_bnd(int(node / M % M), M) || on_bnd(int(node / (size_t(M) * M)), M);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) z[c * nodes + node] = b ? r[c * nodes + node] : double(x[c * nodes + node]);
+}
+
 // ---------------------------------------------------------------- pressure mass
 __global__ void k_mass_p(int n, double h, const double* __restrict__ mu, const double* __restrict__ src,
                          double* __restrict__ dst) {
@@ -348,6 +358,14 @@ cudaError_t launch_zero_boundary(const LevelGeom& g, T* x, cudaStream_t s) {
 }
 template cudaError_t launch_zero_boundary<float>(const LevelGeom&, float*, cudaStream_t);
 template cudaError_t launch_zero_boundary<double>(const LevelGeom&, double*, cudaStream_t);
+
+template <typename T>
+cudaError_t launch_free_rows(const LevelGeom& g, const T* x, const double* r, double* z, cudaStream_t s) {
+    LAUNCH(PROF_CAST, s, (k_free_rows<T><<<blocks_for(g.nodes, 256), 256, 0, s>>>(g.M, x, r, z)));
+    return cudaGetLastError();
+}
+template cudaError_t launch_free_rows<float>(const LevelGeom&, const float*, const double*, double*, cudaStream_t);
+template cudaError_t launch_free_rows<double>(const LevelGeom&, const double*, const double*, double*, cudaStream_t);
 
 cudaError_t launch_stokes_blocks(const LevelGeom& g, const double* mu, const double* src_u, const double* src_p,
                                  double* dst_u, double* dst_p, bool do_a, bool do_bt, bool do_b, cudaStream_t s) {

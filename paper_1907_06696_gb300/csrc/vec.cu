@@ -80,10 +80,6 @@ __global__ void k_cast_d2f(size_t n, const double* __restrict__ in, float* __res
     for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x)
         out[i] = float(in[i]);
 }
-__global__ void k_cast_f2d(size_t n, const float* __restrict__ in, double* __restrict__ out) {
-    for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x)
-        out[i] = double(in[i]);
-}
 
 template <typename T>
 __global__ void k_coarse_solve(int nf, const int* __restrict__ idx, const double* __restrict__ Ainv,
@@ -348,10 +344,6 @@ template cudaError_t launch_residual<double>(size_t, const double*, const double
 
 cudaError_t launch_cast_d2f(size_t n, const double* in, float* out, cudaStream_t s) {
     LAUNCH(PROF_CAST, s, k_cast_d2f<<<grid_stride_blocks(n), 256, 0, s>>>(n, in, out));
-    return cudaGetLastError();
-}
-cudaError_t launch_cast_f2d(size_t n, const float* in, double* out, cudaStream_t s) {
-    LAUNCH(PROF_CAST, s, k_cast_f2d<<<grid_stride_blocks(n), 256, 0, s>>>(n, in, out));
     return cudaGetLastError();
 }
 
