@@ -69,6 +69,7 @@ __host__ __device__ __forceinline__ void outer_atomic_add(double* p, double v) {
 constexpr int kFixBits = 54;      // |X| <= 2^54
 constexpr int kFixMid = 12;       // bits dropped after the element matrix
 constexpr int kFixMinExp = 64;    // cells whose largest value is below 2^-958 read as 0
+constexpr int kFixNone = -4096;   // exponent of a cell that reads as 0
 
 __host__ __device__ __forceinline__ double bits_to_dbl(long long b) {
 #ifdef __CUDA_ARCH__
@@ -116,12 +117,17 @@ __host__ __device__ __forceinline__ double fix_out(long long x, double scale) {
     const long long b = a ? m + ((long long)(1085 - lz) << 52) : 0;   // m in [2^52, 2^53]: |x| = m 2^(11 - lz)
     return bits_to_dbl(b | (sign & (long long)(1ull << 63))) * scale;
 }
-// s 2^e; NaN where the cell holds one (or an infinity).
+// s 2^e, |e| < 2044; NaN where the cell holds one (or an infinity). A pressure against a large or small viscosity can
+// take 2^e alone out of the FP64 range: two factors.
 __host__ __device__ __forceinline__ double fix_scale(double s, int e, bool zero, bool bad) {
     if (bad) return bits_to_dbl(0x7FF8000000000000LL);
     if (zero) return 0.0;
-    const int k = e < -1022 ? -1022 : (e > 1023 ? 1023 : e);
-    return s * bits_to_dbl((long long)(k + 1023) << 52);
+    int k = 0;
+    if (e < -1022 || e > 1023) {
+        k = e / 2;
+        s *= bits_to_dbl((long long)(k + 1023) << 52);
+    }
+    return s * bits_to_dbl((long long)(e - k + 1023) << 52);
 }
 // A 96-bit sum of products of modes with non-negative table entries below 2^12: high and low words apart.
 struct FixSum {
@@ -314,7 +320,8 @@ __host__ __device__ __forceinline__ double outer_velocity(int C, int g, const Ou
                 }
                 Y[m] = y.shifted();
             }
-    int E = DO_A && eu >= kFixMinExp ? eu : 0;
+    const int eu0 = DO_A && eu >= kFixMinExp ? eu : kFixNone;
+    int E = eu0;
     bool bad = DO_A && eu == 0x7FF;
     if (DO_BT) {
         // p' = 112.5 h/mu p: the vertex modes times the factor's significand, |R| <= 2^61; |p'| < 2^(epk - 1022)
@@ -331,7 +338,7 @@ __host__ __device__ __forceinline__ double outer_velocity(int C, int g, const Ou
                 P[v] = sh.P[((v & 1) << C) + (((v >> 1) & 1) << D1) + ((v >> 2) << D2)][g];
             q2::to_pressure_modes(P);
             const int sp = E - epk + 16 < 63 ? E - epk + 16 : 63;
-            const int sa = DO_A ? (E - eu < 63 ? E - eu : 63) : 0;
+            const int sa = DO_A ? (E - eu0 < 63 ? E - eu0 : 63) : 0;
             if (sa > 0) {
 #pragma unroll
                 for (int m = 0; m < 27; ++m) Y[m] >>= sa;
@@ -347,7 +354,7 @@ __host__ __device__ __forceinline__ double outer_velocity(int C, int g, const Ou
     fix_from_modes<2>(Y);
     fix_from_modes<1>(Y);
     fix_from_modes<0>(Y);
-    return fix_scale(mu * h * (1.0 / 97200.0), E - 1022 - kFixBits + kFixMid, E == 0, bad);
+    return fix_scale(mu * h * (1.0 / 97200.0), E - 1022 - kFixBits + kFixMid, E == kFixNone, bad);
 }
 
 // Phase 1b (after a barrier): fixed point and modes.
