@@ -398,7 +398,9 @@ stokes_status stokes_precondition(stokes_ctx* ctx, int vcycle_prec, const double
                                   void* stream);
 
 /* Autotuner (no counterpart in the paper). what = 1: threads per block of the cell-parallel level
- * operator (64, 128 or 256; the fastest FP32 product on the finest level); what = 2: the Chebyshev
+ * operator (32, 64, 128 or 256, 32 unless tuned; the fastest FP32 product on the finest level that takes
+ * this operator, by default one of 17 to 63 cells per axis. Where none does, nothing is timed and block_out
+ * is 128, a setting that no FP32 level uses; with vmult_kernel other than 0 it is 0); what = 2: the Chebyshev
  * degree (3..6) with the shortest wall time of an FGMRES solve to relative residual 1e-3 with the
  * FP32 V-cycle and the context's own right-hand side; what = 3: both. The choice is kept in the
  * context for later V-cycles and solves (captured graphs are dropped and recaptured). Outputs may

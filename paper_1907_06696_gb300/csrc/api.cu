@@ -311,9 +311,10 @@ constexpr int kBlockMaxN = 16, kMarchMinN = 64;
 // Blocks of the cell kernel on FP32 levels unless tuned: with 32 threads its gathers and atomic adds spread over more
 // SMs (V-cycle 20^3 137 -> 131 us, 32^3 268 -> 264 us, 40^3 287 -> 273 us; product at 20^3 14.3 -> 12.1 us
 // against blocks of 128; 24^3 and 48^3 the same).
+constexpr int kCellThreadsF32 = 32;
 template <typename T>
 int cell_threads(const stokes_ctx* c) {
-    return sizeof(T) == 4 && !c->cell_tuned ? 32 : c->cell_block;
+    return sizeof(T) == 4 && !c->cell_tuned ? kCellThreadsF32 : c->cell_block;
 }
 
 template <typename T>
@@ -2666,33 +2667,42 @@ stokes_status stokes_autotune(stokes_ctx* c, int what, void* stream, int* block_
         CKS(dalloc(c, &c->tune_r, n));
         CKS(dalloc(c, &c->tune_b, n));
     }
-    // seeded right-hand side with zero constrained entries
-    CK(launch_splitmix_vector(n, 4242, nullptr, c->tu, s));
-    CK(launch_cast_d2f(n, c->tu, c->tune_b, s));
-    CK(launch_zero_boundary<float>(F.g, c->tune_b, s));
+    int lt = c->L - 1;   // the finest level that takes the cell kernel in FP32, -1: none does
+    while (lt >= 0 && (c->opt.vmult_kernel != 0 || level_kernel<float>(c, lt) != cell_threads<float>(c))) --lt;
+    if ((what & 1) && lt >= 0) {   // seeded operand with zero constrained entries
+        const LevelGeom& g = c->lev[lt].g;
+        CK(launch_splitmix_vector(g.n_u, 4242, nullptr, c->tu, s));
+        CK(launch_cast_d2f(g.n_u, c->tu, c->tune_b, s));
+        CK(launch_zero_boundary<float>(g, c->tune_b, s));
+    }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     stokes_status st = STOKES_OK;
-    // only the cell kernel has a block size
-    if ((what & 1) && c->opt.vmult_kernel == 0 && level_kernel<float>(c, c->L - 1) == cell_threads<float>(c)) {
-        // threads per block of the cell kernel: the fastest FP32 level operator on the finest level
-        float best = 1e30f;
-        int best_bs = c->cell_block;
+    if ((what & 1) && lt >= 0) {
+        // threads per block of the cell kernel: the fastest FP32 product on the finest level that takes it. The default
+        // stays unless another size is faster by more than a short timing's noise.
+        const bool tuned = c->cell_tuned;
+        const int keep = c->cell_block;
+        float best = 0.0f;
+        int best_bs = kCellThreadsF32;
         c->cell_tuned = true;
-        for (int bs : {64, 128, 256}) {
+        for (int bs : {kCellThreadsF32, 64, 128, 256}) {
             c->cell_block = bs;
-            for (int it = 0; it < 2; ++it) st = vmult_level<float>(c, c->L - 1, c->tune_b, c->tune_r, s);
-            cudaEventRecord(e0, s);
-            for (int it = 0; it < 10 && st == STOKES_OK; ++it) st = vmult_level<float>(c, c->L - 1, c->tune_b, c->tune_r, s);
-            cudaEventRecord(e1, s);
-            cudaEventSynchronize(e1);
-            float ms = 0.0f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            if (st != STOKES_OK) break;
-            if (ms < best) { best = ms; best_bs = bs; }
+            float ms = 1e30f;
+            for (int rep = 0; rep < 4 && st == STOKES_OK; ++rep) {   // the first one warms up
+                cudaEventRecord(e0, s);
+                for (int it = 0; it < 10 && st == STOKES_OK; ++it) st = vmult_level<float>(c, lt, c->tune_b, c->tune_r, s);
+                cudaEventRecord(e1, s);
+                cudaEventSynchronize(e1);
+                float t = 0.0f;
+                cudaEventElapsedTime(&t, e0, e1);
+                if (rep > 0) ms = std::min(ms, t);
+            }
+            if (bs == kCellThreadsF32 || ms < 0.98f * best) { best = ms; best_bs = bs; }
         }
-        c->cell_block = best_bs;
+        c->cell_tuned = st == STOKES_OK || tuned;
+        c->cell_block = st == STOKES_OK ? best_bs : keep;
         if (st == STOKES_OK) st = drop_graphs(c);
     }
     if (st == STOKES_OK && (what & 2)) {
@@ -2725,7 +2735,7 @@ stokes_status stokes_autotune(stokes_ctx* c, int what, void* stream, int* block_
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (st != STOKES_OK) return st;
-    if (block_out) *block_out = c->opt.vmult_kernel != 0 ? 0 : c->cell_block;
+    if (block_out) *block_out = c->opt.vmult_kernel != 0 ? 0 : (lt >= 0 ? cell_threads<float>(c) : c->cell_block);
     if (degree_out) *degree_out = c->opt.cheb_degree;
     return STOKES_OK;
 }
