@@ -1386,10 +1386,9 @@ stokes_status ensure_idr(stokes_ctx* c, int sdim) {
         CKS(dalloc(c, &c->idr_G, size_t(sdim) * N));
         CKS(dalloc(c, &c->idr_U, size_t(sdim) * N));
         CKS(dalloc(c, &c->idr_P, size_t(sdim) * N));
-        if (!c->idr_r) {
-            for (double** q : {&c->idr_r, &c->idr_v, &c->idr_t, &c->idr_tmp}) CKS(dalloc(c, q, N));
-            CKS(dalloc(c, &c->idr_c, 16));
-        }
+        for (double** q : {&c->idr_r, &c->idr_v, &c->idr_t, &c->idr_tmp})
+            if (!*q) CKS(dalloc(c, q, N));
+        if (!c->idr_c) CKS(dalloc(c, &c->idr_c, 16));
         c->idr_alloc_s = sdim;
     }
     if (!c->bvec) CKS(dalloc(c, &c->bvec, N));
@@ -2662,11 +2661,8 @@ stokes_status stokes_autotune(stokes_ctx* c, int what, void* stream, int* block_
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     Level& F = c->lev[c->L - 1];
     const size_t n = F.g.n_u;
-    if (!c->tune_x) {
-        CKS(dalloc(c, &c->tune_x, n));
-        CKS(dalloc(c, &c->tune_r, n));
-        CKS(dalloc(c, &c->tune_b, n));
-    }
+    for (float** q : {&c->tune_x, &c->tune_r, &c->tune_b})
+        if (!*q) CKS(dalloc(c, q, n));   // each on its own: an earlier call may have got some of them only
     int lt = c->L - 1;   // the finest level that takes the cell kernel in FP32, -1: none does
     while (lt >= 0 && (c->opt.vmult_kernel != 0 || level_kernel<float>(c, lt) != cell_threads<float>(c))) --lt;
     if ((what & 1) && lt >= 0) {   // seeded operand with zero constrained entries
@@ -2813,10 +2809,8 @@ stokes_status stokes_solve_host(stokes_ctx* c, int vcycle_prec, const double* rh
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t N = active_nu(c) + active_np(c);
     const auto t0 = std::chrono::steady_clock::now();
-    if (!c->h_up_dev) {
-        CKS(dalloc(c, &c->h_up_dev, N));
-        CKS(dalloc(c, &c->h_rhs_dev, N));
-    }
+    for (double** q : {&c->h_up_dev, &c->h_rhs_dev})
+        if (!*q) CKS(dalloc(c, q, N));
     const double* rhs_dev = nullptr;
     if (rhs_host) {
         CK(cudaMemcpyAsync(c->h_rhs_dev, rhs_host, N * sizeof(double), cudaMemcpyHostToDevice, s));
