@@ -105,12 +105,14 @@ typedef struct {
     int schur_degree;           /* Chebyshev degree of S_hat^-1 on M_p, interval [1/8, 27/8] (5); 0 = S_hat =
                                    diag(M_p) itself (Section 3.4; degree 1 is (4/7) diag(M_p)^-1) */
     int restart;                /* FGMRES restart length (50, Section 3.4) */
-    int outer_arith;            /* arithmetic behind the FP64 interface: 0 = FP64 or its accuracy everywhere
-                                   (A, B, B^T and the Stokes block in 64-bit fixed point, which GB300
-                                   runs ~9x faster than FP64 instructions; FP64 Krylov basis);
-                                   1 = as 0, but the Krylov basis and the preconditioner's B^T in
-                                   double-float (pairs of floats, ~48-bit significand) on the FP32
-                                   units (default). Both match the FP64 oracle to 1e-12.
+    int outer_arith;            /* arithmetic behind the FP64 interface: 0 = FP64 or its accuracy (A, B and
+                                   the Stokes block in 64-bit fixed point, which GB300 runs ~9x faster
+                                   than FP64 instructions; B^T and the Krylov basis in FP64; S_hat^-1's
+                                   M_p products of uniform meshes in double-float for every value);
+                                   1 = as 0, but the Krylov basis and, before an FP32 V-cycle on a
+                                   uniform mesh, the preconditioner's B^T in double-float (pairs of
+                                   floats, ~48-bit significand) on the FP32 units (default). Both match
+                                   the FP64 oracle to 1e-12.
                                    2 = the whole operator [A B^T; B 0] of uniform meshes on the tensor
                                    cores, exactly: each cell's FP64 inputs in fixed point against their
                                    largest magnitude, split into 7 digit slices of 8 bits, times the

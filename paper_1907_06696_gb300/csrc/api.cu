@@ -775,7 +775,7 @@ stokes_status precondition_head(stokes_ctx* c, const double* r, double* z, cudaS
     CKS(schur_inverse(c, r + nu, zp, s));
     if (c->opt.precond_kind != 1) {
         CK(launch_axpby(F.g.n_p, -1.0, zp, 0.0, zp, s));                      // z_p = -S^-1 r_p
-        CK(launch_bt_resid<T>(F.g, zp, r, vecs<T>(F).b, s));
+        CK(launch_bt_resid<T>(F.g, zp, r, vecs<T>(F).b, c->opt.outer_arith >= 1, s));
         return STOKES_OK;
     }   // else P_D: z_p = S_hat^-1 r_p, z_u = A_hat^-1 r_u
     if constexpr (sizeof(T) == 4) CK(launch_cast_d2f(nu, r, F.v32.b, s));

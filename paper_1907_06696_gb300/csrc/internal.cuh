@@ -53,9 +53,9 @@ cudaError_t launch_outer_tc(const LevelGeom& g, const double* mu, const double* 
 // dst = M_p src (weighted pressure mass, FP64).
 cudaError_t launch_mass_p(const LevelGeom& g, const double* mu, const double* src, double* dst, cudaStream_t s);
 // out = r - B^T p on the uniform mesh's free nodes (boundary entries of out left as they are), gathered, no
-// atomics; T = float: the product in double-float, one rounding at the end.
+// atomics; T = float: in double-float (df) or FP64, one rounding at the end; T = double: in FP64.
 template <typename T>
-cudaError_t launch_bt_resid(const LevelGeom& g, const double* p, const double* r, T* out, cudaStream_t s);
+cudaError_t launch_bt_resid(const LevelGeom& g, const double* p, const double* r, T* out, bool df, cudaStream_t s);
 // scale[cell] = h^3 / mu[cell]
 cudaError_t launch_mass_scale(const LevelGeom& g, const double* mu, double* scale, cudaStream_t s);
 // One Chebyshev step of S_hat^-1 with M_p gathered per vertex (double-float products):

@@ -82,28 +82,29 @@ __global__ void k_mass_p(int n, double h, const double* __restrict__ mu, const d
 // ---- B^T on the uniform mesh as a gather, one thread per cell (e, f, g) and its 8 nodes of lower or odd
 // index (pressure.cuh bt_nodes); nodes on the domain boundary are left as they are.
 // BT_PLAIN: out = B^T p;  BT_RESID: out = r - B^T p (the V-cycle's right-hand side), TO = double in FP64,
-// TO = float in double-float without an FP64 instruction, rounded once at the end.
+// TO = float (the right-hand side of an FP32 V-cycle) in double-float without an FP64 instruction, or in FP64 where
+// the caller asked for that arithmetic (outer_arith = 0), rounded once at the end.
 // Bound by memory (r read, out written) and, in FP64, by its ~3 FP64 instructions per node. At 64^3 the
 // fused FP32 right-hand side takes 38 us; one thread per vertex of a line and component, with the moments
 // as double-float weights, took 101 us for B^T p alone, 49 us for the FP64 block now.
 enum BtMode { BT_PLAIN = 0, BT_RESID = 1 };
 
-template <typename TO> struct BtArith;
-template <> struct BtArith<double> {
+template <typename TO, bool DF>
+struct BtArith {
     using type = double;
     static __device__ __forceinline__ double in(double v) { return v; }
-    static __device__ __forceinline__ double out(double v) { return v; }
+    static __device__ __forceinline__ TO out(double v) { return TO(v); }
 };
-template <> struct BtArith<float> {
+template <> struct BtArith<float, true> {
     using type = q2::df64;
     static __device__ __forceinline__ q2::df64 in(double v) { return q2::split_double(v); }
     static __device__ __forceinline__ float out(const q2::df64& v) { return v.hi; }
 };
 
-template <int C, int MODE, typename TO>
-__device__ __forceinline__ void bt_store(const typename BtArith<TO>::type (&v)[3][3][3], double h, int e, int f, int g, int M,
+template <int C, int MODE, typename TO, bool DF>
+__device__ __forceinline__ void bt_store(const typename BtArith<TO, DF>::type (&v)[3][3][3], double h, int e, int f, int g, int M,
                                          const double* __restrict__ r, TO* __restrict__ out) {
-    using A = BtArith<TO>;
+    using A = BtArith<TO, DF>;
     using T = typename A::type;
     T b[8];
     bt_nodes<C>(v, b);
@@ -122,10 +123,10 @@ __device__ __forceinline__ void bt_store(const typename BtArith<TO>::type (&v)[3
             }
 }
 
-template <int MODE, typename TO>
+template <int MODE, typename TO, bool DF>
 __global__ void __launch_bounds__(128) k_bt(int n, double h, const double* __restrict__ p, const double* __restrict__ r,
                                             TO* __restrict__ out) {
-    using A = BtArith<TO>;
+    using A = BtArith<TO, DF>;
     const size_t cell = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (cell >= size_t(n) * n * n) return;
     const int e = int(cell % n), f = int((cell / n) % n), g = int(cell / (size_t(n) * n));
@@ -141,9 +142,9 @@ __global__ void __launch_bounds__(128) k_bt(int n, double h, const double* __res
                 const int a = max(e - 1 + i, 0), b = max(f - 1 + j, 0), c = max(g - 1 + k, 0);
                 v[k][j][i] = A::in(p[size_t(a) + size_t(P) * (b + size_t(P) * c)]);
             }
-    bt_store<0, MODE, TO>(v, h, e, f, g, M, r, out);
-    bt_store<1, MODE, TO>(v, h, e, f, g, M, r, out);
-    bt_store<2, MODE, TO>(v, h, e, f, g, M, r, out);
+    bt_store<0, MODE, TO, DF>(v, h, e, f, g, M, r, out);
+    bt_store<1, MODE, TO, DF>(v, h, e, f, g, M, r, out);
+    bt_store<2, MODE, TO, DF>(v, h, e, f, g, M, r, out);
 }
 
 // s_K = h^3 / mu_K per cell: the factor of the cell's pressure mass matrix (Section 2.2.2, the
@@ -371,7 +372,7 @@ cudaError_t launch_stokes_blocks(const LevelGeom& g, const double* mu, const dou
                                  double* dst_u, double* dst_p, bool do_a, bool do_bt, bool do_b, cudaStream_t s) {
     cudaError_t e;
     if (!do_a && do_bt && !do_b) {   // B^T alone: the gather, and the boundary rows
-        LAUNCH(PROF_BT_F64, s, (k_bt<BT_PLAIN, double><<<blocks_for(g.cells, 128), 128, 0, s>>>(g.n, g.h, src_p, nullptr, dst_u)));
+        LAUNCH(PROF_BT_F64, s, (k_bt<BT_PLAIN, double, false><<<blocks_for(g.cells, 128), 128, 0, s>>>(g.n, g.h, src_p, nullptr, dst_u)));
         return launch_zero_boundary<double>(g, dst_u, s);
     }
     if (do_a || do_bt) {
@@ -399,12 +400,15 @@ cudaError_t launch_mass_p(const LevelGeom& g, const double* mu, const double* sr
 }
 
 template <typename T>
-cudaError_t launch_bt_resid(const LevelGeom& g, const double* p, const double* r, T* out, cudaStream_t s) {
-    LAUNCH(PROF_BT_F64, s, (k_bt<BT_RESID, T><<<blocks_for(g.cells, 128), 128, 0, s>>>(g.n, g.h, p, r, out)));
+cudaError_t launch_bt_resid(const LevelGeom& g, const double* p, const double* r, T* out, bool df, cudaStream_t s) {
+    if (sizeof(T) == 4 && df)
+        LAUNCH(PROF_BT_F64, s, (k_bt<BT_RESID, T, sizeof(T) == 4><<<blocks_for(g.cells, 128), 128, 0, s>>>(g.n, g.h, p, r, out)));
+    else
+        LAUNCH(PROF_BT_F64, s, (k_bt<BT_RESID, T, false><<<blocks_for(g.cells, 128), 128, 0, s>>>(g.n, g.h, p, r, out)));
     return cudaGetLastError();
 }
-template cudaError_t launch_bt_resid<float>(const LevelGeom&, const double*, const double*, float*, cudaStream_t);
-template cudaError_t launch_bt_resid<double>(const LevelGeom&, const double*, const double*, double*, cudaStream_t);
+template cudaError_t launch_bt_resid<float>(const LevelGeom&, const double*, const double*, float*, bool, cudaStream_t);
+template cudaError_t launch_bt_resid<double>(const LevelGeom&, const double*, const double*, double*, bool, cudaStream_t);
 
 cudaError_t launch_mass_scale(const LevelGeom& g, const double* mu, double* scale, cudaStream_t s) {
     LAUNCH(PROF_MASS_P, s, k_mass_scale<<<blocks_for(g.cells, 256), 256, 0, s>>>(g.cells, g.h, mu, scale));
