@@ -53,12 +53,6 @@ using q2::df64;
 constexpr int kGsMaxK = 64;                 // largest basis of the double-float passes
 constexpr int kGsMaxBlocks = 2432;          // 16 per SM on 152 SMs; the partials buffer is sized for this
 
-// The second projection's coefficients c / alpha are of the size of the first one's rounding, about
-// 1e-13. Up to this size a product c v_i in single precision (relative error 2^-23) errs by less than
-// 2^-53 of v_i, the sum over 64 rows by less than 2^-47, the last bits of a double-float pair; above it
-// the products are double-float. That takes 11 of the 36 arithmetic instructions per basis entry out.
-constexpr double kSmallC = 9.31322574615478515625e-10;   // 2^-30
-
 enum GsMode { GS_DOT = 0, GS_PROJECT_DOT = 1, GS_PROJECT_SCALE = 2, GS_LAG = 3 };
 
 // An entry pair is handled by TPE adjacent lanes, each with RB basis rows (at most 16: with 32 rows
@@ -199,8 +193,8 @@ __global__ void __launch_bounds__(kGsThreads, RB <= 12 ? 4 : 3) k_gs_df(size_t n
                     q2::mac(s0, hs[r0 + r], df64(v[r].x, v[r].y));
                     q2::mac(s1, hs[r0 + r], df64(v[r].z, v[r].w));
                     const float c = hf[r0 + r];
-                    f0 = fmaf(c, v[r].x, f0);
-                    f1 = fmaf(c, v[r].z, f1);
+                    f0 = gs_small(c, v[r].x, f0);
+                    f1 = gs_small(c, v[r].z, f1);
                 }
 #pragma unroll
                 for (int o = 1; o < TPE; o <<= 1) {

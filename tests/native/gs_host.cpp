@@ -3,6 +3,7 @@
 #include <cstddef>
 #include <vector>
 
+#include "df64.cuh"
 #include "gs.cuh"
 
 // For rows of n entries, `blocks` CTAs and tpe threads to a pair: the first pair whose rows threads of more than one
@@ -26,4 +27,21 @@ extern "C" long long gs_shared_pair(size_t n, unsigned blocks, int tpe) {
     for (size_t p = 0; p < np; ++p)
         if (owner[p] < 0) return (long long)np;
     return -1;
+}
+
+extern "C" double gs_small_limit() { return stk::kSmallC; }
+
+// sum_i c[i] v[i] of one entry in the single-precision form of k_gs_df: lane g has rows g rb .. g rb + rb - 1, the
+// lanes' sums are added as its shuffles add them.
+extern "C" double gs_small_sum(int tpe, int rb, const double* c, const double* v) {
+    float lane[4] = {};
+    for (int g = 0; g < tpe; ++g)
+        for (int r = 0; r < rb; ++r)
+            lane[g] = stk::gs_small(float(c[g * rb + r]), q2::split_double(v[g * rb + r]).hi, lane[g]);
+    for (int o = 1; o < tpe; o <<= 1) {
+        float next[4];
+        for (int g = 0; g < tpe; ++g) next[g] = lane[g] + lane[g ^ o];
+        for (int g = 0; g < tpe; ++g) lane[g] = next[g];
+    }
+    return double(lane[0]);
 }
