@@ -94,9 +94,6 @@ cudaError_t launch_restrict(const LevelGeom& fine, const T* finev, T* coarse, cu
 template <typename T>
 cudaError_t launch_cheb_update(size_t n, const T* b, const T* Ax, const T* dinv, T* d, T* x, double c1, double c2,
                                bool x_valid, cudaStream_t s);
-// r = b - Ax
-template <typename T>
-cudaError_t launch_residual(size_t n, const T* b, const T* Ax, T* r, cudaStream_t s);
 // Zero the velocity entries on boundary nodes of a level vector.
 template <typename T>
 cudaError_t launch_zero_boundary(const LevelGeom& g, T* x, cudaStream_t s);

@@ -44,8 +44,6 @@ cudaError_t launch_outer_fix(const LevelGeom& g, const double* mu, const double*
         LAUNCH(PROF_STOKES_F64, s, (k_outer_fix<true, true, true><<<nb, kOuterThreads, 0, s>>>(a)));
     else if (do_a && !do_bt && !do_b)
         LAUNCH(PROF_VMULT_F64, s, (k_outer_fix<true, false, false><<<nb, kOuterThreads, 0, s>>>(a)));
-    else if (!do_a && do_bt && !do_b)
-        LAUNCH(PROF_BT_F64, s, (k_outer_fix<false, true, false><<<nb, kOuterThreads, 0, s>>>(a)));
     else if (!do_a && !do_bt && do_b)
         LAUNCH(PROF_STOKES_F64, s, (k_outer_fix<false, false, true><<<nb, kOuterThreads, 0, s>>>(a)));
     else

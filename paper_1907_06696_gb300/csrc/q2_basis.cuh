@@ -186,17 +186,7 @@ __host__ __device__ __forceinline__ void cell_A(T (&u)[3][27], T (&w)[3][27]) {
 
 // ---- B and B^T in the modes: a Q1 pressure with vertex values p0, p1 along an axis has the modes
 // P = p0 + p1, D = p1 - p0 (p = P/2 + D/2 P_1), and int v p = (w P + d D)/12, int v' p = d P/2 + e D/3.
-// So mode (i,j,k) of component C meets the pressure mode with index i - 1 along C and i elsewhere.
-template <int C>
-__host__ __device__ constexpr int mode_pressure(int i, int j, int k) {
-    const int b0 = i - (C == 0), b1 = j - (C == 1), b2 = k - (C == 2);
-    return (b0 < 0 || b0 > 1 || b1 < 0 || b1 > 1 || b2 < 0 || b2 > 1) ? -1 : b0 + 2 * b1 + 4 * b2;
-}
-template <int C>
-__host__ __device__ constexpr double mode_moment(int i, int j, int k) {
-    const int m[3] = {i, j, k};
-    return (m[C] == 1 ? 1.0 / 2.0 : 1.0 / 3.0) / 144.0;
-}
+// So mode (i,j,k) of component C meets the pressure mode with index i - 1 along C and i elsewhere (outer.cuh).
 // Vertex values -> pressure modes (in place), and the transpose.
 template <typename T>
 __host__ __device__ __forceinline__ void to_pressure_modes(T (&p)[8]) {
@@ -222,72 +212,6 @@ __host__ __device__ __forceinline__ void from_pressure_modes(T (&p)[8]) {
                 p[v + s] = a + b;
             }
 }
-// w += modes of int d_C(phi) p (B^T without -h^2); P += pressure modes of int d_C(u_C) psi (B without -h^2).
-template <int C, typename T>
-__host__ __device__ __forceinline__ void modes_BT(const T (&P)[8], T* w) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                const int q = mode_pressure<C>(i, j, k);
-                if (q >= 0) w[i + 3 * j + 9 * k] += T(mode_moment<C>(i, j, k) * mode_out(i, j, k)) * P[q < 0 ? 0 : q];
-            }
-}
-template <int C, typename T>
-__host__ __device__ __forceinline__ void modes_B(const T* U, T (&P)[8]) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                const int q = mode_pressure<C>(i, j, k);
-                if (q >= 0) P[q < 0 ? 0 : q] += T(mode_moment<C>(i, j, k)) * U[i + 3 * j + 9 * k];
-            }
-}
-
-// The blocks [A, B^T; B, 0] of one cell: in: u[c] nodal values (DO_A or DO_B; overwritten by their
-// modes), p vertex values times -h^2 (DO_BT; overwritten), sA = mu h; out: w = sA A u + B^T p
-// (DO_A or DO_BT), pb = B u without -h^2 (DO_B).
-template <bool DO_A, bool DO_BT, bool DO_B, typename T>
-__host__ __device__ __forceinline__ void cell_stokes(T (&u)[3][27], T (&p)[8], T sA, T (&w)[3][27], T (&pb)[8]) {
-    if (DO_A || DO_B) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) to_modes3(u[c]);
-    }
-    if (DO_B) {
-#pragma unroll
-        for (int v = 0; v < 8; ++v) pb[v] = T(0);
-        modes_B<0>(u[0], pb);
-        modes_B<1>(u[1], pb);
-        modes_B<2>(u[2], pb);
-        from_pressure_modes(pb);
-    }
-    if (DO_A) {
-        modes_A<0>(u[0], u[1], u[2], w[0]);
-        modes_A<1>(u[1], u[2], u[0], w[1]);
-        modes_A<2>(u[2], u[0], u[1], w[2]);
-    }
-    if (DO_A || DO_BT) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-#pragma unroll
-            for (int m = 0; m < 27; ++m) w[c][m] = DO_A ? w[c][m] * sA : T(0);
-    }
-    if (DO_BT) {
-        to_pressure_modes(p);
-        modes_BT<0>(p, w[0]);
-        modes_BT<1>(p, w[1]);
-        modes_BT<2>(p, w[2]);
-    }
-    if (DO_A || DO_BT) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) from_modes3(w[c]);
-    }
-}
-
 // 1D moments of the Q2 basis against the Q1 basis on [0,1], exact by the same
 // quadrature: VP(m,v) = int l_m psi_v, DP(m,v) = int l_m' psi_v.
 __host__ __device__ constexpr double VP(int m, int v) {

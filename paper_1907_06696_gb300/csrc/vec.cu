@@ -70,12 +70,6 @@ __global__ void k_cheb_update(size_t n, const T* __restrict__ b, const T* __rest
     }
 }
 
-template <typename T>
-__global__ void k_residual(size_t n, const T* __restrict__ b, const T* __restrict__ Ax, T* __restrict__ r) {
-    for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x)
-        r[i] = b[i] - Ax[i];
-}
-
 __global__ void k_cast_d2f(size_t n, const double* __restrict__ in, float* __restrict__ out) {
     for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x)
         out[i] = float(in[i]);
@@ -333,14 +327,6 @@ template cudaError_t launch_cheb_update<float>(size_t, const float*, const float
                                                double, double, bool, cudaStream_t);
 template cudaError_t launch_cheb_update<double>(size_t, const double*, const double*, const double*, double*,
                                                 double*, double, double, bool, cudaStream_t);
-
-template <typename T>
-cudaError_t launch_residual(size_t n, const T* b, const T* Ax, T* r, cudaStream_t s) {
-    LAUNCH(PROF_SMOOTH_VEC, s, k_residual<T><<<grid_stride_blocks(n), 256, 0, s>>>(n, b, Ax, r));
-    return cudaGetLastError();
-}
-template cudaError_t launch_residual<float>(size_t, const float*, const float*, float*, cudaStream_t);
-template cudaError_t launch_residual<double>(size_t, const double*, const double*, double*, cudaStream_t);
 
 cudaError_t launch_cast_d2f(size_t n, const double* in, float* out, cudaStream_t s) {
     LAUNCH(PROF_CAST, s, k_cast_d2f<<<grid_stride_blocks(n), 256, 0, s>>>(n, in, out));
