@@ -15,9 +15,15 @@ constexpr int kGsThreads = 128;
 __host__ __device__ __forceinline__ size_t gs_pair(size_t base, unsigned block, int thread, int tpe) {
     return base + size_t(block) * unsigned(kGsThreads / tpe) + unsigned(thread / tpe);
 }
-// Whether the thread reads the basis rows at its pair p of np where the pass writes one of them (GS_LAG, row j): past
-// the end there is nothing to read, the last pair is another thread's, which writes it in the same sweep.
-__host__ __device__ __forceinline__ bool gs_reads(size_t p, size_t np) { return p < np; }
+// The pair whose rows it reads: lanes past the last pair repeat that one, with w = 0.
+__host__ __device__ __forceinline__ size_t gs_read_pair(size_t p, size_t np) { return p < np - 1 ? p : np - 1; }
+// How many of its group's rows r0 .. r0 + rb - 1 it reads in a pass that writes row k - 1 of the k (GS_LAG): that row's
+// last pair is another thread's, which writes it in the same sweep, so a lane past the end leaves it alone. (Reading
+// no row at all there takes a predicate per row and entry pair: Krylov kernels of a 96^3 solve 341 -> 350 ms.)
+__host__ __device__ __forceinline__ int gs_read_rows(bool past_end, int k, int r0, int rb) {
+    const int n = k - r0 - (past_end ? 1 : 0);
+    return n < 0 ? 0 : (n < rb ? n : rb);
+}
 
 // The second projection's coefficients c / alpha are of the size of the first one's rounding, about 1e-13. While all
 // of them are at most kSmallC, sum_i c_i v_i over the k <= 64 rows is formed in single precision from the rows' high

@@ -58,11 +58,11 @@ enum GsMode { GS_DOT = 0, GS_PROJECT_DOT = 1, GS_PROJECT_SCALE = 2, GS_LAG = 3 }
 // An entry pair is handled by TPE adjacent lanes, each with RB basis rows (at most 16: with 32 rows
 // per thread, or with 8 and 4 and more threads per pair, whole solves are slower). The shape is the
 // smallest that holds k rows (gs_shapes); every lane runs its RB rows without tests: rows past the
-// k-th are zero with zero coefficients, lanes past the last pair repeat it (GS_LAG: load nothing, gs_reads) with
-// w = 0. (One test per row and entry pair cost as many instructions as the arithmetic.) Measured at 48^3 with 24
-// rows of 2.9 M entries: dot products 91 us, 6.3 TB/s; GS_LAG 114 us, bound by the arithmetic of its two
-// double-float products per entry (134 and 210 us with tests and with the rows passing through shared
-// memory). 16 rows per thread at most: 168 registers, three CTAs per SM; up to 12 rows four.
+// k-th are zero with zero coefficients, lanes past the last pair repeat it with w = 0 (gs.cuh). (One
+// test per row and entry pair cost as many instructions as the arithmetic.) Measured at 48^3 with 24 rows of 2.9 M
+// entries: dot products 91 us, 6.3 TB/s; GS_LAG 114 us, bound by the arithmetic of its two double-float
+// products per entry (134 and 210 us with tests and with the rows passing through shared memory). 16 rows
+// per thread at most: 168 registers, three CTAs per SM; up to 12 rows four.
 struct GsShapeId { int tpe, rb; };
 constexpr GsShapeId kGsShapes[] = {{1, 4}, {1, 8}, {1, 12}, {1, 16}, {2, 12}, {2, 16}, {4, 10}, {4, 12}, {4, 14}, {4, 16}};
 constexpr int kGsShapeCount = int(sizeof(kGsShapes) / sizeof(kGsShapes[0]));
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(kGsThreads, RB <= 12 ? 4 : 3) k_gs_df(size_t n
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int g = tid % TPE;              // row group: rows r0 .. r0 + RB - 1
     const int r0 = g * RB;
-    const int nr = max(0, min(RB, k - r0));   // rows of the group below k
+    const int nr = gs_read_rows(false, k, r0, RB);   // rows of the group below k
     constexpr int NH = MODE == GS_LAG ? 3 : 1;
     df64* hs = reinterpret_cast<df64*>(smem);               // split coefficients
     df64* hb = hs + KB;                                     // GS_LAG: those of v_j
@@ -163,13 +163,14 @@ __global__ void __launch_bounds__(kGsThreads, RB <= 12 ? 4 : 3) k_gs_df(size_t n
     load_w(p0, wn0, wn1);
     for (int it = 0; warp_first + base < np; ++it) {
         const size_t p = p0 + base;
-        const bool in = gs_reads(p, np);
+        const bool in = p < np;
         const bool in1 = 2 * p + 1 < n;
         {
-            const double* src = V + 2 * (MODE == GS_LAG ? p : min(p, np - 1)) + size_t(r0) * ld;
+            const double* src = V + 2 * gs_read_pair(p, np) + size_t(r0) * ld;
+            const int rows = MODE == GS_LAG ? gs_read_rows(!in, k, r0, RB) : nr;
 #pragma unroll
             for (int r = 0; r < RB; ++r) {
-                if (r < nr && (MODE != GS_LAG || in)) v[r] = load_pairs(src);
+                if (r < rows) v[r] = load_pairs(src);
                 src += ld;
             }
         }

@@ -6,26 +6,31 @@
 #include "df64.cuh"
 #include "gs.cuh"
 
-// For rows of n entries, `blocks` CTAs and tpe threads to a pair: the first pair whose rows threads of more than one
-// group of tpe, or of more than one sweep, read, np if a pair is left out, -1 if each is read by its own group only.
-extern "C" long long gs_shared_pair(size_t n, unsigned blocks, int tpe) {
+// For k rows of n entries, `blocks` CTAs, tpe threads to a pair and rb rows to a thread: the first pair of row k - 1 that
+// threads of more than one group of tpe, or in more than one sweep, read; np if some pair of some row is left
+// out or something past the rows or pairs is read; -1 if neither.
+extern "C" long long gs_shared_pair(size_t n, unsigned blocks, int tpe, int rb, int k) {
     using namespace stk;
     const size_t np = (n + 1) / 2, stride = size_t(blocks) * unsigned(kGsThreads / tpe);
-    std::vector<long long> owner(np, -1);
+    std::vector<long long> owner(np, -1);         // of row k - 1's pairs
+    std::vector<char> seen(np * size_t(k), 0);   // pairs of all rows
     for (unsigned b = 0; b < blocks; ++b)
         for (int t = 0; t < kGsThreads; ++t) {
             const size_t warp_first = gs_pair(0, b, t / 32 * 32, tpe);
             for (size_t base = 0; warp_first + base < np; base += stride) {
                 const size_t p = gs_pair(base, b, t, tpe);
-                if (!gs_reads(p, np)) continue;
-                if (p >= np) return (long long)np;
+                const size_t rp = gs_read_pair(p, np);
+                const int r0 = t % tpe * rb, rows = gs_read_rows(p >= np, k, r0, rb);
+                if (rp >= np || r0 + rows > k) return (long long)np;
+                for (int r = 0; r < rows; ++r) seen[size_t(r0 + r) * np + rp] = 1;
+                if (r0 + rows < k || rows == 0) continue;
                 const long long who = (long long)((base / stride * blocks + b) * kGsThreads + t / tpe);
-                if (owner[p] >= 0 && owner[p] != who) return (long long)p;
-                owner[p] = who;
+                if (owner[rp] >= 0 && owner[rp] != who) return (long long)rp;
+                owner[rp] = who;
             }
         }
-    for (size_t p = 0; p < np; ++p)
-        if (owner[p] < 0) return (long long)np;
+    for (char s : seen)
+        if (!s) return (long long)np;
     return -1;
 }
 
