@@ -156,7 +156,7 @@ KERNEL_SOURCES = {
     "stokes_fixed": ("q2_basis.cuh", "outer.cuh", "outer.cu"),
     "stokes_fixed_inst": ("q2_basis.cuh", "outer.cuh", "outer.cu"),
     "vmult_A_fp32": ("q2_basis.cuh", "brick.cuh", "march.cu"),
-    "krylov_vec": ("krylov.cu", "vec.cu"),
+    "krylov_vec": ("krylov.cu", "gs.cuh", "vec.cu"),
 }
 
 

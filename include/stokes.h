@@ -449,8 +449,8 @@ stokes_status stokes_schur_inverse_noalloc(int n, const double* mu_dev, const do
 /* Kernel classes timed by stokes_profile: 0 velocity cell kernel FP32, 1 velocity
  * cell kernel FP64, 2 fused A+B^T+B cell kernel, 3 B^T cell kernel, 4 pressure mass
  * cell kernel, 5 transfers, 6 smoother / residual vector kernels, 7 Krylov vector
- * kernels, 8 coarse solve, 9 precision casts, 10 the outer operator applied for the solvers' residuals
- * for the solvers' restart and final residuals (uniform meshes). */
+ * kernels, 8 coarse solve, 9 precision casts, 10 the outer operator for the solvers' restart and final
+ * residuals (uniform meshes). */
 #define STOKES_PROF_NCLASS 11
 /* enable = 1: record a CUDA event pair around every kernel launch the library
  * issues from now on (adds two event records per launch); 0: stop. Process-wide,

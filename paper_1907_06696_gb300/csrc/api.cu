@@ -301,10 +301,11 @@ double tridiag_max_eig(const std::vector<double>& a, const std::vector<double>& 
 // Level-operator selector for launch_level_op: 1 = brick kernel, 2 = tensor-core brick kernel,
 // 3 = component-split kernel (FP32 levels), else the cell kernel's block size. By default the smallest and the
 // largest FP32 levels take the operators with the epilogue in the same launch:
-// - at most kBlockMaxN cells per axis: blocks of 2 x 2 x 2 cells (block.cu). With the limit at 24 cells 20^3 takes 132
-//   instead of 125 us and 24^3 181 instead of 146: its blocks compute 27 cells for 8 that they own;
-// - from kMarchMinN up: tiles that march over layers (march.cu), 197 / 528 / 1,196 us at 64^3 / 96^3 / 128^3 (cell
-//   kernel and vector passes 208 / 702 / 1,624 us); below, the layers are too few to hide one layer's latency;
+// - at most kBlockMaxN cells per axis: blocks of 2 x 2 x 2 cells (block.cu). With the limit at 24 cells a V-cycle at 20^3
+//   takes 132 instead of 125 us and at 24^3 181 instead of 146: its blocks compute 27 cells for 8 that they own;
+// - from kMarchMinN up: tiles that march over layers (march.cu), a degree-4 smoothing takes 197 / 528 / 1,196 us at
+//   64^3 / 96^3 / 128^3 (cell kernel and vector passes 208 / 702 / 1,624 us). Below, the layers are too few to hide one
+//   layer's latency: V-cycle at 48^3 341 us marching, 330 us here; 40^3 281 and 264, 32^3 262 and 234 us;
 // - between them the cell kernel and vector passes.
 constexpr int kBlockMaxN = 16, kMarchMinN = 64;
 
@@ -733,25 +734,25 @@ stokes_status schur_inverse(stokes_ctx* c, const double* rp, double* zp, cudaStr
     return STOKES_OK;
 }
 
-// dst = K src. native: FP64 arithmetic whatever outer_arith says; the solvers use it for the
-// residuals b - K x they restart from and report, so that the ~2^-47 relative rounding of the
-// double-float operator (amplified by the viscosity contrast) enters only the Krylov recurrences,
-// which the restarts correct like iterative refinement.
-stokes_status apply_stokes(stokes_ctx* c, const double* src, double* dst, cudaStream_t s, bool native = false) {
+// dst = K src. resid: for the residuals b - K x that the solvers restart from and report, a profile class of its own
+// and the FP64-accurate operator of outer_arith 0 and 1 with outer_arith 2 too (whose digit slices are recombined in
+// double-float: 2^-47, amplified by the viscosity contrast, enters only the Krylov recurrences, which the restarts
+// correct like iterative refinement).
+stokes_status apply_stokes(stokes_ctx* c, const double* src, double* dst, cudaStream_t s, bool resid = false) {
     if (c->oct) {
         const size_t nu = 3 * c->oct->act.nu_nodes;
         CK(launch_oct_active(c->oct->act, src, src + nu, dst, dst + nu, true, true, true, s));
         return STOKES_OK;
     }
     Level& F = c->lev[c->L - 1];
-    if (!native && c->opt.outer_arith == 2 && c->outer_tc_table) {   // exact digit slices on the tensor cores
+    if (!resid && c->opt.outer_arith == 2 && c->outer_tc_table) {   // exact digit slices on the tensor cores
         CK(cudaMemsetAsync(dst, 0, (F.g.n_u + F.g.n_p) * sizeof(double), s));
         CK(launch_outer_tc(F.g, F.v64.mu, src, src + F.g.n_u, dst, dst + F.g.n_u, c->outer_tc_table, c->tc.status,
                            c->tc.wait_ns, s));
         CK(launch_copy_boundary<double>(F.g, src, dst, s));   // identity rows
         return STOKES_OK;
     }
-    if (native) prof_override(PROF_RESID_F64);
+    if (resid) prof_override(PROF_RESID_F64);
     const cudaError_t e = launch_stokes_blocks(F.g, F.v64.mu, src, src + F.g.n_u, dst, dst + F.g.n_u, true, true, true, s);
     prof_override(-1);
     CK(e);

@@ -424,7 +424,7 @@ cudaError_t launch_cell_tc(const BrickArgs<float>& a, float* acc, const TcArgs& 
 constexpr int kMarchKernel = 4;
 cudaError_t launch_march(int epi, const LevelGeom& g, const float* mu, const float* src, float* dst, const float* b,
                          const float* dinv, const float* d, float* d_new, double c1, double c2, cudaStream_t s);
-// The same on levels of any size in blocks of 4 x 4 x 4 cells (block.cu), no alignment asked; entries on the
+// The same on levels of any size in blocks of 2 x 2 x 2 owned cells (block.cu), no alignment asked; entries on the
 // domain boundary are left as they are. EPI_CHEB with src null: the first step from zero is pending,
 // src = d = c0 dinv b.
 constexpr int kBlockKernel = 5;

@@ -363,7 +363,8 @@ struct OctRefs {
 // operator on as many cells takes some 60.
 // On meshes of at most one block per SM the time is that of the block with the most hanging nodes (up to 600,
 // 20 rounds of 32 lanes): there GROUPS - 1 more warps per component take part in those rounds alone. Stokes operator on 3,431
-// leaves 49.2 -> 32.8 us, with the Dirichlet flags folded into the tables; that alone on 79,080 leaves 149 -> 132 us.
+// leaves 49.2 -> 32.8 us, with the Dirichlet flags folded into the tables; that alone took this kernel (without the
+// clearing and the boundary rows) on 79,080 leaves from 149 to 132 us, the operator to 146 us.
 template <bool DO_A, bool DO_BT, bool DO_B, int GROUPS>
 __global__ void __launch_bounds__(kOuterThreads * GROUPS, GROUPS == 1 ? 5 : 1)
     k_oct_active(OctActiveDev a, const double* __restrict__ src_u, const double* __restrict__ src_p, double* __restrict__ dst_u,

@@ -18,7 +18,7 @@ enum ProfClass {
     PROF_KRYLOV = 7,      // multi-dot, multi-axpy, axpby, norms
     PROF_COARSE = 8,      // coarse solve
     PROF_CAST = 9,        // precision casts
-    PROF_RESID_F64 = 10,  // outer operator for the solvers' restart and final residuals (native FP64)
+    PROF_RESID_F64 = 10,  // outer operator for the solvers' restart and final residuals
     PROF_NCLASS = 11
 };
 
