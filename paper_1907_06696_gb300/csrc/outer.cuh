@@ -11,7 +11,7 @@
 //   97200 A is an integer matrix in the modes (stiffness (0,3,4)/3, mass (5,15,4)/180, derivative
 //       couplings (1,2)/6): Y = 97200 A U, |Y| <= 2^(54 + 15.99), formed in 96 bits and kept without
 //       its lowest 12;
-//   B^T p is added as (3|2) p' with p' = 112.5 h/mu p in the same units;
+//   B^T p is added as (3|2) p' with p' = 112.5 h/mu p in the same units (fix_factor);
 //   the transposed transform gives |result| < 2^(42 + 20.43) (sums that leave 64 bits on the way
 //       return: two's complement), rounded to 53 bits and multiplied by mu h 2^E / 97200.
 // B u is (3|2) U / 864 without its lowest 2 bits, |result| <= 2^(52 + 10.1).
@@ -20,7 +20,8 @@
 // in double-float pairs 6.4e-15 and 3.6e-14), against the size of the cell's values: a value far below its
 // cell's largest keeps the bits above 2^-55 of that one. With nodal values over 8 decades at random within every cell
 // (4^3) the error is 1.6e-16 in the 2-norm and 4e-14 of (|A| |u|) in the worst row; sum factorisation in FP64, which mixes a
-// cell's values too, 3.2e-16 and 1.5e-14.
+// cell's values too, 3.2e-16 and 1.5e-14. Where B^T p is the larger term (|p| 1e4 and 1e6, 3^3 to 8^3 cells) 1.5e-16 to
+// 2.6e-16 in the 2-norm; in FP64 2.1e-16 to 2.8e-16.
 //
 // A CTA holds 32 cells and 96 threads; warp c owns velocity component c of
 // the 32 cells (lane g = cell g) and the three exchange their modes through shared memory (20.7 KB).
@@ -90,6 +91,13 @@ __host__ __device__ __forceinline__ long long mul_hi(long long a, long long b) {
     return (long long)(((__int128)a * b) >> 64);
 #endif
 }
+__host__ __device__ __forceinline__ unsigned long long mul_hi_u(unsigned long long a, unsigned long long b) {
+#ifdef __CUDA_ARCH__
+    return __umul64hi(a, b);
+#else
+    return (unsigned long long)(((unsigned __int128)a * b) >> 64);
+#endif
+}
 __host__ __device__ __forceinline__ int clz_u64(unsigned long long x) {   // x > 0
 #ifdef __CUDA_ARCH__
     return __clzll((long long)x);
@@ -120,17 +128,43 @@ __host__ __device__ __forceinline__ double fix_out(long long x, double scale) {
     const long long b = a ? m + ((long long)(1085 - lz) << 52) : 0;   // m in [2^52, 2^53]: |x| = m 2^(11 - lz)
     return bits_to_dbl(b | (sign & (long long)(1ull << 63))) * scale;
 }
-// s 2^e, |e| < 2044; NaN where the cell holds one (or an infinity). A pressure against a large or small viscosity can
-// take 2^e alone out of the FP64 range: two factors.
+// s 2^e, |e| < 3066; NaN where the cell holds one (or an infinity). A pressure against a large or small viscosity can
+// take 2^e alone out of the FP64 range: three factors.
 __host__ __device__ __forceinline__ double fix_scale(double s, int e, bool zero, bool bad) {
     if (bad) return bits_to_dbl(0x7FF8000000000000LL);
     if (zero) return 0.0;
     int k = 0;
     if (e < -1022 || e > 1023) {
-        k = e / 2;
-        s *= bits_to_dbl((long long)(k + 1023) << 52);
+        k = e / 3;
+        const double f = bits_to_dbl((long long)(k + 1023) << 52);
+        s = s * f * f;
+        k *= 2;
     }
     return s * bits_to_dbl((long long)(e - k + 1023) << 52);
+}
+// B^T's factor (h^2 / 864) / s = km 2^(ek - 1084), km in [2^61, 2^62), to 2^-57. The result is multiplied by s, whose
+// roundings would be the whole cell's if the factor did not take them back. In integers (Newton's iteration for 1/s
+// from a single-precision start): the Stokes operator takes 23.6 us at 20^3 and 197 us at 64^3, 23.6 and 195 us with an
+// FP64 division and its rounding; the division with its remainder in FP64 took 26.6 instead of 24.6 us at 20^3.
+__host__ __device__ __forceinline__ long long fix_factor(double s, double h, int& ek) {
+    const unsigned long long one = 1ull << 52;
+    const long long sb = (long long)q2::dbl_bits(s), hb = (long long)q2::dbl_bits(h);
+    const unsigned long long sm = (unsigned long long)(sb & (long long)(one - 1)) | (exp_of(sb) ? one : 0ull);
+    const int lz = sm ? clz_u64(sm) : 0;                       // 11, more where s is subnormal
+    const unsigned long long S = sm << lz;                     // s = S 2^(es - 1086)
+    const int es = (exp_of(sb) ? exp_of(sb) : 1) + 11 - lz;
+    unsigned long long X = (unsigned long long)(0x1p125f / float(S));   // 2^125 / S
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const long long err = (long long)((1ull << 61) - mul_hi_u(S, X));
+        X += (unsigned long long)mul_hi((long long)X, err << 3);
+    }
+    const unsigned long long H = ((unsigned long long)(hb & (long long)(one - 1)) | one) << 11;
+    const unsigned long long T = mul_hi_u(mul_hi_u(H, H), 0x97B425ED097B425Eull);   // 2^68 / 27
+    const unsigned long long K = mul_hi_u(T, X);               // in [2^58, 2^62)
+    const int sh = K ? clz_u64(K) - 2 : 0;
+    ek = 2 * exp_of(hb) - es - sh - 8;
+    return (long long)(K << sh);
 }
 // A 96-bit sum of products of modes with non-negative table entries below 2^12: high and low words apart.
 struct FixSum {
@@ -323,24 +357,25 @@ __host__ __device__ __forceinline__ double outer_velocity(int C, int g, const Ou
                 }
                 Y[m] = y.shifted();
             }
+    const double s = mu * h * (1.0 / 97200.0);
     const int eu0 = DO_A && eu >= kFixMinExp ? eu : kFixNone;
     int E = eu0;
     bool bad = DO_A && eu == 0x7FF;
     if (DO_BT) {
-        // p' = 112.5 h/mu p: the vertex modes times the factor's significand, |R| <= 2^61; |p'| < 2^(epk - 1022)
+        // p' = 112.5 h/mu p: the vertex modes times the factor's significand, |R| <= 2^60; |p'| < 2^(epk - 1022)
         // may exceed |u| by 2^10 before its share of the result is the larger one
         const int ep = max3(sh.ep, g);
         if (ep >= kFixMinExp) {
-            const long long kb = (long long)q2::dbl_bits(112.5 * h / mu);
-            const long long km = ((kb & 0xFFFFFFFFFFFFFLL) | (1LL << 52)) << 10;
-            const int epk = ep + exp_of(kb) - 1022;
+            int ek;
+            const long long km = fix_factor(s, h, ek);
+            const int epk = ep + ek - 1022;
             E = E > epk - 10 ? E : epk - 10;
             long long P[8];
 #pragma unroll
             for (int v = 0; v < 8; ++v)
                 P[v] = sh.P[((v & 1) << C) + (((v >> 1) & 1) << D1) + ((v >> 2) << D2)][g];
             q2::to_pressure_modes(P);
-            const int sp = E - epk + 16 < 63 ? E - epk + 16 : 63;
+            const int sp = E - epk + 15 < 63 ? E - epk + 15 : 63;
             const int sa = DO_A ? (E - eu0 < 63 ? E - eu0 : 63) : 0;
             if (sa > 0) {
 #pragma unroll
@@ -357,7 +392,7 @@ __host__ __device__ __forceinline__ double outer_velocity(int C, int g, const Ou
     fix_from_modes<2>(Y);
     fix_from_modes<1>(Y);
     fix_from_modes<0>(Y);
-    return fix_scale(mu * h * (1.0 / 97200.0), E - 1022 - kFixBits + kFixMid, E == kFixNone, bad);
+    return fix_scale(s, E - 1022 - kFixBits + kFixMid, E == kFixNone, bad);
 }
 
 // Phase 1b (after a barrier): fixed point and modes.
