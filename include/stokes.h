@@ -120,7 +120,7 @@ typedef struct {
                                    tcgen05.mma with FP32 accumulation, exact because every partial sum
                                    is an integer below 2^24), recombined in double-float and written
                                    as FP64 with integer instructions; every other block and the
-                                   Krylov basis as in 1. Not the default: 832 us at 64^3 against 195 us for 1. */
+                                   Krylov basis as in 1. Not the default: 832 us at 64^3 against 197 us for 1. */
     int vmult_kernel;           /* level operator of the V-cycle: 0 = by level size (default): FP32 levels of at
                                    most 16^3 cells in blocks of 2^3 cells and those from 64^3 up in tiles
                                    that march over layers, both with the epilogue inside; between them

@@ -21,7 +21,8 @@
 // cell's largest keeps the bits above 2^-55 of that one. With nodal values over 8 decades at random within every cell
 // (4^3) the error is 1.6e-16 in the 2-norm and 4e-14 of (|A| |u|) in the worst row; sum factorisation in FP64, which mixes a
 // cell's values too, 3.2e-16 and 1.5e-14. Where B^T p is the larger term (|p| 1e4 and 1e6, 3^3 to 8^3 cells) 1.5e-16 to
-// 2.6e-16 in the 2-norm; in FP64 2.1e-16 to 2.8e-16.
+// 2.6e-16 in the 2-norm; in FP64 2.1e-16 to 2.8e-16. On octrees of 4,635 and 15,548 leaves (viscosity ratio 1e6, against
+// sums in extended precision) 1.8e-16; in FP64 3.7e-16.
 //
 // A CTA holds 32 cells and 96 threads; warp c owns velocity component c of
 // the 32 cells (lane g = cell g) and the three exchange their modes through shared memory (20.7 KB).
