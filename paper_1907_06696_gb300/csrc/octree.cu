@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(kOuterThreads, 5)
     __syncthreads();
     if (first + g >= size_t(L.n_cells)) return;
     long long Y[27];
-    const double s = outer_velocity<true, false>(C, g, sh, mu[first + g], L.h, Y);
+    const FixScale s = outer_velocity<true, false>(C, g, sh, mu[first + g], L.h, Y);
 #pragma unroll
     for (int m = 0; m < 27; ++m) {
         const int32_t v = node[(m % 3) * q0 + (m / 3 % 3) * q1 + (m / 9) * q2][g];
@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(kOuterThreads * GROUPS, GROUPS == 1 ? 5 : 1)
     const double h = valid ? ldexp(1.0, -int(a.level[leaf])) : 1.0;
     if (DO_B && valid) {
         long long b[8];
-        const double s = outer_pressure(C, g, sh, h, b);
+        const FixScale s = outer_pressure(C, g, sh, h, b);
         const int v1 = 1 << C, v6 = 7 - v1;   // as in outer_phase2: each vertex by one warp
         scatter_p(a, dst_p, rp[v1], fix_out(b[1], s), size_t(leaf) * 8 + v1);
         scatter_p(a, dst_p, rp[v6], fix_out(b[6], s), size_t(leaf) * 8 + v6);
@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(kOuterThreads * GROUPS, GROUPS == 1 ? 5 : 1)
     }
     if (DO_A || DO_BT) {
         long long Y[27];
-        double s = 0.0;
+        FixScale s;
         if (main) s = outer_velocity<DO_A, DO_BT>(C, g, sh, valid ? a.mu[leaf] : 1.0, h, Y);
         __syncthreads();   // every warp has read the modes
         if (main) {

@@ -73,7 +73,8 @@ __host__ __device__ __forceinline__ void outer_atomic_add(double* p, double v) {
 // ---- fixed point
 constexpr int kFixBits = 54;      // |X| <= 2^54
 constexpr int kFixMid = 12;       // bits dropped after the element matrix
-constexpr int kFixMinExp = 64;    // cells whose largest value is below 2^-958 read as 0
+constexpr int kFixMinExp = 64;    // below this largest exponent a zero does not fall out of fix_round by itself
+constexpr int kFixLift = 128;     // such cells are read times 2^128; subnormal values read as 0
 constexpr int kFixNone = -4096;   // exponent of a cell that reads as 0
 
 __host__ __device__ __forceinline__ double bits_to_dbl(long long b) {
@@ -109,7 +110,7 @@ __host__ __device__ __forceinline__ int clz_u64(unsigned long long x) {   // x >
 __host__ __device__ __forceinline__ int exp_of(long long bits) { return int(bits >> 52) & 0x7FF; }
 
 // X = round(v 2^(54 - E)) for the FP64 bits of v, |v| < 2^E with E = emax - 1022 (emax >= kFixMinExp,
-// the largest biased exponent of the cell). Zero, and what is below 2^-60 of the largest, gives 0.
+// the largest biased exponent of the cell; cells below that: fix_lift). Zero, and what is below 2^-60 of the largest, gives 0.
 __host__ __device__ __forceinline__ long long fix_round(long long bits, int emax) {
     const unsigned long long m = (unsigned long long)(bits & 0xFFFFFFFFFFFFFLL) << 2 | (1ull << 54);
     const int r = emax - exp_of(bits);
@@ -119,21 +120,31 @@ __host__ __device__ __forceinline__ long long fix_round(long long bits, int emax
 }
 
 // x scale with x rounded to 53 bits (half up), |x| < 2^63: the significand is placed by integer
-// instructions, one FP64 multiplication.
-__host__ __device__ __forceinline__ double fix_out(long long x, double scale) {
+// instructions (from exponent scale.base), one FP64 multiplication.
+struct FixScale {
+    double s = 0.0;
+    int base = 1085;
+};
+__host__ __device__ __forceinline__ double fix_out(long long x, const FixScale& scale) {
     const long long sign = x >> 63;
     const unsigned long long a = (unsigned long long)((x ^ sign) - sign);
     const int lz = a ? clz_u64(a) : 0;
     const unsigned long long v = a << lz;
     const long long m = (long long)((v >> 11) + ((v >> 10) & 1));
-    const long long b = a ? m + ((long long)(1085 - lz) << 52) : 0;   // m in [2^52, 2^53]: |x| = m 2^(11 - lz)
-    return bits_to_dbl(b | (sign & (long long)(1ull << 63))) * scale;
+    const long long b = a ? m + ((long long)(scale.base - lz) << 52) : 0;   // m in [2^52, 2^53]: |x| = m 2^(11 - lz)
+    return bits_to_dbl(b | (sign & (long long)(1ull << 63))) * scale.s;
 }
 // s 2^e, |e| < 3066; NaN where the cell holds one (or an infinity). A pressure against a large or small viscosity can
-// take 2^e alone out of the FP64 range: three factors.
-__host__ __device__ __forceinline__ double fix_scale(double s, int e, bool zero, bool bad) {
-    if (bad) return bits_to_dbl(0x7FF8000000000000LL);
-    if (zero) return 0.0;
+// take 2^e alone out of the FP64 range: three factors. For small values fix_out places |x| < 2^63 below 2, so that
+// the factor is a normal number where the results can be.
+__host__ __device__ __forceinline__ FixScale fix_scale(double s, int e, bool zero, bool bad) {
+    FixScale r;
+    if (bad) r.s = bits_to_dbl(0x7FF8000000000000LL);
+    if (bad || zero) return r;
+    if (e < -500) {
+        r.base -= 62;
+        e += 62;
+    }
     int k = 0;
     if (e < -1022 || e > 1023) {
         k = e / 3;
@@ -141,7 +152,12 @@ __host__ __device__ __forceinline__ double fix_scale(double s, int e, bool zero,
         s = s * f * f;
         k *= 2;
     }
-    return s * bits_to_dbl((long long)(e - k + 1023) << 52);
+    r.s = s * bits_to_dbl((long long)(e - k + 1023) << 52);
+    return r;
+}
+// The FP64 bits of a value of a cell with largest exponent emax < kFixMinExp, times 2^128.
+__host__ __device__ __forceinline__ long long fix_lift(long long bits) {
+    return exp_of(bits) ? bits + ((long long)kFixLift << 52) : 0;
 }
 // B^T's factor (h^2 / 864) / s = km 2^(ek - 1084), km in [2^61, 2^62), to 2^-57. The result is multiplied by s, whose
 // roundings would be the whole cell's if the factor did not take them back. In integers (Newton's iteration for 1/s
@@ -301,9 +317,19 @@ __host__ __device__ __forceinline__ int max3(const int (&e)[3][kOuterCells], int
 // This thread's component (raw FP64 bits T) in fixed point against the cell's largest magnitude, and its
 // modes; every third pressure value (sh.P) in fixed point. After the barrier behind sh.eu and sh.ep.
 template <bool DO_U, bool DO_P, typename V>
-__host__ __device__ __forceinline__ void outer_modes(int C, int g, OuterShared& sh, const V (&T)[27]) {
+__host__ __device__ __forceinline__ void outer_modes(int C, int g, OuterShared& sh, V (&T)[27]) {
     if (DO_U) {
-        const int e = max3(sh.eu, g);
+        int e = max3(sh.eu, g);
+        if (e < kFixMinExp) {
+            e += kFixLift;
+#pragma unroll
+            for (int m = 0; m < 27; ++m) {
+                long long b;
+                memcpy(&b, &T[m], 8);
+                b = fix_lift(b);
+                memcpy(&T[m], &b, 8);
+            }
+        }
         long long X[27];
 #pragma unroll
         for (int m = 0; m < 27; ++m) {
@@ -319,13 +345,14 @@ __host__ __device__ __forceinline__ void outer_modes(int C, int g, OuterShared& 
     }
     if (DO_P) {
         const int e = max3(sh.ep, g);
-        for (int v = C; v < 8; v += 3) sh.P[v][g] = fix_round(sh.P[v][g], e);
+        for (int v = C; v < 8; v += 3)
+            sh.P[v][g] = e < kFixMinExp ? fix_round(fix_lift(sh.P[v][g]), e + kFixLift) : fix_round(sh.P[v][g], e);
     }
 }
 
 // B u of a cell of side h at its vertices (warp C's frame: bit d of the index along global axis C + d), as
 // b scale. After the barrier behind outer_modes.
-__host__ __device__ __forceinline__ double outer_pressure(int C, int g, const OuterShared& sh, double h, long long (&b)[8]) {
+__host__ __device__ __forceinline__ FixScale outer_pressure(int C, int g, const OuterShared& sh, double h, long long (&b)[8]) {
     const int D1 = (C + 1) % 3, D2 = (C + 2) % 3, eu = max3(sh.eu, g);
 #pragma unroll
     for (int v = 0; v < 8; ++v) {
@@ -334,13 +361,13 @@ __host__ __device__ __forceinline__ double outer_pressure(int C, int g, const Ou
                ((3 - k) * sh.U[D2][(k + 1) + 3 * i + 9 * j][g] >> 2);
     }
     q2::from_pressure_modes(b);
-    return fix_scale(-h * h / 864.0, eu - 1022 - kFixBits + 2, eu < kFixMinExp, eu == 0x7FF);
+    return fix_scale(-h * h / 864.0, eu - 1022 - kFixBits + 2, eu == 0, eu == 0x7FF);
 }
 
 // Component C of A u + B^T p of a cell of side h and viscosity mu, in warp C's frame, as Y scale.
 template <bool DO_A, bool DO_BT>
-__host__ __device__ __forceinline__ double outer_velocity(int C, int g, const OuterShared& sh, double mu, double h,
-                                                          long long (&Y)[27]) {
+__host__ __device__ __forceinline__ FixScale outer_velocity(int C, int g, const OuterShared& sh, double mu, double h,
+                                                            long long (&Y)[27]) {
     const int D1 = (C + 1) % 3, D2 = (C + 2) % 3;
     const int eu = DO_A ? max3(sh.eu, g) : 0;
 #pragma unroll
@@ -359,14 +386,14 @@ __host__ __device__ __forceinline__ double outer_velocity(int C, int g, const Ou
                 Y[m] = y.shifted();
             }
     const double s = mu * h * (1.0 / 97200.0);
-    const int eu0 = DO_A && eu >= kFixMinExp ? eu : kFixNone;
+    const int eu0 = DO_A && eu > 0 ? eu : kFixNone;
     int E = eu0;
     bool bad = DO_A && eu == 0x7FF;
     if (DO_BT) {
         // p' = 112.5 h/mu p: the vertex modes times the factor's significand, |R| <= 2^60; |p'| < 2^(epk - 1022)
         // may exceed |u| by 2^10 before its share of the result is the larger one
         const int ep = max3(sh.ep, g);
-        if (ep >= kFixMinExp) {
+        if (ep > 0) {
             int ek;
             const long long km = fix_factor(s, h, ek);
             const int epk = ep + ek - 1022;
@@ -399,7 +426,7 @@ __host__ __device__ __forceinline__ double outer_velocity(int C, int g, const Ou
 // Phase 1b (after a barrier): fixed point and modes.
 template <bool DO_A, bool DO_B = true, bool DO_BT = true, typename V>
 __host__ __device__ __forceinline__ void outer_phase1b(const OuterArgs&, int C, int, int g, OuterShared& sh,
-                                                       const V (&T)[27]) {
+                                                       V (&T)[27]) {
     outer_modes<DO_A || DO_B, DO_BT>(C, g, sh, T);
 }
 
@@ -415,7 +442,7 @@ __host__ __device__ __forceinline__ void outer_phase2(const OuterArgs& a, int C,
     const OuterFrame f = outer_frame(a, C, cell);
     if (DO_B) {
         long long b[8];
-        const double s = outer_pressure(C, g, sh, a.h, b);
+        const FixScale s = outer_pressure(C, g, sh, a.h, b);
         // the vertex one step along the own axis and its opposite; the two that no rotation moves
         // go to warps 0 and 1
         outer_atomic_add(a.dst_p + outer_vertex(a, f, 1 << C), fix_out(b[1], s));
@@ -424,7 +451,7 @@ __host__ __device__ __forceinline__ void outer_phase2(const OuterArgs& a, int C,
     }
     if (!(DO_A || DO_BT)) return;
     long long Y[27];
-    const double s = outer_velocity<DO_A, DO_BT>(C, g, sh, a.mu[cell], a.h, Y);
+    const FixScale s = outer_velocity<DO_A, DO_BT>(C, g, sh, a.mu[cell], a.h, Y);
     double* dst = a.dst_u + size_t(C) * a.nodes +
                   (size_t(2 * f.ci) + size_t(a.M) * (size_t(2 * f.cj) + size_t(a.M) * size_t(2 * f.ck)));
 #pragma unroll
