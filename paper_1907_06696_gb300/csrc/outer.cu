@@ -15,7 +15,7 @@ namespace stk {
 
 namespace {
 
-// Bound by the integer pipes: ~13,500 thread instructions per cell, and the FP64 atomic adds of its 81 + 8
+// Bound by the integer pipes: ~13,400 thread instructions per cell, and the FP64 atomic adds of its 81 + 8
 // results. The whole operator (with the clearing of its output) at 64^3: 197 us, at 20^3: 23.6 us; in
 // double-float pairs through the Gauss points 854 and 62 us. A alone at 40^3: 44 us; one thread per
 // cell with FP64 instructions in the same modes 166 us. 5 CTAs per SM: 128 registers without spills.
